@@ -283,11 +283,13 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
     h->kcopy = cv.raw<double>(size_t(nx) * ny);
     h->chol = cv.raw<double>(size_t(h->n0) * h->n0);
     h->chol_idiag = cv.raw<double>(h->n0);
+    h->cinv = cv.raw<double>(size_t(h->n0) * h->n0);
     h->partials = cv.raw<double>(h->npartials);
     h->hist = cv.raw<double>(BMG_MAX_HISTORY);
     h->sc = cv.raw<Scalars>(1);
     h->dlev64 = cv.raw<LevelV<double>>(L);
     h->dlev32 = cv.raw<LevelV<float>>(L);
+    if (opt.smoother == BMG_SMOOTH_POINT) h->coarse_image = cv.raw<unsigned char>(kCoarseImageMax);
     if (opt.solver == BMG_SOLVER_PCG) {
       const Geom& gf = h->geo64.back();
       h->pcg_x = cv.plane<double>(gf);
@@ -341,6 +343,10 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
                         cudaMemcpyHostToDevice, s) != cudaSuccess)
       return fail(BMG_ECUDA);
   }
+  // Level schedule: which levels leave the full-grid launches, and how many
+  // blocks run them.
+  choose_schedule(h);
+  if ((rc = launch_coarse_image(h, s))) return fail(rc);
   if ((rc = check_derr(h, s))) return fail(rc);
 
   // TMA descriptors of every level swept by the TMA-staged kernel
@@ -361,9 +367,6 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
     make_maps(h->f, h->maps32);
   }
 
-  // Level schedule: which levels leave the full-grid launches, and how many
-  // blocks run them.
-  choose_schedule(h);
   h->setup_ms = now_ms() - t0;
   *out = h;
   return BMG_OK;
@@ -436,7 +439,7 @@ void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* d
   }
   {
     NvtxRange r("coarse_cycle", thr - 1);
-    launch_coarse_cycle<T>(h, dlev, thr, s);
+    launch_coarse_cycle<T>(h, lv, dlev, thr, thr - 1 < top || top_zero, s);
   }
   for (int l = thr; l <= top; ++l) {
     NvtxRange r("interp_leg", l);

@@ -112,8 +112,7 @@ __global__ void k_binterp(const LevelV<float>* __restrict__ fine,
 
 struct BCoarse {                  // per problem, for the persistent kernel
   const LevelV<float>* lev;
-  const double* chol;
-  const double* idiag;
+  const double* cinv;
   int thr, n0, top_nine;
 };
 
@@ -131,8 +130,7 @@ __global__ void __launch_bounds__(1024) k_bcoarse(const BCoarse* __restrict__ pc
   a.add_rc = 0;
   a.smoother = BMG_SMOOTH_POINT;
   a.top_nine = q.top_nine;
-  a.chol = q.chol;
-  a.idiag = q.idiag;
+  a.cinv = q.cinv;
   a.n0 = q.n0;
   coarse_cycle_body<float>(a);
 }
@@ -855,7 +853,7 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
   std::vector<BCoarse> pcs(nprob);
   for (int p = 0; p < nprob; ++p) {
     const Hierarchy* h = b->hs[p];
-    pcs[p] = BCoarse{h->dlev32, h->chol, h->chol_idiag, h->threshold, h->n0,
+    pcs[p] = BCoarse{h->dlev32, h->cinv, h->threshold, h->n0,
                      h->threshold < h->L ? 1 : 0};
   }
   cudaMemcpyAsync(b->pc, pcs.data(), sizeof(BCoarse) * nprob, cudaMemcpyHostToDevice, s);

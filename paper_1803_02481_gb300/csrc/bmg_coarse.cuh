@@ -62,8 +62,7 @@ struct CoarseArgs {
   int nu1, nu2, add_rc;
   int smoother;              // BMG_SMOOTH_*
   int top_nine;              // is level thr-1 9-point (else red-black)
-  const double* chol;        // N0 x N0 lower factor
-  const double* idiag;       // 1 / L[i][i]
+  const double* cinv;        // inverse of the coarsest operator
   int n0;
 };
 
@@ -141,49 +140,27 @@ __device__ void blk_interp(const LevelV<T>& F, const T* xc, int add_rc) {
   Team::sync();
 }
 
-// x_0 = A_0^{-1} b_0 with the stored factor (forward then backward
-// substitution, column-oriented, in FP64 shared memory).
+// x_0 = A_0^{-1} b_0 with the stored inverse, one unknown per thread, in FP64.
 template <typename T>
-__device__ void blk_coarse_solve(const LevelV<T>& L0, const double* __restrict__ lo,
-                                 const double* __restrict__ idiag, int n) {
+__device__ void blk_coarse_solve(const LevelV<T>& L0, const double* __restrict__ cinv, int n) {
   __shared__ double v[BMG_MAX_COARSEST];
   const int nx = L0.nx;
   for (int r = threadIdx.x; r < n; r += blockDim.x)
     v[r] = double(L0.b[(r / nx + 1) * L0.pitch + r % nx + 1]);
   __syncthreads();
-  if (n <= 64) {
-    if (threadIdx.x == 0) {
-      for (int j = 0; j < n; ++j) {
-        const double y = v[j] * idiag[j];
-        v[j] = y;
-        for (int i = j + 1; i < n; ++i) v[i] = fma(-lo[size_t(i) * n + j], y, v[i]);
-      }
-      for (int j = n - 1; j >= 0; --j) {
-        const double xj = v[j] * idiag[j];
-        v[j] = xj;
-        for (int i = 0; i < j; ++i) v[i] = fma(-lo[size_t(j) * n + i], xj, v[i]);
-      }
+  for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    auto inv = [&](int c) { return cinv[size_t(c) * n + r]; };
+    auto b = [&](int c) { return v[c]; };
+    double x;
+    if (n <= kInverseSerial) {
+      x = inverse_part(n, 0, 1, inv, b);
+    } else {
+      const double s0 = inverse_part(n, 0, 4, inv, b), s1 = inverse_part(n, 1, 4, inv, b);
+      const double s2 = inverse_part(n, 2, 4, inv, b), s3 = inverse_part(n, 3, 4, inv, b);
+      x = (s0 + s1) + (s2 + s3);
     }
-    __syncthreads();
-  } else {
-    for (int j = 0; j < n; ++j) {
-      const double y = v[j] * idiag[j];
-      __syncthreads();
-      if (threadIdx.x == 0) v[j] = y;
-      for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x)
-        v[i] = fma(-lo[size_t(i) * n + j], y, v[i]);
-      __syncthreads();
-    }
-    for (int j = n - 1; j >= 0; --j) {
-      const double xj = v[j] * idiag[j];
-      __syncthreads();
-      if (threadIdx.x == 0) v[j] = xj;
-      for (int i = threadIdx.x; i < j; i += blockDim.x) v[i] = fma(-lo[size_t(j) * n + i], xj, v[i]);
-      __syncthreads();
-    }
+    L0.x[(r / nx + 1) * L0.pitch + r % nx + 1] = T(x);
   }
-  for (int r = threadIdx.x; r < n; r += blockDim.x)
-    L0.x[(r / nx + 1) * L0.pitch + r % nx + 1] = T(v[r]);
   __syncthreads();
 }
 
@@ -203,7 +180,7 @@ __device__ void coarse_cycle_body(const CoarseArgs<T>& a) {
   }
   // the coarsest solve is one block's work (block rank 0 of a cluster; its
   // own barriers are block barriers), then the whole team resumes
-  if (Team::rank() == 0) blk_coarse_solve<T>(a.lev[0], a.chol, a.idiag, a.n0);
+  if (Team::rank() == 0) blk_coarse_solve<T>(a.lev[0], a.cinv, a.n0);
   if constexpr (Team::kCluster) Team::sync();
   for (int l = 1; l < a.thr; ++l) {
     const LevelV<T> L = a.lev[l];

@@ -450,7 +450,15 @@ int coarse_block_threads() {
 }
 
 template <typename T>
-void launch_coarse_cycle(Hierarchy* h, const LevelV<T>* dev_levels, int thr, cudaStream_t s) {
+void launch_coarse_cycle(Hierarchy* h, const std::vector<LevelV<T>>& lv, const LevelV<T>* dev_levels,
+                         int thr, bool top_zero, cudaStream_t s) {
+  if (h->coarse_smem) {
+    prof_begin(BMG_PROF_COARSE, s);
+    launch_coarse_smem<T>(h, lv[thr - 1], thr, top_zero, s);
+    prof_end(BMG_PROF_COARSE, s);
+    count_launch();
+    return;
+  }
   CoarseArgs<T> a;
   a.lev = dev_levels;
   a.thr = thr;
@@ -459,8 +467,7 @@ void launch_coarse_cycle(Hierarchy* h, const LevelV<T>* dev_levels, int thr, cud
   a.add_rc = h->opt.interp_residual_term;
   a.smoother = h->opt.smoother;
   a.top_nine = (thr < h->L) ? 1 : 0;
-  a.chol = h->chol;
-  a.idiag = h->chol_idiag;
+  a.cinv = h->cinv;
   a.n0 = h->n0;
   prof_begin(BMG_PROF_COARSE, s);
   if (a.smoother != BMG_SMOOTH_POINT)
@@ -523,7 +530,9 @@ template void launch_resid_restrict<float>(const LevelV<float>&, bool, LevelV<fl
 template void launch_interp<double>(const LevelV<double>&, const double*, bool, cudaStream_t,
                                     double*);
 template void launch_interp<float>(const LevelV<float>&, const float*, bool, cudaStream_t, float*);
-template void launch_coarse_cycle<double>(Hierarchy*, const LevelV<double>*, int, cudaStream_t);
-template void launch_coarse_cycle<float>(Hierarchy*, const LevelV<float>*, int, cudaStream_t);
+template void launch_coarse_cycle<double>(Hierarchy*, const std::vector<LevelV<double>>&,
+                                          const LevelV<double>*, int, bool, cudaStream_t);
+template void launch_coarse_cycle<float>(Hierarchy*, const std::vector<LevelV<float>>&,
+                                          const LevelV<float>*, int, bool, cudaStream_t);
 
 }  // namespace bmg

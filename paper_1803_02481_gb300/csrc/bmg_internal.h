@@ -314,6 +314,18 @@ __device__ __forceinline__ T interp_value(T* const* P, int cp, const T* __restri
   return v;
 }
 
+// Unknown r of x = A_0^{-1} b: row r of the stored inverse (entry (r, c) at
+// c * n + r) times b, read through `inv(c)` and `b(c)`.  More than 16
+// unknowns: four interleaved partial sums, part `k` of them here, added as
+// (s0 + s1) + (s2 + s3).
+constexpr int kInverseSerial = 16;
+template <class I, class B>
+__device__ __forceinline__ double inverse_part(int n, int k, int step, I inv, B b) {
+  double acc = 0.0;
+  for (int c = k; c < n; c += step) acc = fma(inv(c), b(c), acc);
+  return acc;
+}
+
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
@@ -366,6 +378,8 @@ struct Hierarchy {
   bmg_options opt{};
   int threshold = 1;                 // levels l < threshold: persistent kernel
   int coarse_ctas = 1;               // its thread blocks (1: one block; more: a cluster)
+  bool coarse_smem = false;          // one block, levels in shared memory
+  unsigned char* coarse_image = nullptr;   // their constant planes, packed
   std::vector<LevelV<double>> d;     // FP64 levels (all for FP64; finest only
                                      // for FP32_REFINE)
   std::vector<LevelV<float>> f;      // FP32 levels (FP32_REFINE)
@@ -373,6 +387,7 @@ struct Hierarchy {
   double* kcopy = nullptr;           // dense (ny, nx) copy of k
   double* chol = nullptr;            // N0 x N0 lower factor (row-major)
   double* chol_idiag = nullptr;      // 1 / L[i][i]
+  double* cinv = nullptr;            // inverse of the coarsest operator, column by column
   int n0 = 0;
   double* partials = nullptr;        // reduction scratch
   double* hist = nullptr;            // relative residual per cycle (BMG_MAX_HISTORY)
@@ -497,9 +512,21 @@ int launch_sweep_pre_norm(const LevelV<double>& L, const SweepMaps<double>* maps
 // run: prescaled TMA levels, and 5-point levels narrower than 1024 (swept by
 // the small tiled kernel) with at most nmax tiles.
 int sweep_norm_partials(const LevelV<double>& L, const SweepMaps<double>* maps, int nmax);
+// The sub-cycle of levels 0 .. threshold-1; top_zero: the iterate of level
+// threshold-1 is zero.
 template <typename T>
-void launch_coarse_cycle(Hierarchy* h, const LevelV<T>* levels, int threshold,
-                         cudaStream_t s);
+void launch_coarse_cycle(Hierarchy* h, const std::vector<LevelV<T>>& lv, const LevelV<T>* levels,
+                         int threshold, bool top_zero, cudaStream_t s);
+// The one-block sub-cycle with its levels in shared memory
+// (bmg_coarse_smem.cu): whether levels 0 .. threshold-1 fit it, the image of
+// their constant planes (setup, after the level views are on the device),
+// and the sub-cycle with level threshold-1 = `top`.
+constexpr size_t kCoarseImageMax = 220 * 1024;
+bool coarse_smem_fits(const Hierarchy* h, int threshold);
+int launch_coarse_image(Hierarchy* h, cudaStream_t s);
+template <typename T>
+void launch_coarse_smem(Hierarchy* h, const LevelV<T>& top, int threshold, bool top_zero,
+                        cudaStream_t s);
 
 // Prescaled finest level (bmg_sweep.cu): whether the finest FP64 level of a
 // hierarchy is prescaled; the coefficient planes W/C, E/C, S/C, N/C (setup)

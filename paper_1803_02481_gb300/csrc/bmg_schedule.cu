@@ -103,6 +103,11 @@ double predict_vcycle_us(const Hierarchy* h, int thr, int ctas) {
   return t;
 }
 
+// Points of the largest level the shared-memory sub-cycle takes by default:
+// a 31^2 level keeps one SM's FP64 pipes busy for longer than it saves in
+// launches.
+constexpr double kSmemPoints = 300.0;
+
 void choose_schedule(Hierarchy* h) {
   const bool point = h->opt.smoother == BMG_SMOOTH_POINT;
   int cands[2] = {1, 1};
@@ -124,6 +129,23 @@ void choose_schedule(Hierarchy* h) {
         h->threshold = thr;
         h->coarse_ctas = cands[k];
       }
+    }
+  }
+  // The one-block sub-cycle in shared memory runs whatever fits it: any
+  // explicit threshold, and by default every level of at most kSmemPoints
+  // points.
+  if (point && h->opt.coarse_ctas <= 1) {
+    int thr = h->opt.coarse_threshold;
+    if (thr < 1) {
+      thr = 1;
+      while (thr < h->L && double(h->geo64[thr].nx) * h->geo64[thr].ny <= kSmemPoints &&
+             coarse_smem_fits(h, thr + 1))
+        ++thr;
+    }
+    if (coarse_smem_fits(h, thr)) {
+      h->coarse_smem = true;
+      h->threshold = thr;
+      h->coarse_ctas = 1;
     }
   }
   for (int thr = 1; thr <= h->L && thr <= 16; ++thr)
