@@ -270,6 +270,7 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
     h->geo32.push_back(make_geom<float>(q.first, q.second));
   }
   h->npartials = 4 * 152;
+  h->max_partials = 2048;
 
   // Two passes: size, then carve.
   std::vector<Geom> g64 = fp32 ? std::vector<Geom>{h->geo64.back()} : h->geo64;
@@ -284,7 +285,7 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
     h->chol = cv.raw<double>(size_t(h->n0) * h->n0);
     h->chol_idiag = cv.raw<double>(h->n0);
     h->cinv = cv.raw<double>(size_t(h->n0) * h->n0);
-    h->partials = cv.raw<double>(h->npartials);
+    h->partials = cv.raw<double>(h->max_partials);
     h->hist = cv.raw<double>(BMG_MAX_HISTORY);
     h->sc = cv.raw<Scalars>(1);
     h->dlev64 = cv.raw<LevelV<double>>(L);
@@ -390,8 +391,9 @@ const SweepMaps<float>* level_maps<float>(const Hierarchy* h, int l) {
 
 template <typename T>
 void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* dlev, int thr,
-                    cudaStream_t s, int top, bool skip_first, bool top_zero) {
+                    cudaStream_t s, int top, bool skip_first, bool top_zero, int* norm_partials) {
   const int L = h->L;
+  if (norm_partials) *norm_partials = 0;
   // a cycle from level `top` down (the finest unless given): the levels
   // below the schedule's threshold still run in the persistent kernel
   if (top < 0 || top > L - 1) top = L - 1;
@@ -421,11 +423,30 @@ void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* d
     if (!nine) prof_end(BMG_PROF_FINE_SMOOTH, s);
     std::swap(V.x, V.x2);
   };
+  // Levels whose legs are one kernel each: the iterate goes x -> x2 -> x, or,
+  // where the first pre-sweep was issued before (skip_first: x holds its
+  // result, x2 is where the cycle's result belongs), x -> r -> x2.  While
+  // kernel classes are being timed one by one every operation is launched by
+  // itself (the same values).
+  auto leg = [&](int l) {
+    const int ns = nu1 - (skip_first && l == top ? 1 : 0);
+    if (h->opt.smoother != BMG_SMOOTH_POINT || rc || nu2 != 1 || ns < 1 || ns > 2 || prof_active() ||
+        lv[l].PR[PR_B])
+      return 0;
+    return leg_shape(lv[l].nx, lv[l].ny, l != L - 1, sizeof(T) == 8);
+  };
   prof_begin(BMG_PROF_CYCLE, s);
   NvtxRange cycle_range("vcycle", top);
   for (int l = top; l >= thr; --l) {
     NvtxRange r("restrict_leg", l);
     const bool nine = l != L - 1;
+    if (const int shape = leg(l)) {
+      LevelV<T>& V = lv[l];
+      const bool skip = skip_first && l == top;
+      launch_down_leg<T>(V, nine, shape, nu1 - (skip ? 1 : 0), zero_start && (l < top || top_zero), V.x,
+                         skip ? V.r : V.x2, lv[l - 1], s);
+      continue;
+    }
     if (nine) prof_begin(BMG_PROF_LEVELS, s);
     for (int k = skip_first && l == top ? 1 : 0; k < nu1; ++k)
       sweep(l, false, k == 0 && (l < top || top_zero));
@@ -444,6 +465,19 @@ void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* d
   for (int l = thr; l <= top; ++l) {
     NvtxRange r("interp_leg", l);
     const bool nine = l != L - 1;
+    if (const int shape = leg(l)) {
+      LevelV<T>& V = lv[l];
+      const bool skip = skip_first && l == top;
+      const int tiles = leg_tiles(shape, V.nx, V.ny);
+      const bool norm = skip && norm_partials && !nine && tiles <= h->max_partials;
+      launch_up_leg<T>(V, nine, shape, skip ? V.r : V.x2, lv[l - 1].x, skip ? V.x2 : V.x, V.x,
+                       norm ? h->partials : nullptr, s);
+      if (norm)
+        *norm_partials = tiles;
+      else if (skip)
+        std::swap(V.x, V.x2);
+      continue;
+    }
     if (nine) prof_begin(BMG_PROF_LEVELS, s);
     if (interp_oop) {
       launch_interp<T>(lv[l], lv[l - 1].x, rc, s, lv[l].x2);
@@ -458,9 +492,9 @@ void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* d
 }
 
 template void enqueue_vcycle<double>(Hierarchy*, std::vector<LevelV<double>>&,
-                                     const LevelV<double>*, int, cudaStream_t, int, bool, bool);
+                                     const LevelV<double>*, int, cudaStream_t, int, bool, bool, int*);
 template void enqueue_vcycle<float>(Hierarchy*, std::vector<LevelV<float>>&, const LevelV<float>*,
-                                    int, cudaStream_t, int, bool, bool);
+                                    int, cudaStream_t, int, bool, bool, int*);
 
 // Stop test inside the next cycle's first fine sweep.  The V(nu1, nu2)
 // cycle's last fine sweep is a post-smoothing sweep (reverse colour order),
@@ -479,7 +513,7 @@ static bool fused_norm_on(const Hierarchy* h) {
   const SweepMaps<double>* m = level_maps<double>(h, L - 1);
   return h->fused_norm_allowed && h->opt.solver == BMG_SOLVER_VCYCLE && h->opt.precision == BMG_FP64 &&
          h->opt.smoother == BMG_SMOOTH_POINT && h->opt.nu1 >= 1 && h->opt.nu2 >= 1 &&
-         h->threshold < L && sweep_norm_partials(h->d.back(), m, h->npartials) > 0;
+         h->threshold < L && sweep_norm_partials(h->d.back(), m, h->max_partials) > 0;
 }
 
 // The finest level's first pre-smoothing sweep of a cycle: plain, or with
@@ -488,7 +522,7 @@ static bool fused_norm_on(const Hierarchy* h) {
 static void fine_presweep(Hierarchy* h, cudaStream_t s, bool with_norm, bool in_graph) {
   LevelV<double>& F = h->d.back();
   const SweepMaps<double>* m = level_maps<double>(h, h->L - 1);
-  const bool fusable = sweep_norm_partials(F, m, h->npartials) > 0 &&
+  const bool fusable = sweep_norm_partials(F, m, h->max_partials) > 0 &&
                        (!(m && m->pre) || F.x == m->xp || F.x == m->x2p);
   if (with_norm && !fusable) {
     // (not reached while fused_norm_on holds) the same result in two passes
@@ -497,7 +531,7 @@ static void fine_presweep(Hierarchy* h, cudaStream_t s, bool with_norm, bool in_
   }
   if (with_norm) {
     prof_begin(BMG_PROF_NORM, s);
-    const int n = launch_sweep_pre_norm(F, m, F.x, F.x2, h->partials, h->npartials, s);
+    const int n = launch_sweep_pre_norm(F, m, F.x, F.x2, h->partials, h->max_partials, s);
     launch_norm_final(h, s, in_graph, n);
     prof_end(BMG_PROF_NORM, s);
   } else {
@@ -506,6 +540,17 @@ static void fine_presweep(Hierarchy* h, cudaStream_t s, bool with_norm, bool in_
     prof_end(BMG_PROF_FINE_SMOOTH, s);
   }
   std::swap(F.x, F.x2);
+}
+
+// The rest of a cycle whose first pre-sweep was issued, the next cycle's first
+// pre-sweep and the stop test of the cycle's result.
+static void fused_cycle(Hierarchy* h, cudaStream_t s, bool in_graph) {
+  int n = 0;
+  enqueue_vcycle<double>(h, h->d, h->dlev64, h->threshold, s, -1, true, false, &n);
+  if (n > 0)
+    launch_norm_final(h, s, in_graph, n);
+  else
+    fine_presweep(h, s, true, in_graph);
 }
 
 static int read_scalars(Hierarchy* h, cudaStream_t s) {
@@ -560,8 +605,7 @@ static int build_solve_graph(Hierarchy* h) {
       launch_refine_update(h, s);
       launch_refine_residual(h, 0.0, s, true);
     } else if (fused) {
-      enqueue_vcycle<double>(h, h->d, h->dlev64, h->threshold, s, -1, true);
-      fine_presweep(h, s, true, true);
+      fused_cycle(h, s, true);
     } else {
       enqueue_vcycle<double>(h, h->d, h->dlev64, h->threshold, s);
       launch_fine_norm(h, F.x, F.b, 1, 0.0, s, true);
@@ -708,8 +752,7 @@ static int solve_impl(Hierarchy* h, const double* b, double* x, double tol, bmg_
       if (h->sc_host->go) {
         fine_presweep(h, s, false, false);
         while (h->sc_host->go) {
-          enqueue_vcycle<double>(h, h->d, h->dlev64, h->threshold, s, -1, true);
-          fine_presweep(h, s, true, false);
+          fused_cycle(h, s, false);
           if ((rc = read_scalars(h, s))) break;
         }
         // the result is the input of the last sweep

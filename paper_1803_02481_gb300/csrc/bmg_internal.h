@@ -391,7 +391,8 @@ struct Hierarchy {
   int n0 = 0;
   double* partials = nullptr;        // reduction scratch
   double* hist = nullptr;            // relative residual per cycle (BMG_MAX_HISTORY)
-  int npartials = 0;
+  int npartials = 0;                 // blocks of the norm kernels
+  int max_partials = 0;              // partial sums the scratch holds
   Scalars* sc = nullptr;             // device scalars
   Scalars* sc_host = nullptr;        // pinned mirror
   LevelV<double>* dlev64 = nullptr;  // device copies of the level views (for
@@ -477,6 +478,22 @@ template <typename T>
 void launch_interp(const LevelV<T>& fine, const T* xc, bool add_r_over_c, cudaStream_t s,
                    T* out = nullptr);
 void prepare_sweep_kernels();
+
+// The legs of a V-cycle level as one kernel each (bmg_legs.cuh).  leg_shape:
+// the tile shape for a level (0: the level keeps the kernels of one operation
+// each).  down: ns (1 or 2) forward sweeps from xin
+// (zero: it is zero and not read) to xout, residual, restriction, zero coarse
+// iterate.  up: x = xin + P xc and one reverse-order sweep to xout; with
+// partials (finest 5-point level), also the next cycle's first pre-sweep of
+// xout into xnext and the squared residual of xout per tile (leg_tiles).
+int leg_shape(int nx, int ny, bool nine, bool fp64);
+int leg_tiles(int shape, int nx, int ny);
+template <typename T>
+void launch_down_leg(const LevelV<T>& F, bool nine, int shape, int ns, bool zero, const T* xin, T* xout,
+                     const LevelV<T>& Cc, cudaStream_t s);
+template <typename T>
+void launch_up_leg(const LevelV<T>& F, bool nine, int shape, const T* xin, const T* xc, T* xout, T* xnext,
+                   double* partials, cudaStream_t s);
 
 // Threads per block of the cluster coarse kernel, and the largest cluster
 // (blocks, a power of two <= 16) the device can run it with; 1 when thread-
@@ -580,9 +597,13 @@ void launch_pcg_precond(Hierarchy* h, cudaStream_t s);
 // skip_first: the top level's first pre-smoothing sweep was already issued;
 // top_zero: the top level's iterate is zero on entry (as every coarser
 // level's is after its restriction).
+// Where `norm_partials` is given (with skip_first) and the top level's up leg
+// can take it, the leg also does the next cycle's first pre-smoothing sweep
+// and the stop test's partial sums, and their number is stored there (else 0).
 template <typename T>
 void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* dlev, int thr,
-                    cudaStream_t s, int top = -1, bool skip_first = false, bool top_zero = false);
+                    cudaStream_t s, int top = -1, bool skip_first = false, bool top_zero = false,
+                    int* norm_partials = nullptr);
 
 void launch_assemble_backward(const double* k, const double* u, const double* lam,
                               double* g, int nx, int ny, cudaStream_t s);

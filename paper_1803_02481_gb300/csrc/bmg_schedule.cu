@@ -103,9 +103,11 @@ double predict_vcycle_us(const Hierarchy* h, int thr, int ctas) {
   return t;
 }
 
-// Points of the largest level the shared-memory sub-cycle takes by default:
-// a 31^2 level keeps one SM's FP64 pipes busy for longer than it saves in
-// launches.
+// Points of the largest level the shared-memory sub-cycle takes by default.
+// Measured us per V-cycle with the largest level at 7^2, 15^2 and 31^2: FP64
+// 255^2 71.2, 67.1, 71.6; FP64 511^2 105, 103, 108; FP32 255^2 47.8, 46.6,
+// 46.8; FP32 511^2 62.2, 60.8, 61.7 (a 31^2 level keeps one SM's FP64 pipes
+// busy for longer than two launches over many SMs take).
 constexpr double kSmemPoints = 300.0;
 
 void choose_schedule(Hierarchy* h) {
