@@ -389,6 +389,38 @@ const SweepMaps<float>* level_maps<float>(const Hierarchy* h, int l) {
   return l >= 0 && l < int(h->maps32.size()) ? h->maps32[l] : nullptr;
 }
 
+// Zero-start first sweeps (environment BMG_ZERO_START=0 turns them off).
+static bool zero_start_on() {
+  static const bool on = [] {
+    const char* e = std::getenv("BMG_ZERO_START");
+    return !(e && e[0] == '0');
+  }();
+  return on;
+}
+
+// The tile shape of level l's fused legs in a cycle whose down leg does ns
+// sweeps there (0: one launch per operation).  While kernel classes are being
+// timed one by one every operation is launched by itself (the same values).
+template <typename T>
+static int level_leg(const Hierarchy* h, const LevelV<T>& V, int l, int ns) {
+  if (h->opt.smoother != BMG_SMOOTH_POINT || h->opt.interp_residual_term || h->opt.nu2 != 1 || ns < 1 ||
+      ns > 2 || prof_active() || V.PR[PR_B])
+    return 0;
+  return leg_shape(V.nx, V.ny, l != h->L - 1, sizeof(T) == 8);
+}
+
+template <typename T>
+static bool reads_zero_top(const Hierarchy* h, const std::vector<LevelV<T>>& lv) {
+  if (!zero_start_on() || h->opt.smoother != BMG_SMOOTH_POINT || h->opt.nu1 < 1) return true;
+  if (h->threshold == h->L) return !h->coarse_smem;
+  return !level_leg<T>(h, lv.back(), h->L - 1, h->opt.nu1) && !level_maps<T>(h, h->L - 1);
+}
+
+bool cycle_reads_zero_top(const Hierarchy* h) {
+  return h->opt.precision == BMG_FP32_REFINE ? reads_zero_top<float>(h, h->f)
+                                             : reads_zero_top<double>(h, h->d);
+}
+
 template <typename T>
 void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* dlev, int thr,
                     cudaStream_t s, int top, bool skip_first, bool top_zero, int* norm_partials) {
@@ -406,11 +438,8 @@ void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* d
   const bool interp_oop = ((nu1 + nu2) & 1) != 0;
   // zero: the level's iterate is zero (its first pre-sweep: every level below
   // the top was zeroed by its restriction); the sweep may then take the
-  // zero-start form (environment BMG_ZERO_START=0 turns it off)
-  static const bool zero_start = [] {
-    const char* e = std::getenv("BMG_ZERO_START");
-    return !(e && e[0] == '0');
-  }();
+  // zero-start form
+  const bool zero_start = zero_start_on();
   auto sweep = [&](int l, bool reverse, bool zero) {
     zero = zero && zero_start;
     LevelV<T>& V = lv[l];
@@ -425,15 +454,9 @@ void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* d
   };
   // Levels whose legs are one kernel each: the iterate goes x -> x2 -> x, or,
   // where the first pre-sweep was issued before (skip_first: x holds its
-  // result, x2 is where the cycle's result belongs), x -> r -> x2.  While
-  // kernel classes are being timed one by one every operation is launched by
-  // itself (the same values).
+  // result, x2 is where the cycle's result belongs), x -> r -> x2.
   auto leg = [&](int l) {
-    const int ns = nu1 - (skip_first && l == top ? 1 : 0);
-    if (h->opt.smoother != BMG_SMOOTH_POINT || rc || nu2 != 1 || ns < 1 || ns > 2 || prof_active() ||
-        lv[l].PR[PR_B])
-      return 0;
-    return leg_shape(lv[l].nx, lv[l].ny, l != L - 1, sizeof(T) == 8);
+    return level_leg<T>(h, lv[l], l, nu1 - (skip_first && l == top ? 1 : 0));
   };
   prof_begin(BMG_PROF_CYCLE, s);
   NvtxRange cycle_range("vcycle", top);

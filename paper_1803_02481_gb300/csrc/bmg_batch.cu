@@ -4,17 +4,23 @@
 //
 // Organisation.  Every problem is set up as a hierarchy of its own.  The
 // solve groups, for every grid side n, the levels of that side across all
-// problems (5-point finest levels and 9-point coarse levels separately) and
-// runs each operation of the V-cycle as ONE launch over all of them: the
-// problem index is blockIdx.z, and a problem that has converged leaves at
-// once.  Levels at or below `coarse_side` run in the persistent coarse
-// kernel, one thread block per problem.  Per-problem FP64 residual norms and
-// stop tests decide which problems stay active; the whole refinement loop is
-// one CUDA graph whose WHILE node repeats while any problem is active.  Tile
-// shapes of the batched sweeps are chosen per level side by timing the
+// problems and runs each leg of the V-cycle (bmg_legs.cuh) as ONE launch over
+// all of them, finest 5-point and coarse 9-point levels alike: the problem
+// index is blockIdx.z, and a problem that has converged leaves at once.
+// Levels of side 31 and below run in the shared-memory coarse kernel, one
+// thread block per problem.  The FP64 work on the finest levels is one launch
+// per pass over all problems, cut into units of some 4096 points, so that a
+// 1023^2 problem gets the blocks its size asks for (64 blocks whatever the
+// size took 18.7 us a pass, 47 % of a 48-problem solve).  Per-problem FP64
+// residual norms and stop tests decide which problems stay active; the whole
+// refinement loop is one CUDA graph whose WHILE node repeats while any
+// problem is active.  V-cycles with other than one or two pre- and one
+// post-smoothing sweep run one launch per operation and level class instead;
+// their sweeps' tile shapes are chosen per level side by timing the
 // candidates on the batch (autotuner, cached per process and optionally in
 // the file named by BMG_TUNE_CACHE).
-#include "bmg_coarse.cuh"
+#include "bmg_krylov.cuh"
+#include "bmg_legs.cuh"
 #include "bmg_sweep_tile.cuh"
 
 #include <algorithm>
@@ -32,26 +38,11 @@ namespace bmg {
 
 namespace {
 
-constexpr int kPB = 64;           // FP64 partial sums per problem
-constexpr int kNT = 256;          // threads of the norm kernels
+constexpr int kUnitRuns = 8;      // runs of kKT pairs a unit of FP64 work holds (4096 points)
+constexpr int kNT = kKT;          // threads of the norm kernels
 constexpr int kCoarseSide = 31;   // levels with side <= this: persistent kernel
 
 inline int cdiv(long a, long b) { return int((a + b - 1) / b); }
-
-__device__ __forceinline__ double bsum(double v) {
-  __shared__ double red[kNT / 32];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  v = lane < kNT / 32 ? red[lane] : 0.0;
-  if (w == 0) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  }
-  return v;
-}
 
 // ---------------------------------------------------------------------------
 // Batched V-cycle kernels (FP32).  z = blockIdx.z indexes the class members.
@@ -110,270 +101,284 @@ __global__ void k_binterp(const LevelV<float>* __restrict__ fine,
   (out_of_place ? F.x2 : F.x)[o] = v;
 }
 
-struct BCoarse {                  // per problem, for the persistent kernel
-  const LevelV<float>* lev;
-  const double* cinv;
-  int thr, n0, top_nine;
-};
+// The legs of the levels of one side: the z-th member's iterate goes
+// x -> x2 -> x.  Its iterate is zero on entry (every level's is: the finest
+// level solves for a correction).  Whether a problem is active was settled
+// before the kernel that precedes this one began, so it is read, and the
+// operator staged, ahead of the wait; a block that leaves waits all the same,
+// because the kernel that follows relies on this one to have waited.
+template <bool NINE, int NS, int TX, int TY, int NT>
+__device__ __forceinline__ void batch_down(const LevelV<float>& F, const LevelV<float>& Cc, float* sm) {
+  float pw[8];
+  down_constants<float, NINE, NS, TX, TY, NT>(F, Cc, sm, blockIdx.x, blockIdx.y, pw);
+  griddep_wait();
+  down_tile<float, NINE, NS, true, TX, TY, NT>(F, F.x, F.x2, Cc, sm, blockIdx.x, blockIdx.y, pw);
+}
+template <int NS, int TX, int TY, int NT>
+__global__ void __launch_bounds__(NT) k_bdown(const LevelV<float>* __restrict__ fine,
+                                              const LevelV<float>* __restrict__ coarse,
+                                              const int* __restrict__ pids,
+                                              const Scalars* __restrict__ sc) {
+  extern __shared__ __align__(16) unsigned char leg_smem[];
+  float* sm = reinterpret_cast<float*>(leg_smem);
+  const int z = blockIdx.z;
+  if (!sc[pids[z]].go) {
+    griddep_wait();
+    return;
+  }
+  const LevelV<float> F = fine[z], Cc = coarse[z];
+  if (F.SW)
+    batch_down<true, NS, TX, TY, NT>(F, Cc, sm);
+  else
+    batch_down<false, NS, TX, TY, NT>(F, Cc, sm);
+}
 
-__global__ void __launch_bounds__(1024) k_bcoarse(const BCoarse* __restrict__ pc,
-                                                  const Scalars* __restrict__ sc, int nu1,
-                                                  int nu2) {
-  const int p = blockIdx.x;
-  if (!sc[p].go) return;
-  const BCoarse q = pc[p];
-  CoarseArgs<float> a;
-  a.lev = q.lev;
-  a.thr = q.thr;
-  a.nu1 = nu1;
-  a.nu2 = nu2;
-  a.add_rc = 0;
-  a.smoother = BMG_SMOOTH_POINT;
-  a.top_nine = q.top_nine;
-  a.cinv = q.cinv;
-  a.n0 = q.n0;
-  coarse_cycle_body<float>(a);
+template <bool NINE, int TX, int TY, int NT>
+__device__ __forceinline__ void batch_up(const LevelV<float>& F, const float* xc, float* sm) {
+  float w[8];
+  up_constants<float, NINE, TX, TY, NT, false>(F, sm, blockIdx.x, blockIdx.y, w);
+  griddep_wait();
+  up_tile<float, NINE, TX, TY, NT, false>(F, F.x2, xc, F.x, nullptr, sm, blockIdx.x, blockIdx.y, w);
+}
+template <int TX, int TY, int NT>
+__global__ void __launch_bounds__(NT) k_bup(const LevelV<float>* __restrict__ fine,
+                                            const LevelV<float>* __restrict__ coarse,
+                                            const int* __restrict__ pids, const Scalars* __restrict__ sc) {
+  extern __shared__ __align__(16) unsigned char leg_smem[];
+  float* sm = reinterpret_cast<float*>(leg_smem);
+  const int z = blockIdx.z;
+  if (!sc[pids[z]].go) {
+    griddep_wait();
+    return;
+  }
+  const LevelV<float> F = fine[z];
+  if (F.SW)
+    batch_up<true, TX, TY, NT>(F, coarse[z].x, sm);
+  else
+    batch_up<false, TX, TY, NT>(F, coarse[z].x, sm);
 }
 
 // ---------------------------------------------------------------------------
-// Batched refinement kernels (FP64 on each problem's finest level).
+// FP64 work on the problems' finest levels: a block per unit.
 // ---------------------------------------------------------------------------
 
+struct BUnit {
+  int p, local, count;           // problem, unit of it, its units
+};
+struct BSpan {
+  int first, count;              // a problem's units
+};
+// Per problem: its finest levels and CG vectors.
+struct BProb {
+  LevelV<double> d;
+  LevelV<float> f;
+  PcgVec v;
+};
+
 // what == 0: partial sums of b^2.  what == 1 (active problems only): r = b -
-// A x in FP64, partial sums of r^2, FP32 right-hand side r / ||r_prev||, FP32
-// iterate reset to zero.  One problem per blockIdx.y, kPB blocks each.
-__global__ void __launch_bounds__(kNT) k_brefine_resid(const LevelV<double>* __restrict__ f64,
-                                                       const LevelV<float>* __restrict__ f32,
-                                                       const int* __restrict__ pids,
-                                                       const Scalars* __restrict__ sc,
-                                                       double* __restrict__ partials, int what) {
-  const int z = blockIdx.y;
-  const int p = pids[z];
-  if (what == 1 && !sc[p].go) return;
-  const LevelV<double> L = f64[z];
-  const LevelV<float> F = f32[z];
-  const double inv = what ? sc[p].inv : 0.0;
+// A x in FP64, partial sums of r^2, FP32 right-hand side r / ||r_prev||
+// (zero_x: and a zero FP32 iterate, for cycles that read it).
+template <int WHAT>
+__global__ void __launch_bounds__(kKT) k_brefine_resid(const BProb* __restrict__ prob,
+                                                       const BUnit* __restrict__ units,
+                                                       const Scalars* __restrict__ sc, int zero_x,
+                                                       double* __restrict__ partials) {
+  griddep_wait();
+  const BUnit u = units[blockIdx.x];
+  if (WHAT == 1 && !sc[u.p].go) return;
+  const LevelV<double>& L = prob[u.p].d;
+  const LevelV<float>& F = prob[u.p].f;
+  const double inv = WHAT ? sc[u.p].inv : 0.0;
   // FP32 scaling of the right-hand side, as in the single-problem kernel
   const bool fp32_scale = inv > 1e-28 && inv < 1e28;
   const float inv32 = float(inv);
   double acc = 0.0;
-  for (int j = blockIdx.x + 1; j <= L.ny; j += gridDim.x) {
-    for (int i = threadIdx.x + 1; i <= L.nx; i += blockDim.x) {
-      const int o = j * L.pitch + i;
+  for_pairs(L.nx, L.ny, u.local, u.count, [&](int j, int i, bool two) {
+    const int o = j * L.pitch + i;
+    const double2 bv = load2(L.b + o);
+    if (WHAT == 0) {
+      acc = fma(bv.x, bv.x, acc);
+      if (two) acc = fma(bv.y, bv.y, acc);
+      return;
+    }
+    const double2 r = resid_pair(load_resid(L, L.x, o), bv);
+    acc = fma(r.x, r.x, acc);
+    const int of = j * F.pitch + i;
+    const float f0 = fp32_scale ? to_float(r.x) * inv32 : to_float(r.x * inv);
+    F.b[of] = f0;
+    if (zero_x) F.x[of] = 0.0f;
+    if (two) {
+      acc = fma(r.y, r.y, acc);
+      F.b[of + 1] = fp32_scale ? to_float(r.y) * inv32 : to_float(r.y * inv);
+      if (zero_x) F.x[of + 1] = 0.0f;
+    }
+  });
+  acc = krylov_block_sum(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+}
+
+// One block per problem: sums its partials and applies the stop test; the
+// last block to finish knows whether any problem is still active, and drives
+// the graph's WHILE node (`count`: problems done and active, back to zero).
+__global__ void __launch_bounds__(kNT) k_bnorm_final(const double* __restrict__ partials,
+                                                     const BSpan* __restrict__ spans,
+                                                     Scalars* __restrict__ sc, int what,
+                                                     cudaGraphConditionalHandle handle, int use_handle,
+                                                     int* __restrict__ count) {
+  griddep_wait();
+  const int p = blockIdx.x;
+  Scalars* s = sc + p;
+  int go = 0;
+  if (what == 0 || s->go) {
+    double acc = 0.0;
+    const BSpan q = spans[p];
+    for (int k = threadIdx.x; k < q.count; k += kNT) acc += partials[q.first + k];
+    acc = krylov_block_sum(acc);
+    if (threadIdx.x == 0) {
       if (what == 0) {
-        const double bv = L.b[o];
-        acc = fma(bv, bv, acc);
+        s->bnorm2 = acc;
+        s->rnorm2 = acc;
+        s->rnorm = sqrt(acc);
+        s->inv = acc > 0.0 ? 1.0 / s->rnorm : 0.0;
+        go = acc > 0.0 ? 1 : 0;     // a zero right-hand side needs no cycle
+        s->go = go;
+        s->rel = 0.0;
       } else {
-        const double r = resid_value<double, false>(L, L.x, L.b[o], o);
-        acc = fma(r, r, acc);
-        const int of = j * F.pitch + i;
-        F.b[of] = fp32_scale ? float(r) * inv32 : float(r * inv);
-        F.x[of] = 0.0f;
+        s->scale2 = s->rnorm2;
+        s->scale = sqrt(s->scale2);
+        s->rnorm2 = acc;
+        s->rnorm = sqrt(acc);
+        s->inv = acc > 0.0 ? 1.0 / s->rnorm : 0.0;
+        const double rel = sqrt(acc / s->bnorm2);
+        s->rel = rel;
+        const bool finite = isfinite(rel);
+        if (!finite) s->err |= DEV_NAN;
+        go = (finite && rel > s->tol && s->cycles < s->max_cycles && s->err == 0) ? 1 : 0;
+        s->go = go;
+        s->cycles += go;
       }
     }
   }
-  acc = bsum(acc);
-  if (threadIdx.x == 0) partials[size_t(p) * kPB + blockIdx.x] = acc;
-}
-
-// One block per problem: sums its partials and applies the stop test.
-__global__ void __launch_bounds__(kNT) k_bnorm_final(const double* __restrict__ partials,
-                                                     Scalars* __restrict__ sc, int what) {
-  const int p = blockIdx.x;
-  Scalars* s = sc + p;
-  if (what == 1 && !s->go) return;
-  double acc = threadIdx.x < kPB ? partials[size_t(p) * kPB + threadIdx.x] : 0.0;
-  acc = bsum(acc);
   if (threadIdx.x != 0) return;
-  if (what == 0) {
-    s->bnorm2 = acc;
-    s->rnorm2 = acc;
-    s->rnorm = sqrt(acc);
-    s->inv = acc > 0.0 ? 1.0 / s->rnorm : 0.0;
-    s->go = acc > 0.0 ? 1 : 0;     // a zero right-hand side needs no cycle
-    s->rel = 0.0;
-    return;
-  }
-  s->scale2 = s->rnorm2;
-  s->scale = sqrt(s->scale2);
-  s->rnorm2 = acc;
-  s->rnorm = sqrt(acc);
-  s->inv = acc > 0.0 ? 1.0 / s->rnorm : 0.0;
-  const double rel = sqrt(acc / s->bnorm2);
-  s->rel = rel;
-  const bool finite = isfinite(rel);
-  if (!finite) s->err |= DEV_NAN;
-  const int go = (finite && rel > s->tol && s->cycles < s->max_cycles && s->err == 0) ? 1 : 0;
-  s->go = go;
-  s->cycles += go;
-}
-
-// Is any problem still active?  Drives the graph's WHILE node.
-__global__ void __launch_bounds__(kNT) k_bany(const Scalars* __restrict__ sc, int nprob,
-                                              cudaGraphConditionalHandle handle, int use_handle,
-                                              int* any_out) {
-  int any = 0;
-  for (int p = threadIdx.x; p < nprob; p += blockDim.x) any |= sc[p].go;
-  any = __syncthreads_or(any);
-  if (threadIdx.x == 0) {
-    *any_out = any;
+  if (go) atomicAdd(&count[1], 1);
+  __threadfence();
+  if (atomicAdd(&count[0], 1) == int(gridDim.x) - 1) {
+    const int any = atomicExch(&count[1], 0);
+    count[0] = 0;
     if (use_handle) cudaGraphSetConditional(handle, any ? 1u : 0u);
   }
 }
 
-__global__ void k_bupdate(const LevelV<double>* __restrict__ f64,
-                          const LevelV<float>* __restrict__ f32, const int* __restrict__ pids,
-                          const Scalars* __restrict__ sc) {
-  const int z = blockIdx.z;
-  const int p = pids[z];
-  if (!sc[p].go) return;
-  const LevelV<double> L = f64[z];
-  const float* e = f32[z].x;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x + 1;
-  const int j = blockIdx.y + 1;
-  if (i > L.nx) return;
-  const double s = sc[p].scale;
-  const int o = j * L.pitch + i;
-  L.x[o] = fma(s, double(e[j * f32[z].pitch + i]), L.x[o]);
+__global__ void __launch_bounds__(kKT) k_bupdate(const BProb* __restrict__ prob,
+                                                 const BUnit* __restrict__ units,
+                                                 const Scalars* __restrict__ sc) {
+  griddep_wait();
+  const BUnit u = units[blockIdx.x];
+  if (!sc[u.p].go) return;
+  const LevelV<double>& L = prob[u.p].d;
+  const LevelV<float>& F = prob[u.p].f;
+  const double s = sc[u.p].scale;
+  for_pairs(L.nx, L.ny, u.local, u.count, [&](int j, int i, bool two) {
+    const int o = j * L.pitch + i;
+    const double2 x = load2(L.x + o);
+    const float2 e = *reinterpret_cast<const float2*>(F.x + j * F.pitch + i);
+    store2(L.x + o, fma(s, to_double(e.x), x.x), fma(s, to_double(e.y), x.y), two);
+  });
 }
 
 // ---------------------------------------------------------------------------
 // Batched conjugate gradients (BMG_SOLVER_PCG): per problem, CG on its finest
 // operator in FP64, preconditioned by one symmetric FP32 V(nu, nu) cycle of
-// the batched V-cycle (r / ||r|| cast to the FP32 finest level, z = ||r|| e
-// cast back), in the single-problem solver's order.  The FP64 finest level's
-// b plane holds r and its x plane z; X, B, P, Q are the problem's CG planes.
+// the batched V-cycle (r / ||r|| cast to the FP32 finest level, z = ||r|| e),
+// in the single-problem solver's order and with its passes (bmg_krylov.cuh).
+// Active problems only.
 // ---------------------------------------------------------------------------
 
-struct BPcg {
-  double *x, *b, *p, *q;
-};
-
-enum { BPCG_INIT = 0, BPCG_AP = 1, BPCG_XR = 2, BPCG_RZ = 3, BPCG_P = 4 };
-
-// One problem per blockIdx.y, kPB blocks each, active problems only:
-// INIT r = B - A X, z = 0, partials of r.r; AP Q = A P, partials of P.Q;
-// XR X += alpha P, r -= alpha Q, z = 0, partials of r.r; RZ partials of r.z;
-// P P = z + beta P.
-__global__ void __launch_bounds__(kNT) k_bpcg(const LevelV<double>* __restrict__ f64,
-                                              const BPcg* __restrict__ vec,
-                                              const int* __restrict__ pids,
+template <int WHAT>
+__global__ void __launch_bounds__(kKT) k_bpcg(const BProb* __restrict__ prob,
+                                              const BUnit* __restrict__ units,
                                               const Scalars* __restrict__ sc,
-                                              double* __restrict__ partials, int what) {
-  const int z = blockIdx.y;
-  const int pr = pids[z];
-  if (!sc[pr].go) return;
-  const LevelV<double> L = f64[z];
-  const BPcg v = vec[z];
-  const double alpha = sc[pr].alpha, beta = sc[pr].beta;
-  double acc = 0.0;
-  for (int j = blockIdx.x + 1; j <= L.ny; j += gridDim.x) {
-    for (int i = threadIdx.x + 1; i <= L.nx; i += blockDim.x) {
-      const int o = j * L.pitch + i;
-      if (what == BPCG_INIT) {
-        const double r = resid_value<double, false>(L, v.x, v.b[o], o);
-        L.b[o] = r;
-        L.x[o] = 0.0;
-        acc = fma(r, r, acc);
-      } else if (what == BPCG_AP) {
-        const double q = -resid_value<double, false>(L, v.p, 0.0, o);
-        v.q[o] = q;
-        acc = fma(v.p[o], q, acc);
-      } else if (what == BPCG_XR) {
-        v.x[o] = fma(alpha, v.p[o], v.x[o]);
-        const double r = fma(-alpha, v.q[o], L.b[o]);
-        L.b[o] = r;
-        L.x[o] = 0.0;
-        acc = fma(r, r, acc);
-      } else if (what == BPCG_RZ) {
-        acc = fma(L.b[o], L.x[o], acc);
-      } else {
-        v.p[o] = fma(beta, v.p[o], L.x[o]);
-      }
-    }
-  }
-  if (what == BPCG_P) return;
-  acc = bsum(acc);
-  if (threadIdx.x == 0) partials[size_t(pr) * kPB + blockIdx.x] = acc;
+                                              double* __restrict__ partials) {
+  griddep_wait();
+  const BUnit u = units[blockIdx.x];
+  if (!sc[u.p].go) return;
+  const BProb& q = prob[u.p];
+  double s = krylov_pass<WHAT, true>(q.d, &q.f, q.v, sc + u.p, false, u.local, u.count);
+  if (WHAT == K_P) return;
+  s = krylov_block_sum(s);
+  if (threadIdx.x == 0) partials[blockIdx.x] = s;
+}
+
+__global__ void __launch_bounds__(kKT) k_bpcg_cast(const BProb* __restrict__ prob,
+                                                   const BUnit* __restrict__ units,
+                                                   const Scalars* __restrict__ sc, int zero_x) {
+  griddep_wait();
+  const BUnit u = units[blockIdx.x];
+  if (!sc[u.p].go) return;
+  krylov_cast(prob[u.p].d, prob[u.p].f, sc + u.p, zero_x != 0, u.local, u.count);
 }
 
 // One block per problem: AP alpha = rz / sum (0 for a zero denominator); RZ
 // beta = sum / rz (0 while rz is 0: the first direction is z), rz = sum.
 __global__ void __launch_bounds__(kNT) k_bpcg_scalar(const double* __restrict__ partials,
+                                                     const BSpan* __restrict__ spans,
                                                      Scalars* __restrict__ sc, int what) {
+  griddep_wait();
   const int pr = blockIdx.x;
   Scalars* s = sc + pr;
   if (!s->go) return;
-  double acc = threadIdx.x < kPB ? partials[size_t(pr) * kPB + threadIdx.x] : 0.0;
-  acc = bsum(acc);
+  double acc = 0.0;
+  const BSpan q = spans[pr];
+  for (int k = threadIdx.x; k < q.count; k += kNT) acc += partials[q.first + k];
+  acc = krylov_block_sum(acc);
   if (threadIdx.x != 0) return;
-  if (what == BPCG_AP) {
+  if (what == K_AP) {
     s->alpha = acc != 0.0 ? s->rz / acc : 0.0;
   } else {
+    acc *= s->rnorm;   // (the partials are of r.e, z = ||r|| e)
     s->beta = s->rz != 0.0 ? acc / s->rz : 0.0;
     s->rz = acc;
   }
 }
 
-// The preconditioner's casts: dir 0, FP32 finest b = r / ||r|| and x = 0;
-// dir 1, z = ||r|| e (||r|| of the latest residual, set once per problem by
-// k_bnorm_final).
-__global__ void k_bpcg_cast(const LevelV<double>* __restrict__ f64,
-                            const LevelV<float>* __restrict__ f32, const int* __restrict__ pids,
-                            const Scalars* __restrict__ sc, int dir) {
-  const int z = blockIdx.z;
-  const int pr = pids[z];
-  if (!sc[pr].go) return;
-  const LevelV<double> L = f64[z];
-  const LevelV<float> F = f32[z];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x + 1;
-  const int j = blockIdx.y + 1;
-  if (i > L.nx) return;
-  const int o = j * L.pitch + i, of = j * F.pitch + i;
-  if (dir == 0) {
-    F.b[of] = float(L.b[o] * sc[pr].inv);
-    F.x[of] = 0.0f;
-  } else {
-    L.x[o] = sc[pr].rnorm * double(F.x[of]);
-  }
+// Dense user arrays <-> the finest planes, all problems in one launch (their
+// b, then their x, in `user`).  In: the right-hand side into the level's b
+// plane and the iterate into its x plane, or (pcg) into the CG vectors, b into
+// both.  Out: the iterate; a problem with a zero right-hand side runs no cycle
+// and has the solution 0.
+__global__ void __launch_bounds__(kKT) k_bpack(const BProb* __restrict__ prob,
+                                               const BUnit* __restrict__ units,
+                                               double* const* __restrict__ user, int nprob, int pcg) {
+  const BUnit u = units[blockIdx.x];
+  const BProb& q = prob[u.p];
+  const LevelV<double>& L = q.d;
+  const double* __restrict__ b = user[u.p];
+  const double* __restrict__ x = user[nprob + u.p];
+  for_pairs(L.nx, L.ny, u.local, u.count, [&](int j, int i, bool two) {
+    const size_t e = size_t(j - 1) * L.nx + i - 1;
+    const int o = j * L.pitch + i;
+    const double b0 = b[e], x0 = x[e], b1 = two ? b[e + 1] : 0.0, x1 = two ? x[e + 1] : 0.0;
+    store2(L.b + o, b0, b1, two);
+    if (pcg) store2(q.v.b + o, b0, b1, two);
+    store2((pcg ? q.v.x : L.x) + o, x0, x1, two);
+  });
 }
 
-// Dense user arrays <-> FP64 finest planes, batched over one finest side.
-// which: 0 the finest b plane, 1 its x plane, 2 the CG right-hand side B,
-// 3 the CG iterate X.
-__global__ void k_bpack(const LevelV<double>* __restrict__ f64, double* const* __restrict__ src,
-                        int which, const BPcg* __restrict__ vec) {
-  const int z = blockIdx.z;
-  const LevelV<double> L = f64[z];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= L.nx) return;
-  const double v = src[z][size_t(j) * L.nx + i];
-  double* dst = which == 0 ? L.b : which == 1 ? L.x : which == 2 ? vec[z].b : vec[z].x;
-  dst[(j + 1) * L.pitch + i + 1] = v;
-}
-
-// x = 0 for problems whose right-hand side is zero (they run no cycle).
-// The iterate (the finest x plane, or the CG iterate X when vec is given).
-__global__ void k_bzero_x(const LevelV<double>* __restrict__ f64, const int* __restrict__ pids,
-                          const Scalars* __restrict__ sc, const BPcg* __restrict__ vec) {
-  const int z = blockIdx.z;
-  if (sc[pids[z]].bnorm2 != 0.0) return;
-  const LevelV<double> L = f64[z];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x + 1;
-  const int j = blockIdx.y + 1;
-  if (i > L.nx) return;
-  (vec ? vec[z].x : L.x)[j * L.pitch + i] = 0.0;
-}
-
-__global__ void k_bunpack(const LevelV<double>* __restrict__ f64, double* const* __restrict__ dst,
-                          const BPcg* __restrict__ vec) {
-  const int z = blockIdx.z;
-  const LevelV<double> L = f64[z];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= L.nx) return;
-  dst[z][size_t(j) * L.nx + i] = (vec ? vec[z].x : L.x)[(j + 1) * L.pitch + i + 1];
+__global__ void __launch_bounds__(kKT) k_bunpack(const BProb* __restrict__ prob,
+                                                 const BUnit* __restrict__ units,
+                                                 const Scalars* __restrict__ sc,
+                                                 double* const* __restrict__ user, int nprob, int pcg) {
+  const BUnit u = units[blockIdx.x];
+  const BProb& q = prob[u.p];
+  const LevelV<double>& L = q.d;
+  double* __restrict__ x = user[nprob + u.p];
+  const bool zero = sc[u.p].bnorm2 == 0.0;
+  for_pairs(L.nx, L.ny, u.local, u.count, [&](int j, int i, bool two) {
+    const size_t e = size_t(j - 1) * L.nx + i - 1;
+    const double2 v = load2((pcg ? q.v.x : L.x) + j * L.pitch + i);
+    x[e] = zero ? 0.0 : v.x;
+    if (two) x[e + 1] = zero ? 0.0 : v.y;
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -458,28 +463,25 @@ struct BClass {                  // levels of one side and one kind across probl
   int parity_after_pre = 0;
 };
 
-struct BFine {                   // FP64 finest levels of the problems of one side
-  int n = 0;
-  int count = 0;
-  int* pids = nullptr;
-  LevelV<double>* f64 = nullptr;
-  LevelV<float>* f32 = nullptr;
-  double** user = nullptr;       // device array of user pointers (b, x)
-  BPcg* pcg = nullptr;           // the problems' CG planes (BMG_SOLVER_PCG), else null
-};
-
 struct Batch {
   int nprob = 0;
   bmg_options opt{};
   std::vector<Hierarchy*> hs;
   std::vector<int> side;
   std::vector<BClass> cls;       // descending side; per side 5-point first
-  std::vector<BFine> fines;
+  std::vector<BClass> sides;     // descending side, both kinds together
   Scalars* sc = nullptr;
   Scalars* sc_host = nullptr;
   double* partials = nullptr;
-  BCoarse* pc = nullptr;
-  int* any = nullptr;
+  BProb* prob = nullptr;
+  double** user = nullptr;       // the callers' b, then x
+  BUnit* units = nullptr;
+  BSpan* spans = nullptr;
+  int nunits = 0;
+  unsigned char* coarse_args = nullptr;   // of the shared-memory coarse kernel
+  size_t coarse_bytes = 0;
+  int* count = nullptr;          // problems done and active (k_bnorm_final)
+  bool legs = false;             // fused legs (one or two pre-, one post-sweep)
   void* arena = nullptr;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -506,9 +508,68 @@ void destroy_batch(Batch* b) {
   delete b;
 }
 
+// Tiles of a side's legs: the largest that still give every SM two blocks.
+template <int TX, int TY>
+int side_tiles(const BClass& c) { return cdiv(c.n, TX) * cdiv(c.n, TY) * c.count; }
+
+template <int NS, int TX, int TY, int NT>
+void launch_bdown(const BClass& c, const Scalars* sc, cudaStream_t s) {
+  constexpr size_t s9 = DownLeg<float, true, NS, TX, TY>::SMEM, s5 = DownLeg<float, false, NS, TX, TY>::SMEM;
+  constexpr size_t smem = s9 > s5 ? s9 : s5;
+  static const bool ready = [] {
+    cudaFuncSetAttribute(k_bdown<NS, TX, TY, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    return true;
+  }();
+  (void)ready;
+  launch_pdl(k_bdown<NS, TX, TY, NT>, dim3(cdiv(c.n, TX), cdiv(c.n, TY), c.count), dim3(NT), smem, s,
+             (const LevelV<float>*)c.view[0], (const LevelV<float>*)c.coarse, (const int*)c.pids, sc);
+  count_launch();
+}
+template <int TX, int TY, int NT>
+void launch_bup(const BClass& c, const Scalars* sc, cudaStream_t s) {
+  constexpr size_t s9 = UpLeg<float, true, TX, TY, false>::SMEM, s5 = UpLeg<float, false, TX, TY, false>::SMEM;
+  constexpr size_t smem = s9 > s5 ? s9 : s5;
+  static const bool ready = [] {
+    cudaFuncSetAttribute(k_bup<TX, TY, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    return true;
+  }();
+  (void)ready;
+  launch_pdl(k_bup<TX, TY, NT>, dim3(cdiv(c.n, TX), cdiv(c.n, TY), c.count), dim3(NT), smem, s,
+             (const LevelV<float>*)c.view[0], (const LevelV<float>*)c.coarse, (const int*)c.pids, sc);
+  count_launch();
+}
+template <int TX, int TY, int NT>
+void launch_bleg(const BClass& c, int ns, const Scalars* sc, cudaStream_t s) {
+  if (ns == 0)
+    launch_bup<TX, TY, NT>(c, sc, s);
+  else if (ns == 1)
+    launch_bdown<1, TX, TY, NT>(c, sc, s);
+  else
+    launch_bdown<2, TX, TY, NT>(c, sc, s);
+}
+// ns pre-sweeps of the down leg, 0: the up leg.
+void launch_side(const BClass& c, int ns, const Scalars* sc, cudaStream_t s) {
+  if (side_tiles<32, 16>(c) >= 2 * 152)
+    launch_bleg<32, 16, 256>(c, ns, sc, s);
+  else if (side_tiles<16, 8>(c) >= 2 * 152)
+    launch_bleg<16, 8, 128>(c, ns, sc, s);
+  else
+    launch_bleg<8, 8, 128>(c, ns, sc, s);
+}
+
+void launch_bcoarse(Batch* b, cudaStream_t s) {
+  launch_coarse_smem_batch(b->coarse_args, b->nprob, b->coarse_bytes, b->sc, s);
+}
+
 // Downward half of the batched V-cycle, coarse kernel, upward half.
 void enqueue_bvcycle(Batch* b, cudaStream_t s) {
   const int nu1 = b->opt.nu1, nu2 = b->opt.nu2;
+  if (b->legs) {
+    for (const BClass& c : b->sides) launch_side(c, nu1, b->sc, s);
+    launch_bcoarse(b, s);
+    for (auto it = b->sides.rbegin(); it != b->sides.rend(); ++it) launch_side(*it, 0, b->sc, s);
+    return;
+  }
   const bool oop = ((nu1 + nu2) & 1) != 0;
   for (BClass& c : b->cls) {
     int par = 0;
@@ -528,8 +589,7 @@ void enqueue_bvcycle(Batch* b, cudaStream_t s) {
     count_launch(2);
     c.parity_after_pre = par;
   }
-  k_bcoarse<<<b->nprob, 1024, 0, s>>>(b->pc, b->sc, nu1, nu2);
-  count_launch();
+  launch_bcoarse(b, s);
   for (auto it = b->cls.rbegin(); it != b->cls.rend(); ++it) {
     BClass& c = *it;
     int par = c.parity_after_pre;
@@ -545,59 +605,63 @@ void enqueue_bvcycle(Batch* b, cudaStream_t s) {
   }
 }
 
+void launch_bnorm_final(Batch* b, int what, bool use_handle, cudaStream_t s) {
+  launch_pdl(k_bnorm_final, dim3(b->nprob), dim3(kNT), 0, s, (const double*)b->partials,
+             (const BSpan*)b->spans, b->sc, what, b->handle, use_handle ? 1 : 0, b->count);
+  count_launch();
+}
+
 void enqueue_residuals(Batch* b, int what, bool use_handle, cudaStream_t s) {
-  for (BFine& f : b->fines) {
-    k_brefine_resid<<<dim3(kPB, f.count), kNT, 0, s>>>(f.f64, f.f32, f.pids, b->sc, b->partials,
-                                                      what);
-  }
-  k_bnorm_final<<<b->nprob, kNT, 0, s>>>(b->partials, b->sc, what);
-  k_bany<<<1, kNT, 0, s>>>(b->sc, b->nprob, b->handle, use_handle ? 1 : 0, b->any);
-  count_launch(int(b->fines.size()) + 2);
+  if (what == 0)
+    launch_pdl(k_brefine_resid<0>, dim3(b->nunits), dim3(kKT), 0, s, (const BProb*)b->prob,
+               (const BUnit*)b->units, (const Scalars*)b->sc, 0, b->partials);
+  else
+    launch_pdl(k_brefine_resid<1>, dim3(b->nunits), dim3(kKT), 0, s, (const BProb*)b->prob,
+               (const BUnit*)b->units, (const Scalars*)b->sc, b->legs ? 0 : 1, b->partials);
+  count_launch();
+  launch_bnorm_final(b, what, use_handle, s);
 }
 
 void enqueue_update(Batch* b, cudaStream_t s) {
-  for (BFine& f : b->fines) {
-    k_bupdate<<<dim3(cdiv(f.n, 128), f.n, f.count), 128, 0, s>>>(f.f64, f.f32, f.pids, b->sc);
-  }
-  count_launch(int(b->fines.size()));
+  launch_pdl(k_bupdate, dim3(b->nunits), dim3(kKT), 0, s, (const BProb*)b->prob, (const BUnit*)b->units,
+             (const Scalars*)b->sc);
+  count_launch();
 }
 
-void enqueue_pcg_vec(Batch* b, int what, cudaStream_t s) {
-  for (BFine& f : b->fines)
-    k_bpcg<<<dim3(kPB, f.count), kNT, 0, s>>>(f.f64, f.pcg, f.pids, b->sc, b->partials, what);
-  count_launch(int(b->fines.size()));
+template <int WHAT>
+void enqueue_pcg_vec(Batch* b, cudaStream_t s) {
+  launch_pdl(k_bpcg<WHAT>, dim3(b->nunits), dim3(kKT), 0, s, (const BProb*)b->prob, (const BUnit*)b->units,
+             (const Scalars*)b->sc, b->partials);
+  count_launch();
 }
 
-void enqueue_pcg_cast(Batch* b, int dir, cudaStream_t s) {
-  for (BFine& f : b->fines)
-    k_bpcg_cast<<<dim3(cdiv(f.n, 128), f.n, f.count), 128, 0, s>>>(f.f64, f.f32, f.pids, b->sc, dir);
-  count_launch(int(b->fines.size()));
+void enqueue_pcg_scalar(Batch* b, int what, cudaStream_t s) {
+  launch_pdl(k_bpcg_scalar, dim3(b->nprob), dim3(kNT), 0, s, (const double*)b->partials,
+             (const BSpan*)b->spans, b->sc, what);
+  count_launch();
 }
 
-// The first residual of PCG (r = B - A X, z = 0) and its stop test.
+// The first residual of PCG (r = B - A X) and its stop test.
 void enqueue_pcg_init(Batch* b, cudaStream_t s) {
-  enqueue_pcg_vec(b, BPCG_INIT, s);
-  k_bnorm_final<<<b->nprob, kNT, 0, s>>>(b->partials, b->sc, 1);
-  k_bany<<<1, kNT, 0, s>>>(b->sc, b->nprob, b->handle, 0, b->any);
-  count_launch(2);
+  enqueue_pcg_vec<K_INIT>(b, s);
+  launch_bnorm_final(b, 1, false, s);
 }
 
 // One batched PCG iteration of the active problems: z = M^{-1} r (the FP32
-// batched V-cycle between the casts), r.z and beta, p = z + beta p,
-// q = A p and alpha, x += alpha p and r -= alpha q, the stop test, any.
+// batched V-cycle after the cast), r.z and beta, p = z + beta p, q = A p and
+// alpha, x += alpha p and r -= alpha q, the stop test.
 void enqueue_pcg_iter(Batch* b, bool use_handle, cudaStream_t s) {
-  enqueue_pcg_cast(b, 0, s);
+  launch_pdl(k_bpcg_cast, dim3(b->nunits), dim3(kKT), 0, s, (const BProb*)b->prob, (const BUnit*)b->units,
+             (const Scalars*)b->sc, b->legs ? 0 : 1);
+  count_launch();
   enqueue_bvcycle(b, s);
-  enqueue_pcg_cast(b, 1, s);
-  enqueue_pcg_vec(b, BPCG_RZ, s);
-  k_bpcg_scalar<<<b->nprob, kNT, 0, s>>>(b->partials, b->sc, BPCG_RZ);
-  enqueue_pcg_vec(b, BPCG_P, s);
-  enqueue_pcg_vec(b, BPCG_AP, s);
-  k_bpcg_scalar<<<b->nprob, kNT, 0, s>>>(b->partials, b->sc, BPCG_AP);
-  enqueue_pcg_vec(b, BPCG_XR, s);
-  k_bnorm_final<<<b->nprob, kNT, 0, s>>>(b->partials, b->sc, 1);
-  k_bany<<<1, kNT, 0, s>>>(b->sc, b->nprob, b->handle, use_handle ? 1 : 0, b->any);
-  count_launch(4);
+  enqueue_pcg_vec<K_RZ>(b, s);
+  enqueue_pcg_scalar(b, K_RZ, s);
+  enqueue_pcg_vec<K_P>(b, s);
+  enqueue_pcg_vec<K_AP>(b, s);
+  enqueue_pcg_scalar(b, K_AP, s);
+  enqueue_pcg_vec<K_XR>(b, s);
+  launch_bnorm_final(b, 1, use_handle, s);
 }
 
 // Pick the fastest tile variant of every class by timing sweeps on the batch
@@ -766,16 +830,18 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
     std::vector<int> pids;
     std::vector<LevelV<float>> v0, v1, vc;
   };
+  b->legs = (opt.nu1 == 1 || opt.nu1 == 2) && opt.nu2 == 1;
   std::vector<HostClass> hc;
   for (int m : sides) {
-    for (int kind = 0; kind < 2; ++kind) {
+    // legs: one class per side (kind 2); else one per side and kind
+    for (int kind = b->legs ? 2 : 0; kind < (b->legs ? 3 : 2); ++kind) {
       HostClass x;
       x.c.n = m;
       x.c.nine = kind == 1;
       for (int p = 0; p < nprob; ++p) {
         const Hierarchy* h = b->hs[p];
         const bool finest = b->side[p] == m;
-        if (b->side[p] < m || finest == x.c.nine) continue;
+        if (b->side[p] < m || (kind < 2 && finest == x.c.nine)) continue;
         int l = h->L - 1;
         while (h->f[l].nx != m) --l;
         LevelV<float> a = h->f[l], bb = h->f[l];
@@ -789,18 +855,25 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
       if (x.c.count) hc.push_back(std::move(x));
     }
   }
-  std::map<int, std::vector<int>> by_side;
-  for (int p = 0; p < nprob; ++p) by_side[b->side[p]].push_back(p);
   // device arena for the descriptors
   size_t bytes = 0;
   auto al = [](size_t v) { return ((v + 255) / 256) * 256; };
   for (auto& x : hc) bytes += al(sizeof(int) * x.c.count) + 3 * al(sizeof(LevelV<float>) * x.c.count);
-  for (auto& kv : by_side)
-    bytes += al(sizeof(int) * kv.second.size()) + al(sizeof(LevelV<double>) * kv.second.size()) +
-             al(sizeof(LevelV<float>) * kv.second.size()) + al(sizeof(double*) * kv.second.size()) +
-             al(sizeof(BPcg) * kv.second.size());
-  bytes += al(sizeof(Scalars) * nprob) + al(sizeof(double) * kPB * nprob) +
-           al(sizeof(BCoarse) * nprob) + al(sizeof(int));
+  // units of FP64 work, by problem
+  std::vector<BUnit> units;
+  std::vector<BSpan> spans;
+  for (int p = 0; p < nprob; ++p) {
+    const int k = cdiv(pair_runs(n[p], n[p]), kUnitRuns);
+    spans.push_back(BSpan{int(units.size()), k});
+    for (int i = 0; i < k; ++i) units.push_back(BUnit{p, i, k});
+  }
+  b->nunits = int(units.size());
+  std::vector<unsigned char> cargs;
+  coarse_smem_batch_args(b->hs[0], nullptr, cargs);
+  const size_t cargs_one = cargs.size();
+  bytes += al(sizeof(Scalars) * nprob) + al(sizeof(double) * b->nunits) + al(sizeof(BProb) * nprob) +
+           al(sizeof(BUnit) * b->nunits) + al(sizeof(BSpan) * nprob) + al(cargs_one * nprob) +
+           al(2 * sizeof(int)) + al(2 * sizeof(double*) * nprob);
   if (cudaMalloc(&b->arena, bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(BMG_ENOMEM);
@@ -817,48 +890,31 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
     cudaMemcpyAsync(c.view[0], x.v0.data(), sizeof(LevelV<float>) * c.count, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(c.view[1], x.v1.data(), sizeof(LevelV<float>) * c.count, cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(c.coarse, x.vc.data(), sizeof(LevelV<float>) * c.count, cudaMemcpyHostToDevice, s);
-    b->cls.push_back(c);
-  }
-  for (auto& kv : by_side) {
-    BFine f;
-    f.n = kv.first;
-    f.count = int(kv.second.size());
-    std::vector<LevelV<double>> v64;
-    std::vector<LevelV<float>> v32;
-    std::vector<BPcg> vp;
-    for (int p : kv.second) {
-      const Hierarchy* h = b->hs[p];
-      v64.push_back(h->d.back());
-      v32.push_back(h->f.back());
-      vp.push_back(BPcg{h->pcg_x, h->pcg_b, h->pcg_p, h->pcg_q});
-    }
-    f.pids = carve<int>(cur, f.count);
-    f.f64 = carve<LevelV<double>>(cur, f.count);
-    f.f32 = carve<LevelV<float>>(cur, f.count);
-    f.user = carve<double*>(cur, f.count);
-    BPcg* pcg_dev = carve<BPcg>(cur, f.count);
-    if (opt.solver == BMG_SOLVER_PCG) {
-      f.pcg = pcg_dev;
-      cudaMemcpyAsync(f.pcg, vp.data(), sizeof(BPcg) * f.count, cudaMemcpyHostToDevice, s);
-    }
-    cudaMemcpyAsync(f.pids, kv.second.data(), sizeof(int) * f.count, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(f.f64, v64.data(), sizeof(LevelV<double>) * f.count, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(f.f32, v32.data(), sizeof(LevelV<float>) * f.count, cudaMemcpyHostToDevice, s);
-    b->fines.push_back(f);
+    (b->legs ? b->sides : b->cls).push_back(c);
   }
   b->sc = carve<Scalars>(cur, nprob);
-  b->partials = carve<double>(cur, size_t(kPB) * nprob);
-  b->pc = carve<BCoarse>(cur, nprob);
-  b->any = carve<int>(cur, 1);
-  std::vector<BCoarse> pcs(nprob);
+  b->partials = carve<double>(cur, b->nunits);
+  b->prob = carve<BProb>(cur, nprob);
+  b->units = carve<BUnit>(cur, b->nunits);
+  b->spans = carve<BSpan>(cur, nprob);
+  b->coarse_args = carve<unsigned char>(cur, cargs_one * nprob);
+  b->count = carve<int>(cur, 2);
+  b->user = carve<double*>(cur, 2 * nprob);
+  std::vector<BProb> probs;
+  cargs.clear();
   for (int p = 0; p < nprob; ++p) {
     const Hierarchy* h = b->hs[p];
-    pcs[p] = BCoarse{h->dlev32, h->cinv, h->threshold, h->n0,
-                     h->threshold < h->L ? 1 : 0};
+    probs.push_back(BProb{h->d.back(), h->f.back(), PcgVec{h->pcg_x, h->pcg_b, h->pcg_p, h->pcg_q}});
+    b->coarse_bytes = std::max(b->coarse_bytes, coarse_smem_batch_args(h, &b->sc[p].err, cargs));
+    if (!h->coarse_smem) return fail(BMG_ECUDA);   // (levels of side <= 31 always fit)
   }
-  cudaMemcpyAsync(b->pc, pcs.data(), sizeof(BCoarse) * nprob, cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(b->prob, probs.data(), sizeof(BProb) * nprob, cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(b->units, units.data(), sizeof(BUnit) * units.size(), cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(b->spans, spans.data(), sizeof(BSpan) * nprob, cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(b->coarse_args, cargs.data(), cargs.size(), cudaMemcpyHostToDevice, s);
+  cudaMemsetAsync(b->count, 0, 2 * sizeof(int), s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(BMG_ECUDA);
-  int rc = autotune(b, s);
+  int rc = b->legs ? BMG_OK : autotune(b, s);
   if (rc) return fail(rc);
   if ((rc = build_graph(b))) {
     set_last_error("batch setup: building the CUDA graph failed (%s)",
@@ -877,23 +933,15 @@ extern "C" int bmg_batch_solve(bmg_batch* bp, const double* const* b_dev, double
   if (!b || !b_dev || !x_dev || !(tol > 0.0)) return BMG_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const double t0 = now_ms();
-  // pack b and x (batched per finest side)
-  std::map<int, std::vector<int>> by_side;
-  for (int p = 0; p < b->nprob; ++p) by_side[b->side[p]].push_back(p);
   const bool pcg = b->opt.solver == BMG_SOLVER_PCG;
-  for (int pass = 0; pass < 2; ++pass) {
-    for (BFine& f : b->fines) {
-      std::vector<double*> ptr;
-      for (int p : by_side[f.n]) ptr.push_back(pass == 0 ? const_cast<double*>(b_dev[p]) : x_dev[p]);
-      cudaMemcpyAsync(f.user, ptr.data(), sizeof(double*) * ptr.size(), cudaMemcpyHostToDevice, s);
-      const dim3 g(cdiv(f.n, 128), f.n, f.count);
-      // V-cycles: b and x into the finest planes; PCG: b also into B, x into X
-      if (pass == 0 || !pcg) k_bpack<<<g, 128, 0, s>>>(f.f64, f.user, pass, f.pcg);
-      if (pcg) k_bpack<<<g, 128, 0, s>>>(f.f64, f.user, pass == 0 ? 2 : 3, f.pcg);
-      count_launch(pcg && pass == 0 ? 2 : 1);
-    }
-    if (cudaStreamSynchronize(s) != cudaSuccess) return BMG_ECUDA;
+  std::vector<double*> user(2 * size_t(b->nprob));
+  for (int p = 0; p < b->nprob; ++p) {
+    user[p] = const_cast<double*>(b_dev[p]);
+    user[b->nprob + p] = x_dev[p];
   }
+  cudaMemcpyAsync(b->user, user.data(), sizeof(double*) * user.size(), cudaMemcpyHostToDevice, s);
+  k_bpack<<<b->nunits, kKT, 0, s>>>(b->prob, b->units, b->user, b->nprob, pcg ? 1 : 0);
+  count_launch();
   for (int p = 0; p < b->nprob; ++p) {
     Scalars z{};
     z.tol = tol;
@@ -907,16 +955,8 @@ extern "C" int bmg_batch_solve(bmg_batch* bp, const double* const* b_dev, double
   else
     enqueue_residuals(b, 1, false, s);     // first residual and stop test
   if (cudaGraphLaunch(b->exec, s) != cudaSuccess) return BMG_ECUDA;
-  for (BFine& f : b->fines) {
-    k_bzero_x<<<dim3(cdiv(f.n, 128), f.n, f.count), 128, 0, s>>>(f.f64, f.pids, b->sc, f.pcg);
-    count_launch();
-    std::vector<double*> ptr;
-    for (int p : by_side[f.n]) ptr.push_back(x_dev[p]);
-    cudaMemcpyAsync(f.user, ptr.data(), sizeof(double*) * ptr.size(), cudaMemcpyHostToDevice, s);
-    k_bunpack<<<dim3(cdiv(f.n, 128), f.n, f.count), 128, 0, s>>>(f.f64, f.user, f.pcg);
-    count_launch();
-    if (cudaStreamSynchronize(s) != cudaSuccess) return BMG_ECUDA;
-  }
+  k_bunpack<<<b->nunits, kKT, 0, s>>>(b->prob, b->units, b->sc, b->user, b->nprob, pcg ? 1 : 0);
+  count_launch();
   if (cudaMemcpyAsync(b->sc_host, b->sc, sizeof(Scalars) * b->nprob, cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
@@ -927,6 +967,7 @@ extern "C" int bmg_batch_solve(bmg_batch* bp, const double* const* b_dev, double
     const Scalars& r = b->sc_host[p];
     if (per_prob) per_prob[p] = bmg_info{r.cycles, b->hs[p]->threshold, r.rel, b->setup_ms, ms, 1};
     if (r.err & DEV_NAN) rc = BMG_ENAN;
+    else if ((r.err & DEV_TIMEOUT) && (rc == BMG_OK || rc == BMG_ENOCONV)) rc = BMG_ETIMEOUT;
     else if (!(r.rel <= tol) && r.bnorm2 > 0.0 && rc == BMG_OK) rc = BMG_ENOCONV;
   }
   return rc;

@@ -383,7 +383,7 @@ __device__ __forceinline__ void solve0(const SmArgs<T>& a, const Lv& L) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kNT, 1) k_coarse_smem(const __grid_constant__ SmArgs<T> a) {
+__device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   using namespace tma_detail;
   __shared__ __align__(8) uint64_t bar;
   const int top = a.thr - 1;
@@ -449,6 +449,26 @@ __global__ void __launch_bounds__(kNT, 1) k_coarse_smem(const __grid_constant__ 
     const int j = t / L.nx + 1, i = t - (j - 1) * L.nx + 1;
     a.x[j * a.pitch + i] = sh<T>(L.x + j * L.sp + i);
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kNT, 1) k_coarse_smem(const __grid_constant__ SmArgs<T> a) {
+  coarse_smem_body<T>(a);
+}
+
+// One problem per block; a problem that has stopped is left alone.  (`go` was
+// settled before the kernel that precedes this one began.)
+__global__ void __launch_bounds__(kNT, 1) k_coarse_smem_batch(const SmArgs<float>* __restrict__ args,
+                                                             const Scalars* __restrict__ sc) {
+  __shared__ SmArgs<float> a;
+  if (!sc[blockIdx.x].go) {
+    griddep_wait();   // (the kernel that follows relies on it)
+    return;
+  }
+  const int* src = reinterpret_cast<const int*>(args + blockIdx.x);
+  for (int e = threadIdx.x; e < int(sizeof(a) / sizeof(int)); e += kNT) reinterpret_cast<int*>(&a)[e] = src[e];
+  __syncthreads();
+  coarse_smem_body<float>(a);
 }
 
 // The image: blockIdx.x walks the constant planes of the levels (NK9 + NPW
@@ -582,6 +602,33 @@ void launch_coarse_smem(Hierarchy* h, const LevelV<T>& top, int thr, bool top_ze
   a.b = top.b;
   a.pitch = top.pitch;
   launch_pdl(k_coarse_smem<T>, dim3(1), dim3(kNT), bytes, s, a);
+}
+
+size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned char>& out) {
+  static_assert(sizeof(SmArgs<float>) % sizeof(int) == 0, "copied by words");
+  SmArgs<float> a{};
+  const size_t bytes = layout<float>(h, h->threshold, a);
+  const LevelV<float>& top = h->f[h->threshold - 1];
+  a.top_zero = 1;
+  a.err = err;
+  a.x = top.x;
+  a.b = top.b;
+  a.pitch = top.pitch;
+  const unsigned char* p = reinterpret_cast<const unsigned char*>(&a);
+  out.insert(out.end(), p, p + sizeof(a));
+  return bytes;
+}
+
+void launch_coarse_smem_batch(const void* args, int count, size_t bytes, const Scalars* sc, cudaStream_t s) {
+  static const bool ready = [] {
+    cudaFuncSetAttribute(k_coarse_smem_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         int(kCoarseImageMax));
+    return true;
+  }();
+  (void)ready;
+  launch_pdl(k_coarse_smem_batch, dim3(unsigned(count)), dim3(kNT), bytes, s,
+             static_cast<const SmArgs<float>*>(args), sc);
+  count_launch();
 }
 
 template void launch_coarse_smem<double>(Hierarchy*, const LevelV<double>&, int, bool, cudaStream_t);

@@ -545,6 +545,13 @@ template <typename T>
 void launch_coarse_smem(Hierarchy* h, const LevelV<T>& top, int threshold, bool top_zero,
                         cudaStream_t s);
 
+// The sub-cycles of many FP32 hierarchies in one launch, one block each, from
+// zero iterates: appends a hierarchy's arguments (err: its error word) to
+// `out` and returns the shared memory it needs; `args`: their copies on the device, `sc` the
+// problems' states (go).
+size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned char>& out);
+void launch_coarse_smem_batch(const void* args, int count, size_t bytes, const Scalars* sc, cudaStream_t s);
+
 // Prescaled finest level (bmg_sweep.cu): whether the finest FP64 level of a
 // hierarchy is prescaled; the coefficient planes W/C, E/C, S/C, N/C (setup)
 // and b/C (whenever the level's b changes).
@@ -589,8 +596,8 @@ void launch_pcg_xr(Hierarchy* h, cudaStream_t s, bool in_graph);
 void launch_pcg_rz(Hierarchy* h, bool first, cudaStream_t s);
 void launch_pcg_p(Hierarchy* h, cudaStream_t s);
 // z = M^{-1} r for PCG: one V-cycle on the residual in the finest level's b
-// plane (FP64 levels; BMG_FP32_REFINE: r / ||r|| cast to the FP32 finest
-// level, the FP32 cycle, z = ||r|| e cast back).
+// plane (FP64 levels, z in the x plane; BMG_FP32_REFINE: r / ||r|| cast to the
+// FP32 finest level and the FP32 cycle, z = ||r|| times its iterate).
 void launch_pcg_precond(Hierarchy* h, cudaStream_t s);
 
 // One V-cycle of the FP64 (d) or FP32 (f) hierarchy (bmg_api.cu);
@@ -604,6 +611,11 @@ template <typename T>
 void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* dlev, int thr,
                     cudaStream_t s, int top = -1, bool skip_first = false, bool top_zero = false,
                     int* norm_partials = nullptr);
+
+// Whether a cycle that starts from a zero finest iterate (top_zero, on the
+// FP64 or, with BMG_FP32_REFINE, the FP32 hierarchy) reads that iterate, so
+// that it must be stored; most take the zero as given.
+bool cycle_reads_zero_top(const Hierarchy* h);
 
 void launch_assemble_backward(const double* k, const double* u, const double* lam,
                               double* g, int nx, int ny, cudaStream_t s);
