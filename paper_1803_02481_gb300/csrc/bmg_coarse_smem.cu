@@ -549,11 +549,7 @@ size_t layout(const Hierarchy* h, int thr, SmArgs<T>& a) {
 
 template <typename T>
 void prepare() {
-  static const bool done = [] {
-    cudaFuncSetAttribute(k_coarse_smem<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         int(kCoarseImageMax));
-    return true;
-  }();
+  static const bool done = use_shared(k_coarse_smem<T>, kCoarseImageMax);
   (void)done;
 }
 
@@ -620,11 +616,7 @@ size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned
 }
 
 void launch_coarse_smem_batch(const void* args, int count, size_t bytes, const Scalars* sc, cudaStream_t s) {
-  static const bool ready = [] {
-    cudaFuncSetAttribute(k_coarse_smem_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         int(kCoarseImageMax));
-    return true;
-  }();
+  static const bool ready = use_shared(k_coarse_smem_batch, kCoarseImageMax);
   (void)ready;
   launch_pdl(k_coarse_smem_batch, dim3(unsigned(count)), dim3(kNT), bytes, s,
              static_cast<const SmArgs<float>*>(args), sc);

@@ -124,6 +124,21 @@ __device__ __forceinline__ void griddep_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 bool pdl_enabled();
+
+// Opts a kernel into `bytes` of dynamic shared memory and asks for the whole
+// of the unified L1 as shared memory: with the default carve-out the driver
+// made room for one block of the kernels here, and they ran at one block per
+// SM (measured).
+template <typename... KArgs>
+inline bool use_shared(void (*kern)(KArgs...), size_t bytes) {
+  const bool a = bytes <= 48 * 1024 ||
+                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)) ==
+                     cudaSuccess;
+  const bool b = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      int(cudaSharedmemCarveoutMaxShared)) == cudaSuccess;
+  return a && b;
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t s, Args... args) {

@@ -109,6 +109,11 @@ double predict_vcycle_us(const Hierarchy* h, int thr, int ctas) {
 // 46.8; FP32 511^2 62.2, 60.8, 61.7 (a 31^2 level keeps one SM's FP64 pipes
 // busy for longer than two launches over many SMs take).
 constexpr double kSmemPoints = 300.0;
+// The same for line smoothing, whose sub-cycle works from L2.  Measured us
+// per alternating V(2,1) cycle with the largest level at 7^2, 15^2 and 31^2:
+// 255^2 FP64 564, 557, 613, FP32 365, 369, 418; 2047^2 FP64 2273, 2280, 2355,
+// FP32 1402, 1414, 1480.
+constexpr double kLinePoints = 100.0;
 
 void choose_schedule(Hierarchy* h) {
   const bool point = h->opt.smoother == BMG_SMOOTH_POINT;
@@ -149,6 +154,12 @@ void choose_schedule(Hierarchy* h) {
       h->threshold = thr;
       h->coarse_ctas = 1;
     }
+  }
+  if (!point && h->opt.coarse_threshold < 1) {
+    h->threshold = 1;
+    while (h->threshold < h->L &&
+           double(h->geo64[h->threshold].nx) * h->geo64[h->threshold].ny <= kLinePoints)
+      ++h->threshold;
   }
   for (int thr = 1; thr <= h->L && thr <= 16; ++thr)
     h->predicted_us[thr - 1] = predict_vcycle_us(h, thr, h->coarse_ctas);

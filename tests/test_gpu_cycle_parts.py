@@ -83,3 +83,35 @@ def test_coarsest_solve_matches_dense(nx, ny):
     # the dense solve it is compared with: both n kappa eps at most
     tol = 2 * n * np.linalg.cond(a) * np.finfo(float).eps * np.linalg.norm(want)
     assert np.linalg.norm(x.cpu().numpy().ravel() - want) <= tol
+
+
+@pytest.mark.parametrize("smoother", [bm.BMG_SMOOTH_XLINE, bm.BMG_SMOOTH_YLINE, bm.BMG_SMOOTH_ALTLINE])
+@pytest.mark.parametrize("nx,ny", [(2, 9), (15, 16), (16, 15), (17, 33), (31, 300), (257, 47), (530, 560), (560, 530)])
+def test_line_sweep_solves_its_last_lines(nx, ny, smoother):
+    """Line lengths below, at and above one block of 16, several groups of
+    separators, levels on both sides of the one-kernel step's size: after a
+    sweep the lines of the colour solved last have zero residual.  A line's
+    solve is backward stable up to a small factor, so its residual is within
+    64 eps of the terms of its equations (the 9-point diagonal bound
+    2 C |x|)."""
+    rng = np.random.default_rng(nx + ny)
+    h = bm.setup(torch.from_numpy(10.0 ** rng.uniform(-1, 1, (ny, nx))).cuda(),
+                 bm.default_options(smoother=smoother))
+    top = h.nlevels - 1
+    for level in {top, max(1, top - 1)} if top else {0}:
+        if level == 0:
+            continue
+        sx, sy = h.level_shape(level)
+        b = torch.from_numpy(rng.uniform(-1, 1, (sy, sx))).cuda()
+        x = torch.from_numpy(rng.uniform(-1, 1, (sy, sx))).cuda()
+        scale = (2.0 * torch.from_numpy(h.level_stencil(level)["C"]).cuda()).max()
+        for reverse in (False, True):
+            h.op_relax(level, x, b, 1, reverse=reverse)
+            r = h.op_residual(level, x, b, torch.empty_like(b)).abs()
+            # forward: x-lines then y-lines, odd lines first; reverse: the whole turned
+            rows = smoother == bm.BMG_SMOOTH_XLINE or (smoother == bm.BMG_SMOOTH_ALTLINE and reverse)
+            first = 0 if reverse else 1      # 0-based index of the colour solved last
+            last = r[first::2] if rows else r[:, first::2]
+            if last.numel():
+                assert last.max() <= 64 * np.finfo(float).eps * scale * x.abs().max() + 1e-15
+    h.destroy()
