@@ -83,39 +83,69 @@ enum { E3_BADK = 1, E3_BADDEN = 2, E3_NOTSPD = 4 };
 
 __device__ __forceinline__ double hmean(double lo, double hi) { return 2.0 * lo * hi / (lo + hi); }
 
-__global__ void k3_assemble(const double* __restrict__ k, Lev3 L, int* err) {
-  const int i0 = blockIdx.x * blockDim.x + threadIdx.x, j0 = blockIdx.y, k0 = blockIdx.z;
-  if (i0 >= L.nx) return;
+// One thread per cell and z: a block owns kA3X x kA3Y cells of a column of
+// kA3Z layers and forms each face once (the west, south and lower face of its
+// cell, the tile's last column and row the faces beyond), passing them on
+// through shared memory and, upwards, in a register: a division costs nine
+// FP64 instructions, and forming all six faces per cell took 2.5 ms of a
+// 255^3 setup.  The east face of a cell is the same call as the west face of
+// the next, so every value is as before.
+constexpr int kA3X = 32, kA3Y = 8, kA3Z = 16;
+__global__ void __launch_bounds__(kA3X * kA3Y) k3_assemble(const double* __restrict__ k, Lev3 L, int* err) {
+  __shared__ double fw[kA3Y][kA3X + 1], fs[kA3Y + 1][kA3X];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int i0 = blockIdx.x * kA3X + tx, j0 = blockIdx.y * kA3Y + ty;
   const int nx = L.nx, ny = L.ny, nz = L.nz;
+  const bool in = i0 < nx && j0 < ny;
   const size_t sxy = size_t(nx) * ny;
-  const size_t q = size_t(k0) * sxy + size_t(j0) * nx + i0;
-  const double kc = k[q];
-  if (!(kc > 0.0) || !(kc < INFINITY)) atomicOr(err, E3_BADK);
-  const double aE = i0 < nx - 1 ? hmean(kc, k[q + 1]) : 0.0;
-  const double aW = i0 > 0 ? hmean(k[q - 1], kc) : 0.0;
-  const double aN = j0 < ny - 1 ? hmean(kc, k[q + nx]) : 0.0;
-  const double aS = j0 > 0 ? hmean(k[q - nx], kc) : 0.0;
-  const double aU = k0 < nz - 1 ? hmean(kc, k[q + sxy]) : 0.0;
-  const double aD = k0 > 0 ? hmean(k[q - sxy], kc) : 0.0;
-  double c = 0.0;
-  c = __dadd_rn(c, aE);
-  c = __dadd_rn(c, aW);
-  c = __dadd_rn(c, i0 == 0 ? 2.0 * kc : 0.0);
-  c = __dadd_rn(c, i0 == nx - 1 ? 2.0 * kc : 0.0);
-  c = __dadd_rn(c, aN);
-  c = __dadd_rn(c, aS);
-  c = __dadd_rn(c, j0 == 0 ? 2.0 * kc : 0.0);
-  c = __dadd_rn(c, j0 == ny - 1 ? 2.0 * kc : 0.0);
-  c = __dadd_rn(c, aU);
-  c = __dadd_rn(c, aD);
-  c = __dadd_rn(c, k0 == 0 ? 2.0 * kc : 0.0);
-  c = __dadd_rn(c, k0 == nz - 1 ? 2.0 * kc : 0.0);
-  const int o = idx3(L, i0 + 1, j0 + 1, k0 + 1);
-  L.C[o] = c;
-  L.iC[o] = 1.0 / c;
-  L.A[neg_index(-1, 0, 0)][o] = aW;
-  L.A[neg_index(0, -1, 0)][o] = aS;
-  L.A[neg_index(0, 0, -1)][o] = aD;
+  const int k1 = min(int(blockIdx.z + 1) * kA3Z, nz);
+  size_t q = size_t(blockIdx.z) * kA3Z * sxy + size_t(j0) * nx + i0;
+  double kc = 1.0, aD = 0.0;
+  if (in) {
+    kc = k[q];
+    if (blockIdx.z > 0) aD = hmean(k[q - sxy], kc);
+  }
+  for (int k0 = blockIdx.z * kA3Z; k0 < k1; ++k0, q += sxy) {
+    double kn = 1.0, aU = 0.0;
+    if (in) {
+      if (!(kc > 0.0) || !(kc < INFINITY)) atomicOr(err, E3_BADK);
+      if (k0 < nz - 1) {
+        kn = k[q + sxy];
+        aU = hmean(kc, kn);
+      }
+      fw[ty][tx] = i0 > 0 ? hmean(k[q - 1], kc) : 0.0;
+      fs[ty][tx] = j0 > 0 ? hmean(k[q - nx], kc) : 0.0;
+      if (tx == kA3X - 1) fw[ty][kA3X] = i0 < nx - 1 ? hmean(kc, k[q + 1]) : 0.0;
+      if (ty == kA3Y - 1) fs[kA3Y][tx] = j0 < ny - 1 ? hmean(kc, k[q + nx]) : 0.0;
+    }
+    __syncthreads();
+    if (in) {
+      const double aW = fw[ty][tx], aS = fs[ty][tx];
+      const double aE = i0 < nx - 1 ? fw[ty][tx + 1] : 0.0, aN = j0 < ny - 1 ? fs[ty + 1][tx] : 0.0;
+      double c = 0.0;
+      c = __dadd_rn(c, aE);
+      c = __dadd_rn(c, aW);
+      if (i0 == 0) c = __dadd_rn(c, 2.0 * kc);
+      if (i0 == nx - 1) c = __dadd_rn(c, 2.0 * kc);
+      c = __dadd_rn(c, aN);
+      c = __dadd_rn(c, aS);
+      if (j0 == 0) c = __dadd_rn(c, 2.0 * kc);
+      if (j0 == ny - 1) c = __dadd_rn(c, 2.0 * kc);
+      c = __dadd_rn(c, aU);
+      c = __dadd_rn(c, aD);
+      if (k0 == 0) c = __dadd_rn(c, 2.0 * kc);
+      if (k0 == nz - 1) c = __dadd_rn(c, 2.0 * kc);
+      const int o = idx3(L, i0 + 1, j0 + 1, k0 + 1);
+      L.C[o] = c;
+      L.iC[o] = 1.0 / c;
+      L.A[neg_index(-1, 0, 0)][o] = aW;
+      L.A[neg_index(0, -1, 0)][o] = aS;
+      L.A[neg_index(0, 0, -1)][o] = aD;
+    }
+    __syncthreads();
+    kc = kn;
+    aD = aU;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -126,92 +156,133 @@ __global__ void k3_assemble(const double* __restrict__ k, Lev3 L, int* err) {
 // offset order (dk, dj, di) ascending, products and sums unfused.
 // ---------------------------------------------------------------------------
 
-// The weights of fine point (i, j, k) if it belongs to the pass.
-__device__ void weights_point(const Lev3& F, int i, int j, int k, int pass, int* err) {
-  const int fr[3] = {i & 1, j & 1, k & 1};    // 1: between coarse points in that direction
-  const int nb = fr[0] + fr[1] + fr[2];
-  if (nb != pass) return;
+// What bounds it: FP64 instructions.  With the point's kind known at compile
+// time every offset, slot and coupling index is a constant (the general loops
+// kept their 27 couplings in local memory), a 7-point level visits its six
+// couplings only, which are not negative (the other terms are exact zeros),
+// and the divisions by one denominator share its reciprocal: 7.7 -> 2.3 ms at
+// 255^3.
+
+// w / den for several w: q = w r with r = 1 / den rounded, corrected by the
+// exact remainder, which gives the rounded quotient (Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000 processor", 1990),
+// inside the range where no product over- or underflows (judged by the high
+// words, in integers).
+static __device__ __noinline__ double rare_divide(double a, double b) { return a / b; }
+struct Denominator {
+  double den, r;
+  int hd;        // high word of den (its sign and exponent)
+  bool plain;
+};
+__device__ __forceinline__ Denominator denominator(double d) {
+  const int hd = __double2hiint(d);
+  return Denominator{d, __drcp_rn(d), hd, hd < (200 << 20) || hd > (1800 << 20)};
+}
+__device__ __forceinline__ double divide(double w, const Denominator& d) {
+  const int hw = __double2hiint(w) & 0x7FFFFFFF;
+  if (d.plain || (hw != 0 && (hw < d.hd - (100 << 20) || hw > d.hd + (100 << 20)))) return rare_divide(w, d.den);
+  const double q = w * d.r;
+  return fma(fma(-q, d.den, w), d.r, q);
+}
+
+// The weights of fine point (i, j, k) that lies between coarse points in the
+// directions with FX, FY, FZ = 1 (at least one).
+template <bool SEVEN, int FX, int FY, int FZ>
+__device__ __forceinline__ void weights_point(const Lev3& F, int i, int j, int k, int* err) {
+  if (i > F.nx || j > F.ny || k > F.nz) return;
   const int o = idx3(F, i, j, k);
-  if (nb == 0) {
-    F.P[0][o] = 1.0;
-    return;
-  }
-  // couplings with the lumping of non-M-matrix rows
-  double a[27];
+  constexpr int fr[3] = {FX, FY, FZ};
+  // couplings with the lumping of non-M-matrix rows, collapsed onto the
+  // directions the point is not coarse-aligned in
   const double C = F.C[o];
   double sum = 0.0, neg = 0.0;
-  for (int dk = -1; dk <= 1; ++dk)
-    for (int dj = -1; dj <= 1; ++dj)
-      for (int di = -1; di <= 1; ++di) {
-        const int t = (dk + 1) * 9 + (dj + 1) * 3 + (di + 1);
-        if (t == 13) {
-          a[t] = 0.0;
-          continue;
-        }
-        const double v = coupling(F, o, di, dj, dk);
-        sum = __dadd_rn(sum, v);
-        neg = __dadd_rn(neg, fmin(v, 0.0));
-        a[t] = fmax(v, 0.0);
-      }
+  double a[27], coll[27];
+#pragma unroll
+  for (int t = 0; t < 27; ++t) {
+    const int di = t % 3 - 1, dj = t / 3 % 3 - 1, dk = t / 9 - 1;
+    coll[t] = 0.0;
+    a[t] = 0.0;
+    if (t == 13 || (SEVEN && (di != 0) + (dj != 0) + (dk != 0) != 1)) continue;
+    const double v = coupling(F, o, di, dj, dk);
+    sum = __dadd_rn(sum, v);
+    if (!SEVEN) neg = __dadd_rn(neg, fmin(v, 0.0));
+    a[t] = SEVEN ? v : fmax(v, 0.0);
+  }
   const double sigma = __dsub_rn(C, sum);
-  const double ceff = __dsub_rn(__dsub_rn(C, neg), fmin(sigma, 0.0));
-  // collapse the directions the point is coarse-aligned in
-  double coll[27];
-  for (int t = 0; t < 27; ++t) coll[t] = 0.0;
-  double den = ceff;
-  for (int dk = -1; dk <= 1; ++dk)
-    for (int dj = -1; dj <= 1; ++dj)
-      for (int di = -1; di <= 1; ++di) {
-        const int t = (dk + 1) * 9 + (dj + 1) * 3 + (di + 1);
-        if (t == 13) continue;
-        const int pi = fr[0] ? di : 0, pj = fr[1] ? dj : 0, pk = fr[2] ? dk : 0;
-        const int tp = (pk + 1) * 9 + (pj + 1) * 3 + (pi + 1);
-        if (tp == 13)
-          den = __dsub_rn(den, a[t]);
-        else
-          coll[tp] = __dadd_rn(coll[tp], a[t]);
-      }
+  double den = __dsub_rn(__dsub_rn(C, neg), fmin(sigma, 0.0));
+#pragma unroll
+  for (int t = 0; t < 27; ++t) {
+    const int di = t % 3 - 1, dj = t / 3 % 3 - 1, dk = t / 9 - 1;
+    if (t == 13 || (SEVEN && (di != 0) + (dj != 0) + (dk != 0) != 1)) continue;
+    const int tp = ((FZ ? dk : 0) + 1) * 9 + ((FY ? dj : 0) + 1) * 3 + ((FX ? di : 0) + 1);
+    if (tp == 13)
+      den = __dsub_rn(den, a[t]);
+    else
+      coll[tp] = __dadd_rn(coll[tp], a[t]);
+  }
   if (!(den > 0.0)) {
     atomicOr(err, E3_BADDEN);
     return;
   }
+  const Denominator over = denominator(den);
   // weight to each parent: sum over collapsed neighbours of coll times the
-  // neighbour's weight to the same coarse point
+  // neighbour's weight to the same coarse point (1 for the coarse point)
+#pragma unroll
   for (int m = 0; m < NPW3; ++m) {
     const int mc[3] = {m & 1, (m >> 1) & 1, (m >> 2) & 1};
-    if ((mc[0] && !fr[0]) || (mc[1] && !fr[1]) || (mc[2] && !fr[2])) continue;
-    // collapsed couplings live only at offsets that vary in the directions
-    // the point lies between coarse points (integer bounds instead of an
-    // FP64 test per neighbour; the skipped terms are exact zeros)
+    if ((mc[0] && !FX) || (mc[1] && !FY) || (mc[2] && !FZ)) continue;
     double w = 0.0;
-    for (int dk = -fr[2]; dk <= fr[2]; ++dk)
-      for (int dj = -fr[1]; dj <= fr[1]; ++dj)
-        for (int di = -fr[0]; di <= fr[0]; ++di) {
-          const int t = (dk + 1) * 9 + (dj + 1) * 3 + (di + 1);
-          if (t == 13) continue;
-          const int dd[3] = {di, dj, dk};
-          int gslot = 0;
-          bool ok = true;
-          for (int s = 0; s < 3; ++s) {
-            if (!fr[s]) continue;                      // dd[s] == 0 here
-            if (dd[s] == -1) ok = ok && mc[s] == 0;    // neighbour at the lower parent
-            else if (dd[s] == 1) ok = ok && mc[s] == 1;
-            else gslot |= mc[s] << s;                  // still between: same parent
-          }
-          if (!ok) continue;
-          const double wn = F.P[gslot][o + off3(F, di, dj, dk)];
-          w = __dadd_rn(w, __dmul_rn(coll[t], wn));
-        }
-    F.P[m][o] = w / den;
+#pragma unroll
+    for (int t = 0; t < 27; ++t) {
+      const int dd[3] = {t % 3 - 1, t / 3 % 3 - 1, t / 9 - 1};
+      if (t == 13 || (dd[0] && !FX) || (dd[1] && !FY) || (dd[2] && !FZ)) continue;
+      if (SEVEN && (dd[0] != 0) + (dd[1] != 0) + (dd[2] != 0) != 1) continue;
+      int gslot = 0, between = 0;
+      bool ok = true;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (!fr[q]) continue;                      // dd[q] == 0 here
+        if (dd[q] == -1) ok = ok && mc[q] == 0;    // neighbour at the lower parent
+        else if (dd[q] == 1) ok = ok && mc[q] == 1;
+        else { gslot |= mc[q] << q; ++between; }   // still between: same parent
+      }
+      if (!ok) continue;
+      const double wn = between ? F.P[gslot][o + off3(F, dd[0], dd[1], dd[2])] : 1.0;
+      w = __dadd_rn(w, __dmul_rn(coll[t], wn));
+    }
+    F.P[m][o] = divide(w, over);
   }
 }
 
-// One thread per pair of points i = 2t + 1, 2t + 2 of a row (j and k fixed
-// per block): the points of one pass then fill whole warps.
-__global__ void k3_interp_weights(Lev3 F, int pass, int* err) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y + 1, k = blockIdx.z + 1;
-  if (2 * t + 1 <= F.nx) weights_point(F, 2 * t + 1, j, k, pass, err);
-  if (2 * t + 2 <= F.nx) weights_point(F, 2 * t + 2, j, k, pass, err);
+// One thread per cell of fine points (2I + 1..2I + 2, 2J + 1.., 2K + 1..).
+// Pass 1: its coarse point and edge points; 2: its face points (from the
+// edges' weights); 3: its centre.
+template <bool SEVEN, int PASS>
+__global__ void __launch_bounds__(kT) k3_interp_weights(Lev3 F, int* err) {
+  const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + 1, j = 2 * blockIdx.y + 1, k = 2 * blockIdx.z + 1;
+  if (i > F.nx) return;
+  if (PASS == 1) {
+    if (i + 1 <= F.nx && j + 1 <= F.ny && k + 1 <= F.nz) F.P[0][idx3(F, i + 1, j + 1, k + 1)] = 1.0;
+    weights_point<SEVEN, 1, 0, 0>(F, i, j + 1, k + 1, err);
+    weights_point<SEVEN, 0, 1, 0>(F, i + 1, j, k + 1, err);
+    weights_point<SEVEN, 0, 0, 1>(F, i + 1, j + 1, k, err);
+  } else if (PASS == 2) {
+    weights_point<SEVEN, 1, 1, 0>(F, i, j, k + 1, err);
+    weights_point<SEVEN, 1, 0, 1>(F, i, j + 1, k, err);
+    weights_point<SEVEN, 0, 1, 1>(F, i + 1, j, k, err);
+  } else {
+    weights_point<SEVEN, 1, 1, 1>(F, i, j, k, err);
+  }
+}
+
+template <bool SEVEN>
+void launch_weights3(const Lev3& V, int* err, cudaStream_t s) {
+  const int cx = (V.nx + 1) / 2;
+  const dim3 g((cx + kT - 1) / kT, (V.ny + 1) / 2, (V.nz + 1) / 2);
+  k3_interp_weights<SEVEN, 1><<<g, kT, 0, s>>>(V, err);
+  k3_interp_weights<SEVEN, 2><<<g, kT, 0, s>>>(V, err);
+  k3_interp_weights<SEVEN, 3><<<g, kT, 0, s>>>(V, err);
+  count_launch(3);
 }
 
 // ---------------------------------------------------------------------------
@@ -225,71 +296,116 @@ __device__ __forceinline__ int support_slot(int ex, int ey, int ez) {
   return (ex == -1 ? 1 : 0) | ((ey == -1 ? 1 : 0) << 1) | ((ez == -1 ? 1 : 0) << 2);
 }
 
-// One thread per coarse point and stored entry (blockIdx.y = 14 (J - 1) + e):
-// a block's threads share the entry, so their loops run in step.
-__global__ void k3_rap(Lev3 F, Lev3 Cc, int* err) {
-  const int I = blockIdx.x * blockDim.x + threadIdx.x + 1, J = blockIdx.y / 14 + 1, K = blockIdx.z + 1;
-  if (I > Cc.nx) return;
-  const int oc = idx3(Cc, I, J, K);
-  {
-    const int e = blockIdx.y % 14;
-    int di = 0, dj = 0, dk = 0;
-    if (e > 0) {
-      const int m = e - 1;
-      if (m < 9) {
-        dk = -1;
-        dj = m / 3 - 1;
-        di = m % 3 - 1;
-      } else if (m < 12) {
-        dj = -1;
-        di = m - 10;
-      } else {
-        di = -1;
-      }
+// Entry A_c(I, I + (DI, DJ, DK)).  Per direction only the pairs (e, h) with
+// g = e + h - 2 d in -1..1 contribute (fine g in the support of I + d); the
+// loops visit exactly those, in the order of the full 3^6 enumeration, and a
+// 7-point level's h along the axes only (the other terms are exact zeros).
+// With the offsets compile-time constants the plane of every coupling and
+// weight is known (12.3 -> 6.3 ms at 255^3).  Zero weights are not tested for: they add exact
+// zeros, and an FP64 compare costs as much as the multiply-add on this part;
+// the weight of a coarse point is 1.
+__host__ __device__ constexpr int rap_lo(int e, int d) { return -1 - e + 2 * d > -1 ? -1 - e + 2 * d : -1; }
+__host__ __device__ constexpr int rap_hi(int e, int d) { return 1 - e + 2 * d < 1 ? 1 - e + 2 * d : 1; }
+
+template <bool SEVEN, int DI, int DJ, int DK>
+__device__ __forceinline__ double rap3_entry(const Lev3& F, int I, int J, int K) {
+  const int o0 = idx3(F, 2 * I, 2 * J, 2 * K);
+  // fine points beyond an even side do not exist
+  const bool px = 2 * I + 1 <= F.nx, py = 2 * J + 1 <= F.ny, pz = 2 * K + 1 <= F.nz;
+  double val = 0.0;
+#pragma unroll
+  for (int e = 0; e < 27; ++e) {
+    const int ex = e % 3 - 1, ey = e / 3 % 3 - 1, ez = e / 9 - 1;
+    if (rap_lo(ex, DI) > rap_hi(ex, DI) || rap_lo(ey, DJ) > rap_hi(ey, DJ) || rap_lo(ez, DK) > rap_hi(ez, DK))
+      continue;
+    if ((ex == 1 && !px) || (ey == 1 && !py) || (ez == 1 && !pz)) continue;
+    // (7-point: h along one axis at most, so at most one direction with h = 0
+    // excluded; the others' sums are exact zeros)
+    if (SEVEN && (rap_lo(ex, DI) > 0 || rap_hi(ex, DI) < 0) + (rap_lo(ey, DJ) > 0 || rap_hi(ey, DJ) < 0) +
+                         (rap_lo(ez, DK) > 0 || rap_hi(ez, DK) < 0) >
+                     1)
+      continue;
+    const int of = o0 + off3(F, ex, ey, ez);
+    double sum = 0.0;
+#pragma unroll
+    for (int h = 0; h < 27; ++h) {
+      const int hx = h % 3 - 1, hy = h / 3 % 3 - 1, hz = h / 9 - 1;
+      if (hx < rap_lo(ex, DI) || hx > rap_hi(ex, DI) || hy < rap_lo(ey, DJ) || hy > rap_hi(ey, DJ) ||
+          hz < rap_lo(ez, DK) || hz > rap_hi(ez, DK))
+        continue;
+      if (SEVEN && (hx != 0) + (hy != 0) + (hz != 0) > 1) continue;
+      const int gx = ex + hx - 2 * DI, gy = ey + hy - 2 * DJ, gz = ez + hz - 2 * DK;
+      // (beyond the grid coupling and weight are zeros of the ghost layer)
+      const double wg = gx || gy || gz ? F.P[support_slot(gx, gy, gz)][of + off3(F, hx, hy, hz)] : 1.0;
+      const double afg = hx || hy || hz ? -coupling(F, of, hx, hy, hz) : F.C[of];
+      sum = fma(afg, wg, sum);
     }
-    const int I2 = I + di, J2 = J + dj, K2 = K + dk;
-    double val = 0.0;
-    if (I2 >= 1 && J2 >= 1 && K2 >= 1 && I2 <= Cc.nx && J2 <= Cc.ny && K2 <= Cc.nz) {
-      // per direction only the pairs (e, h) with g = e + h - 2d in -1..1 can
-      // contribute (fine g in the support of I + d); the loops visit exactly
-      // those, in the order of the full 3 x 3 x 3 x 3 x 3 x 3 enumeration
-      auto lo = [](int e, int d) { return max(-1, -1 - e + 2 * d); };
-      auto hi = [](int e, int d) { return min(1, 1 - e + 2 * d); };
-      for (int ez = -1; ez <= 1; ++ez)
-        for (int ey = -1; ey <= 1; ++ey)
-          for (int ex = -1; ex <= 1; ++ex) {
-            if (lo(ex, di) > hi(ex, di) || lo(ey, dj) > hi(ey, dj) || lo(ez, dk) > hi(ez, dk))
-              continue;
-            const int fi = 2 * I + ex, fj = 2 * J + ey, fk = 2 * K + ez;
-            if (fi > F.nx || fj > F.ny || fk > F.nz) continue;
-            const int of = idx3(F, fi, fj, fk);
-            // no test for zero weights: they add exact zeros, and an FP64
-            // compare costs as much as the multiply-add on this part
-            const double wf = F.P[support_slot(ex, ey, ez)][of];
-            double s = 0.0;
-            for (int hz = lo(ez, dk); hz <= hi(ez, dk); ++hz)
-              for (int hy = lo(ey, dj); hy <= hi(ey, dj); ++hy)
-                for (int hx = lo(ex, di); hx <= hi(ex, di); ++hx) {
-                  const int gx = ex + hx - 2 * di, gy = ey + hy - 2 * dj, gz = ez + hz - 2 * dk;
-                  const int gi = fi + hx, gj = fj + hy, gk = fk + hz;
-                  if (gi < 1 || gj < 1 || gk < 1 || gi > F.nx || gj > F.ny || gk > F.nz) continue;
-                  const int og = idx3(F, gi, gj, gk);
-                  const double wg = F.P[support_slot(gx, gy, gz)][og];
-                  const double afg =
-                      (hx | hy | hz) == 0 ? F.C[of] : -coupling(F, of, hx, hy, hz);
-                  s = fma(afg, wg, s);
-                }
-            val = fma(wf, s, val);
-          }
-    }
-    if (e == 0) {
-      if (!(val > 0.0) || !(val < INFINITY)) atomicOr(err, E3_NOTSPD);
-      Cc.C[oc] = val;
-      Cc.iC[oc] = 1.0 / val;
-    } else {
-      Cc.A[e - 1][oc] = -val;
-    }
+    val = fma(ex || ey || ez ? F.P[support_slot(ex, ey, ez)][of] : 1.0, sum, val);
   }
+  return val;
+}
+
+// One thread per coarse point and stored entry E.
+template <bool SEVEN, int E>
+__device__ __forceinline__ void rap3_point(const Lev3& F, const Lev3& Cc, int I, int J, int K, int* err) {
+  constexpr int m = E - 1;
+  constexpr int DK = E > 0 && m < 9 ? -1 : 0;
+  constexpr int DJ = E == 0 ? 0 : m < 9 ? m / 3 - 1 : m < 12 ? -1 : 0;
+  constexpr int DI = E == 0 ? 0 : m < 9 ? m % 3 - 1 : m < 12 ? m - 10 : -1;
+  const int oc = idx3(Cc, I, J, K);
+  const int I2 = I + DI, J2 = J + DJ, K2 = K + DK;
+  double val = 0.0;
+  if (I2 >= 1 && J2 >= 1 && K2 >= 1 && I2 <= Cc.nx && J2 <= Cc.ny && K2 <= Cc.nz)
+    val = rap3_entry<SEVEN, DI, DJ, DK>(F, I, J, K);
+  if (E == 0) {
+    if (!(val > 0.0) || !(val < INFINITY)) atomicOr(err, E3_NOTSPD);
+    Cc.C[oc] = val;
+    Cc.iC[oc] = 1.0 / val;
+  } else {
+    Cc.A[E > 0 ? E - 1 : 0][oc] = -val;
+  }
+}
+
+// The entries by kind, a launch each: diagonal, faces, edges, corners.  A
+// thread forms all of a kind for its coarse point, so the rows of weights and
+// couplings they share come from L1, and the unrolled code of a launch stays
+// small: with all 14 entries in one kernel, one per block or one after the
+// other, the warps mostly waited for instructions (255^3: 12.3 ms with general
+// loops, 11.6 and 8.4 in those two forms).
+constexpr int kRapT = 64;
+template <bool SEVEN, int KIND>
+__global__ void __launch_bounds__(kRapT) k3_rap(Lev3 F, Lev3 Cc, int* err) {
+  const int I = blockIdx.x * blockDim.x + threadIdx.x + 1, J = blockIdx.y + 1, K = blockIdx.z + 1;
+  if (I > Cc.nx) return;
+  if constexpr (KIND == 0) {
+    rap3_point<SEVEN, 0>(F, Cc, I, J, K, err);
+  } else if constexpr (KIND == 1) {
+    rap3_point<SEVEN, 5>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 11>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 13>(F, Cc, I, J, K, err);
+  } else if constexpr (KIND == 2) {
+    rap3_point<SEVEN, 2>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 4>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 6>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 8>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 10>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 12>(F, Cc, I, J, K, err);
+  } else {
+    rap3_point<SEVEN, 1>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 3>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 7>(F, Cc, I, J, K, err);
+    rap3_point<SEVEN, 9>(F, Cc, I, J, K, err);
+  }
+}
+
+template <bool SEVEN>
+void launch_rap3(const Lev3& V, const Lev3& Cc, int* err, cudaStream_t s) {
+  const dim3 g((Cc.nx + kRapT - 1) / kRapT, Cc.ny, Cc.nz);
+  k3_rap<SEVEN, 0><<<g, kRapT, 0, s>>>(V, Cc, err);
+  k3_rap<SEVEN, 1><<<g, kRapT, 0, s>>>(V, Cc, err);
+  k3_rap<SEVEN, 2><<<g, kRapT, 0, s>>>(V, Cc, err);
+  k3_rap<SEVEN, 3><<<g, kRapT, 0, s>>>(V, Cc, err);
+  count_launch(4);
 }
 
 // ---------------------------------------------------------------------------
@@ -453,51 +569,73 @@ __global__ void k3_residual(Lev3T<T> L) {
   L.r[o] = fma(-L.C[o], L.x[o], L.b[o]) + nb_sum<SEVEN>(L, L.x, o);
 }
 
-// b_c(I) = sum over the fine support of I of P(f, I) r(f); x_c = 0.
+// b_c(I) = sum over the fine support of I of P(f, I) r(f); x_c = 0.  Unrolled,
+// so that the planes are constants and all loads are in flight (beyond an
+// even side weight and residual are zeros of the ghost layer).
 template <typename T>
-__global__ void k3_restrict(Lev3T<T> F, Lev3T<T> Cc) {
+__global__ void __launch_bounds__(kT) k3_restrict(Lev3T<T> F, Lev3T<T> Cc) {
   griddep_wait();
   const int I = blockIdx.x * blockDim.x + threadIdx.x + 1, J = blockIdx.y + 1, K = blockIdx.z + 1;
   if (I > Cc.nx) return;
+  const int o0 = idx3(F, 2 * I, 2 * J, 2 * K);
   T s = T(0);
-  for (int ez = -1; ez <= 1; ++ez)
-    for (int ey = -1; ey <= 1; ++ey)
-      for (int ex = -1; ex <= 1; ++ex) {
-        const int fi = 2 * I + ex, fj = 2 * J + ey, fk = 2 * K + ez;
-        if (fi > F.nx || fj > F.ny || fk > F.nz) continue;
-        const int of = idx3(F, fi, fj, fk);
-        s = fma(F.P[support_slot(ex, ey, ez)][of], F.r[of], s);
-      }
+#pragma unroll
+  for (int e = 0; e < 27; ++e) {
+    const int ex = e % 3 - 1, ey = e / 3 % 3 - 1, ez = e / 9 - 1;
+    const int of = o0 + off3(F, ex, ey, ez);
+    s = fma(F.P[support_slot(ex, ey, ez)][of], F.r[of], s);
+  }
   const int oc = idx3(Cc, I, J, K);
   Cc.b[oc] = s;
   Cc.x[oc] = T(0);
 }
 
 // x(f) += sum over f's parents of P(f, I) x_c(I).  A point has 1, 2, 4 or 8
-// parents by the parities of i, j, k; each thread takes one point of each
-// parity of i in turn (j and k are fixed per block), so the lanes of a warp
-// always follow the same parents.
-template <typename T>
+// parents by the parities of i, j, k, compile-time constants here; each
+// thread takes one point of each parity of i in turn (j and k are fixed per
+// block), so the lanes of a warp always follow the same parents.
+template <int OX, int OY, int OZ, typename T>
 __device__ __forceinline__ void interp_point(const Lev3T<T>& F, const Lev3T<T>& Cc, int i, int j, int k) {
   const int o = idx3(F, i, j, k);
+  const int oc = idx3(Cc, i >> 1, j >> 1, k >> 1);   // odd: (i - 1) / 2, even: i / 2
   T s = T(0);
+#pragma unroll
   for (int m = 0; m < NPW3; ++m) {
     const int cx = m & 1, cy = (m >> 1) & 1, cz = m >> 2;
-    if ((cx && !(i & 1)) || (cy && !(j & 1)) || (cz && !(k & 1))) continue;
-    const int I = (i & 1) ? (i - 1) / 2 + cx : i / 2;
-    const int J = (j & 1) ? (j - 1) / 2 + cy : j / 2;
-    const int K = (k & 1) ? (k - 1) / 2 + cz : k / 2;
-    s = fma(F.P[m][o], Cc.x[idx3(Cc, I, J, K)], s);
+    if ((cx && !OX) || (cy && !OY) || (cz && !OZ)) continue;
+    s = fma(F.P[m][o], Cc.x[oc + off3(Cc, cx, cy, cz)], s);
   }
   F.x[o] += s;
 }
 
+// kept: every point; or (a 7-point level whose next operation is a sweep in
+// reverse colour order) only those of even i + j + k (0-based), since the
+// sweep's first colour replaces the others without reading them: half of the
+// points, and 14 of 27 weights.
+template <int OY, int OZ, typename T>
+__device__ __forceinline__ void interp_row(const Lev3T<T>& F, const Lev3T<T>& Cc, int t, int j, int k, int half) {
+  // 1-based: i + j + k odd
+  constexpr bool want_odd = ((OY + OZ) & 1) == 0;
+  if (2 * t + 1 <= F.nx && (!half || want_odd)) interp_point<1, OY, OZ>(F, Cc, 2 * t + 1, j, k);
+  if (2 * t + 2 <= F.nx && (!half || !want_odd)) interp_point<0, OY, OZ>(F, Cc, 2 * t + 2, j, k);
+}
+
 template <typename T>
-__global__ void k3_interp(Lev3T<T> F, Lev3T<T> Cc) {
+__global__ void __launch_bounds__(kT) k3_interp(Lev3T<T> F, Lev3T<T> Cc, int half) {
   griddep_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y + 1, k = blockIdx.z + 1;
-  if (2 * t + 1 <= F.nx) interp_point(F, Cc, 2 * t + 1, j, k);
-  if (2 * t + 2 <= F.nx) interp_point(F, Cc, 2 * t + 2, j, k);
+  if (2 * t + 1 > F.nx) return;
+  if (j & 1) {
+    if (k & 1)
+      interp_row<1, 1>(F, Cc, t, j, k, half);
+    else
+      interp_row<1, 0>(F, Cc, t, j, k, half);
+  } else {
+    if (k & 1)
+      interp_row<0, 1>(F, Cc, t, j, k, half);
+    else
+      interp_row<0, 0>(F, Cc, t, j, k, half);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -823,31 +961,51 @@ __global__ void k3_coarse_factor(Lev3 L0, double* __restrict__ lo, double* __res
   }
 }
 
+// The inverse, one column per block (bmg_setup.cu's k_coarse_inverse on the
+// same kind of factor; entry (r, c) at c * n + r).
+__global__ void __launch_bounds__(128) k3_coarse_inverse(const double* __restrict__ lo,
+                                                         const double* __restrict__ idiag, int n,
+                                                         double* __restrict__ inv) {
+  __shared__ double v[BMG_MAX_COARSEST], y[BMG_MAX_COARSEST];
+  const int c = blockIdx.x;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    v[i] = i == c ? 1.0 : 0.0;
+    y[i] = 0.0;
+  }
+  for (int j = c; j < n; ++j) {
+    __syncthreads();
+    const double yj = v[j] * idiag[j];
+    if (threadIdx.x == 0) y[j] = yj;
+    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) v[i] = fma(-lo[size_t(i) * n + j], yj, v[i]);
+  }
+  for (int j = n - 1; j >= 0; --j) {
+    __syncthreads();
+    const double xj = y[j] * idiag[j];
+    if (threadIdx.x == 0) inv[size_t(c) * n + j] = xj;
+    for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-lo[size_t(j) * n + i], xj, y[i]);
+  }
+}
+
+// x_0 = A_0^{-1} b_0 with the stored inverse: four lanes per unknown, one of
+// four interleaved partial sums each.  Substitution with the factor took 2 n
+// dependent steps with two barriers each (27 unknowns 20.6 us, 60 37 us).
+constexpr int kSolveT = 256;
 template <typename T>
-__global__ void k3_coarse_solve(Lev3T<T> L0, const double* __restrict__ lo,
-                                const double* __restrict__ idiag) {
+__global__ void __launch_bounds__(kSolveT) k3_coarse_solve(Lev3T<T> L0, const double* __restrict__ inv) {
   griddep_wait();
   __shared__ double v[BMG_MAX_COARSEST];
   const int nx = L0.nx, ny = L0.ny, n = nx * ny * L0.nz;
-  for (int r = threadIdx.x; r < n; r += blockDim.x)
-    v[r] = double(L0.b[idx3(L0, r % nx + 1, (r / nx) % ny + 1, r / (nx * ny) + 1)]);
+  auto at = [&](int r) { return idx3(L0, r % nx + 1, (r / nx) % ny + 1, r / (nx * ny) + 1); };
+  for (int r = threadIdx.x; r < n; r += kSolveT) v[r] = double(L0.b[at(r)]);
   __syncthreads();
-  for (int j = 0; j < n; ++j) {
-    const double y = v[j] * idiag[j];
-    __syncthreads();
-    if (threadIdx.x == 0) v[j] = y;
-    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) v[i] = fma(-lo[size_t(i) * n + j], y, v[i]);
-    __syncthreads();
+  for (int e = threadIdx.x; e < (4 * n + 31) / 32 * 32; e += kSolveT) {   // (whole warps)
+    const int r = e >> 2, q = r < n ? r : 0;
+    double x = bmg::inverse_part(
+        n, e & 3, 4, [&](int c) { return inv[size_t(c) * n + q]; }, [&](int c) { return v[c]; });
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    if ((e & 3) == 0 && r < n) L0.x[at(r)] = T(x);
   }
-  for (int j = n - 1; j >= 0; --j) {
-    const double xj = v[j] * idiag[j];
-    __syncthreads();
-    if (threadIdx.x == 0) v[j] = xj;
-    for (int i = threadIdx.x; i < j; i += blockDim.x) v[i] = fma(-lo[size_t(j) * n + i], xj, v[i]);
-    __syncthreads();
-  }
-  for (int r = threadIdx.x; r < n; r += blockDim.x)
-    L0.x[idx3(L0, r % nx + 1, (r / nx) % ny + 1, r / (nx * ny) + 1)] = T(v[r]);
 }
 
 // dense (nz, ny, nx) <-> plane interior
@@ -881,7 +1039,7 @@ struct bmg3_hierarchy {
   cudaGraph_t pcg_graph[2] = {nullptr, nullptr};          // first iteration, later ones
   cudaGraphExec_t pcg_exec[2] = {nullptr, nullptr};
   void* arena = nullptr;
-  double *chol = nullptr, *chol_idiag = nullptr, *partials = nullptr;
+  double *chol = nullptr, *chol_idiag = nullptr, *cinv = nullptr, *partials = nullptr;
   Scal3* sc = nullptr;
   Scal3* sc_host = nullptr;
   int* err = nullptr;
@@ -991,11 +1149,12 @@ void enqueue_vcycle3(bmg3_hierarchy* h, std::vector<Lev3T<T>>& lv, cudaStream_t 
     bmg::launch_pdl(k3_restrict<T>, dim3(grid_pts(lv[l - 1])), dim3(kT), 0, s, V, lv[l - 1]);
     count_launch(2);
   }
-  bmg::launch_pdl(k3_coarse_solve<T>, dim3(1), dim3(256), 0, s, lv[0], h->chol, h->chol_idiag);
+  bmg::launch_pdl(k3_coarse_solve<T>, dim3(1), dim3(kSolveT), 0, s, lv[0], (const double*)h->cinv);
   count_launch();
   for (int l = 1; l < L; ++l) {
     bmg::NvtxRange r("interp_leg", l);
-    bmg::launch_pdl(k3_interp<T>, dim3(cdiv((lv[l].nx + 1) / 2, kT), lv[l].ny, lv[l].nz), dim3(kT), 0, s, lv[l], lv[l - 1]);
+    bmg::launch_pdl(k3_interp<T>, dim3(cdiv((lv[l].nx + 1) / 2, kT), lv[l].ny, lv[l].nz), dim3(kT), 0, s, lv[l], lv[l - 1],
+                    int(l == L - 1 && h->opt.nu2 > 0));
     count_launch();
     sweep(l, h->opt.nu2, true, false);
   }
@@ -1232,6 +1391,10 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     return o;
   };
   std::vector<size_t> offs;
+  // planes of a level's couplings: the 7-point finest level has three, and one
+  // plane of zeros stands for the ten others
+  auto acount = [&](int l) { return l == L - 1 && L > 1 ? 4 : NA; };
+  auto aplane = [&](int l, int m) { return acount(l) == NA ? m : m == 4 ? 0 : m == 10 ? 1 : m == 12 ? 2 : 3; };
   for (int l = 0; l < L; ++l) {
     Lev3& V = h->lv[l];
     const int src = L - 1 - l;
@@ -1241,7 +1404,7 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     V.px = (V.nx + 2 + 15) / 16 * 16;
     V.py = V.ny + 2;
     const size_t pb = size_t(V.nz + 2) * V.py * V.px * sizeof(double);
-    const int nplanes = 2 + NA + 3 + (l >= 1 ? NPW3 : 0);
+    const int nplanes = 2 + acount(l) + 3 + (l >= 1 ? NPW3 : 0);
     for (int p = 0; p < nplanes; ++p) offs.push_back(reserve(pb));
   }
   h->refine = opt.precision == BMG_FP32_REFINE;
@@ -1257,7 +1420,7 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
       W.px = (V.nx + 2 + 31) / 32 * 32;
       W.py = V.ny + 2;
       const size_t pb = size_t(W.nz + 2) * W.py * W.px * sizeof(float);
-      const int nplanes = 2 + NA + 3 + (l >= 1 ? NPW3 : 0);
+      const int nplanes = 2 + acount(l) + 3 + (l >= 1 ? NPW3 : 0);
       for (int p = 0; p < nplanes; ++p) offs32.push_back(reserve(pb));
     }
   }
@@ -1280,6 +1443,7 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
   }
   const size_t o_chol = reserve(sizeof(double) * size_t(h->n0) * h->n0);
   const size_t o_idiag = reserve(sizeof(double) * h->n0);
+  const size_t o_cinv = reserve(sizeof(double) * size_t(h->n0) * h->n0);
   const size_t o_part = reserve(sizeof(double) * kNormBlocks);
   const size_t o_sc = reserve(sizeof(Scal3));
   if (cudaMalloc(&h->arena, total) != cudaSuccess) {
@@ -1298,7 +1462,11 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     auto next = [&]() { return reinterpret_cast<double*>(base + offs[pi++]); };
     V.C = next();
     V.iC = next();
-    for (int m = 0; m < NA; ++m) V.A[m] = next();
+    {
+      double* a[NA];
+      for (int m = 0; m < acount(l); ++m) a[m] = next();
+      for (int m = 0; m < NA; ++m) V.A[m] = a[aplane(l, m)];
+    }
     V.x = next();
     V.b = next();
     V.r = next();
@@ -1310,7 +1478,11 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     auto next = [&]() { return reinterpret_cast<float*>(base + offs32[qi++]); };
     W.C = next();
     W.iC = next();
-    for (int m = 0; m < NA; ++m) W.A[m] = next();
+    {
+      float* a[NA];
+      for (int m = 0; m < acount(l); ++m) a[m] = next();
+      for (int m = 0; m < NA; ++m) W.A[m] = a[aplane(l, m)];
+    }
     W.x = next();
     W.b = next();
     W.r = next();
@@ -1327,6 +1499,7 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
   if (h->fused) h->x2 = reinterpret_cast<double*>(base + o_x2);
   h->chol = reinterpret_cast<double*>(base + o_chol);
   h->chol_idiag = reinterpret_cast<double*>(base + o_idiag);
+  h->cinv = reinterpret_cast<double*>(base + o_cinv);
   h->partials = reinterpret_cast<double*>(base + o_part);
   h->sc = reinterpret_cast<Scal3*>(base + o_sc);
   h->err = &h->sc->err;
@@ -1335,22 +1508,22 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     return BMG_ECUDA;
   }
   const Lev3& F = h->lv[L - 1];
-  k3_assemble<<<dim3(cdiv(F.nx, kT), F.ny, F.nz), kT, 0, s>>>(k, F, h->err);
+  k3_assemble<<<dim3(cdiv(F.nx, kA3X), cdiv(F.ny, kA3Y), cdiv(F.nz, kA3Z)), dim3(kA3X, kA3Y), 0, s>>>(k, F, h->err);
   count_launch();
   for (int l = L - 1; l >= 1; --l) {
     const Lev3& V = h->lv[l];
-    for (int pass = 0; pass <= 3; ++pass) {
-      k3_interp_weights<<<dim3(cdiv((V.nx + 1) / 2, kT), V.ny, V.nz), kT, 0, s>>>(V, pass, h->err);
-      count_launch();
+    const Lev3& Cc = h->lv[l - 1];
+    if (l == L - 1) {
+      launch_weights3<true>(V, h->err, s);
+      launch_rap3<true>(V, Cc, h->err, s);
+    } else {
+      launch_weights3<false>(V, h->err, s);
+      launch_rap3<false>(V, Cc, h->err, s);
     }
-    {
-      const Lev3& Cc = h->lv[l - 1];
-      k3_rap<<<dim3(cdiv(Cc.nx, kT), 14 * Cc.ny, Cc.nz), kT, 0, s>>>(V, Cc, h->err);
-    }
-    count_launch();
   }
   k3_coarse_factor<<<1, 512, 0, s>>>(h->lv[0], h->chol, h->chol_idiag, h->err);
-  count_launch();
+  k3_coarse_inverse<<<h->n0, 128, 0, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv);
+  count_launch(2);
   for (int l = 0; l < int(h->lv32.size()); ++l) {
     const Lev3& V = h->lv[l];
     k3_downcast<<<dim3(cdiv(V.nx + 2, kT), V.ny + 2, V.nz + 2), kT, 0, s>>>(V, h->lv32[l], l >= 1 ? 1 : 0);
