@@ -1077,8 +1077,8 @@ void free3(bmg3_hierarchy* h) {
     if (h->pcg_exec[g]) cudaGraphExecDestroy(h->pcg_exec[g]);
     if (h->pcg_graph[g]) cudaGraphDestroy(h->pcg_graph[g]);
   }
-  if (h->arena) cudaFree(h->arena);
-  if (h->sc_host) cudaFreeHost(h->sc_host);
+  bmg::pool_free(h->arena);   // (waits for the device)
+  bmg::pinned_slot_free(h->sc_host);
   delete h;
 }
 
@@ -1446,12 +1446,13 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
   const size_t o_cinv = reserve(sizeof(double) * size_t(h->n0) * h->n0);
   const size_t o_part = reserve(sizeof(double) * kNormBlocks);
   const size_t o_sc = reserve(sizeof(Scal3));
-  if (cudaMalloc(&h->arena, total) != cudaSuccess) {
-    cudaGetLastError();
+  h->arena = bmg::pool_alloc(total);
+  if (!h->arena) {
     delete h;
     return BMG_ENOMEM;
   }
-  if (cudaMallocHost(&h->sc_host, sizeof(Scal3)) != cudaSuccess) {
+  h->sc_host = static_cast<Scal3*>(bmg::pinned_slot(sizeof(Scal3)));
+  if (!h->sc_host) {
     free3(h);
     return BMG_ENOMEM;
   }

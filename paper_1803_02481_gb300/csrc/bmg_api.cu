@@ -177,8 +177,8 @@ void free_hierarchy(Hierarchy* h) {
   if (!h) return;
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
   if (h->graph) cudaGraphDestroy(h->graph);
-  if (h->arena) cudaFree(h->arena);
-  if (h->sc_host) cudaFreeHost(h->sc_host);
+  pool_free(h->arena);   // (waits for the device)
+  pinned_slot_free(h->sc_host);
   for (auto* m : h->maps64) delete m;
   for (auto* m : h->maps32) delete m;
   delete h;
@@ -300,15 +300,16 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
     }
     if (pass == 0) {
       h->arena_bytes = cv.off;
-      if (cudaMalloc(&h->arena, h->arena_bytes) != cudaSuccess) {
-        cudaGetLastError();
+      h->arena = pool_alloc(h->arena_bytes);
+      if (!h->arena) {
         delete h;
         return BMG_ENOMEM;
       }
       cv.base = static_cast<char*>(h->arena);
     }
   }
-  if (cudaMallocHost(&h->sc_host, sizeof(Scalars)) != cudaSuccess) {
+  h->sc_host = static_cast<Scalars*>(pinned_slot(sizeof(Scalars)));
+  if (!h->sc_host) {
     free_hierarchy(h);
     return BMG_ENOMEM;
   }
@@ -884,11 +885,8 @@ int bmg_solve_host(const double* k_host, const double* b_host, double* x_host, i
   if (!bmg::valid_side(nx) || !bmg::valid_side(ny)) return BMG_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const size_t bytes = sizeof(double) * size_t(nx) * ny;
-  double* buf = nullptr;
-  if (cudaMalloc(&buf, 3 * bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return BMG_ENOMEM;
-  }
+  double* buf = static_cast<double*>(bmg::pool_alloc(3 * bytes));
+  if (!buf) return BMG_ENOMEM;
   double *k = buf, *b = buf + size_t(nx) * ny, *x = buf + 2 * size_t(nx) * ny;
   int rc = BMG_OK;
   bmg_hierarchy* h = nullptr;
@@ -910,7 +908,7 @@ int bmg_solve_host(const double* k_host, const double* b_host, double* x_host, i
   }
   if (info) info->setup_ms = setup_ms;
   bmg_destroy(h);
-  cudaFree(buf);
+  bmg::pool_free(buf);
   return rc;
 }
 

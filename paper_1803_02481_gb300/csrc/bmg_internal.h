@@ -453,6 +453,14 @@ struct NvtxRange {
 void prof_begin(int which, cudaStream_t s);
 void prof_end(int which, cudaStream_t s);
 
+// Device memory kept between hierarchies, and pinned slots of up to 256 bytes
+// (bmg_pool.cu); null when there is none to be had.  pool_free and
+// pinned_slot_free take what these returned, or null.
+void* pool_alloc(size_t bytes);
+void pool_free(void* p);
+void* pinned_slot(size_t bytes);
+void pinned_slot_free(void* p);
+
 // Hierarchy lifetime (bmg_api.cu).
 int setup_impl(const double* k, int nx, int ny, const bmg_options* opt, cudaStream_t s,
                Hierarchy** out);
