@@ -180,6 +180,24 @@ __device__ __forceinline__ void load_cell(Cell<T>& q, const Lv& L, int t) {
   }
 }
 
+// The cells' coefficients kept over the whole sub-cycle: every level has
+// threads of its own (`own`: this thread's level is the one at work), so they
+// are loaded once, before the kernel waits for its predecessor, instead of in
+// each leg of each level (500 ns a time).  Colour phase c.
+template <typename T, bool NINE>
+__device__ __forceinline__ void colour_own(const Cell<T>& q, const Lv& L, bool own, int c, unsigned mask) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (NINE ? k != c : ((k >> 1) ^ (k & 1)) != c) continue;
+    if (own && q.in[k]) {
+      const int d = q.o + (k >> 1) * L.sp + (k & 1);
+      const int o = L.x + d;
+      sh<T>(o) = gauss_seidel<T, NINE>(q.c[k], sh<T>(L.b + d), o, L.sp, mask);
+    }
+  }
+  __syncthreads();
+}
+
 // Colour phase c (0 .. 3, or red 0 and black 1) on the cells of the block:
 // `held` is the thread's own cell (of the first kNT); levels with more cells
 // load the others' coefficients in the phase.
@@ -207,35 +225,48 @@ __device__ __forceinline__ void colour(const Cell<T>& held, const Lv& L, int nce
   __syncthreads();
 }
 
-template <typename T, bool NINE, bool REVERSE>
-__device__ __forceinline__ void sweep(const Cell<T>& held, const Lv& L, int ncell) {
+template <typename T, bool NINE, bool REVERSE, bool OWN>
+__device__ __forceinline__ void sweep(const Cell<T>& held, const Lv& L, bool own, int ncell) {
   constexpr int NC = NINE ? 4 : 2;
 #pragma unroll
-  for (int k = 0; k < NC; ++k)
-    colour<T, NINE>(held, L, ncell, REVERSE ? NC - 1 - k : k, NINE ? 0xFFu : 0x0Fu);
+  for (int k = 0; k < NC; ++k) {
+    const int c = REVERSE ? NC - 1 - k : k;
+    if (OWN)
+      colour_own<T, NINE>(held, L, own, c, NINE ? 0xFFu : 0x0Fu);
+    else
+      colour<T, NINE>(held, L, ncell, c, NINE ? 0xFFu : 0x0Fu);
+  }
 }
 
 // Pre-smoothing, residual and restriction of a level.  Enters and leaves
 // with every thread's writes visible.
-template <typename T, bool NINE>
-__device__ __forceinline__ void down(const Lv& L, const Lv& C, int nu1, bool zero) {
+template <typename T, bool NINE, bool OWN>
+__device__ __forceinline__ void down(const Lv& L, const Lv& C, Cell<T>& held, bool own, int nu1, bool zero) {
   const int ncell = ((L.nx + 1) >> 1) * ((L.ny + 1) >> 1);
-  Cell<T> held{};
-  if (int(threadIdx.x) < ncell) load_cell<T, NINE>(held, L, threadIdx.x);
+  if (!OWN) {
+    held = Cell<T>{};
+    if (int(threadIdx.x) < ncell) load_cell<T, NINE>(held, L, threadIdx.x);
+  }
   int s = 0;
   if (zero && nu1 > 0) {
     constexpr int NC = NINE ? 4 : 2;
 #pragma unroll
-    for (int k = 0; k < NC; ++k) colour<T, NINE>(held, L, ncell, k, zero_start_mask(NINE, k));
+    for (int k = 0; k < NC; ++k) {
+      if (OWN)
+        colour_own<T, NINE>(held, L, own, k, zero_start_mask(NINE, k));
+      else
+        colour<T, NINE>(held, L, ncell, k, zero_start_mask(NINE, k));
+    }
     s = 1;
   }
-  for (; s < nu1; ++s) sweep<T, NINE, false>(held, L, ncell);
-  if (4 * ncell <= kNT) {
+  for (; s < nu1; ++s) sweep<T, NINE, false, OWN>(held, L, own, ncell);
+  if (OWN || 4 * ncell <= kNT) {
     // one point per thread, over all warps, instead of four in a few
-    const int k = int(threadIdx.x) / (kNT / 4), t = int(threadIdx.x) % (kNT / 4);
+    const int k = int(threadIdx.x) / (kNT / 4);
     const int hx = (L.nx + 1) >> 1;
-    const int jj = t / hx, ii = t - jj * hx;
-    if (t < ncell && 2 * ii + (k & 1) < L.nx && 2 * jj + (k >> 1) < L.ny) {
+    for (int t = int(threadIdx.x) % (kNT / 4); t < ncell; t += kNT / 4) {
+      const int jj = t / hx, ii = t - jj * hx;
+      if (2 * ii + (k & 1) >= L.nx || 2 * jj + (k >> 1) >= L.ny) continue;
       const int o = (1 + 2 * jj + (k >> 1)) * L.sp + 1 + 2 * ii + (k & 1);
       Coef<T> cf;
       load_coef<T, NINE>(cf, L, o);
@@ -249,7 +280,7 @@ __device__ __forceinline__ void down(const Lv& L, const Lv& C, int nu1, bool zer
         sh<T>(L.r + held.o + d) = residual<T, NINE>(held.c[k], held.b[k], L.x + held.o + d, L.sp);
     }
   }
-  for (int t = int(threadIdx.x) + kNT; t < ncell; t += kNT) {
+  for (int t = int(threadIdx.x) + kNT; !OWN && t < ncell; t += kNT) {
     const int hx = (L.nx + 1) >> 1;
     const int jj = t / hx, ii = t - jj * hx;
 #pragma unroll 1
@@ -347,14 +378,16 @@ __device__ __forceinline__ void interpolate(const Lv& L, const Lv& C, bool add_r
   }
 }
 
-template <typename T, bool NINE>
-__device__ __forceinline__ void up(const Lv& L, const Lv& C, int nu2, bool add_rc) {
+template <typename T, bool NINE, bool OWN>
+__device__ __forceinline__ void up(const Lv& L, const Lv& C, Cell<T>& held, bool own, int nu2, bool add_rc) {
   const int ncell = ((L.nx + 1) >> 1) * ((L.ny + 1) >> 1);
-  Cell<T> held{};
-  if (nu2 > 0 && int(threadIdx.x) < ncell) load_cell<T, NINE>(held, L, threadIdx.x);
+  if (!OWN) {
+    held = Cell<T>{};
+    if (nu2 > 0 && int(threadIdx.x) < ncell) load_cell<T, NINE>(held, L, threadIdx.x);
+  }
   interpolate<T>(L, C, add_rc, NINE && nu2 > 0);
   __syncthreads();
-  for (int s = 0; s < nu2; ++s) sweep<T, NINE, true>(held, L, ncell);
+  for (int s = 0; s < nu2; ++s) sweep<T, NINE, true, OWN>(held, L, own, ncell);
 }
 
 // x_0 = A_0^{-1} b_0 with the stored inverse (the sums of blk_coarse_solve):
@@ -382,7 +415,7 @@ __device__ __forceinline__ void solve0(const SmArgs<T>& a, const Lv& L) {
   }
 }
 
-template <typename T>
+template <typename T, bool OWN>
 __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   using namespace tma_detail;
   __shared__ __align__(8) uint64_t bar;
@@ -401,7 +434,28 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   // restriction of an even side reads
   for (int e = a.voff[0] + threadIdx.x; e < a.end; e += kNT) sh<T>(e) = T(0);
   __syncthreads();
+  Cell<T> held{};
+  int mine = 0;                          // OWN: this thread's level
+  bool ok = true;
+  if (OWN) {
+    // levels top .. 1 take warps in turn
+    ok = mbar_wait_bounded(&bar, 0);
+    int first = 0;
+    for (int l = top; ok && l >= 1; --l) {
+      const Lv L(a, l);
+      const int n = ((L.nx + 1) >> 1) * ((L.ny + 1) >> 1), t = int(threadIdx.x) - first;
+      if (t >= 0 && t < n) {
+        mine = l;
+        if (l < top || a.top_nine)
+          load_cell<T, true>(held, L, t);
+        else
+          load_cell<T, false>(held, L, t);
+      }
+      first += (n + 31) & ~31;
+    }
+  }
   griddep_wait();
+  griddep_launch();
   {
     const Lv L(a, top);
     const int w = L.nx;
@@ -411,7 +465,7 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
       if (!a.top_zero) sh<T>(L.x + j * L.sp + i) = a.x[j * a.pitch + i];
     }
   }
-  const bool ok = mbar_wait_bounded(&bar, 0);
+  if (!OWN) ok = mbar_wait_bounded(&bar, 0);
   if (!__syncthreads_and(ok)) {
     if (threadIdx.x == 0) {
       atomicOr(a.err, DEV_TIMEOUT);
@@ -424,9 +478,9 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
     const Lv L(a, l), C(a, l - 1);
     const bool zero = l < top || a.top_zero;
     if (l < top || a.top_nine)
-      down<T, true>(L, C, a.nu1, zero);
+      down<T, true, OWN>(L, C, held, mine == l, a.nu1, zero);
     else
-      down<T, false>(L, C, a.nu1, zero);
+      down<T, false, OWN>(L, C, held, mine == l, a.nu1, zero);
   }
   {
     const Lv L(a, 0);
@@ -439,9 +493,9 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   for (int l = 1; l <= top; ++l) {
     const Lv L(a, l), C(a, l - 1);
     if (l < top || a.top_nine)
-      up<T, true>(L, C, a.nu2, a.add_rc != 0);
+      up<T, true, OWN>(L, C, held, mine == l, a.nu2, a.add_rc != 0);
     else
-      up<T, false>(L, C, a.nu2, a.add_rc != 0);
+      up<T, false, OWN>(L, C, held, mine == l, a.nu2, a.add_rc != 0);
     if (a.nu2 == 0) __syncthreads();
   }
   const Lv L(a, top);
@@ -451,9 +505,9 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   }
 }
 
-template <typename T>
+template <typename T, bool OWN>
 __global__ void __launch_bounds__(kNT, 1) k_coarse_smem(const __grid_constant__ SmArgs<T> a) {
-  coarse_smem_body<T>(a);
+  coarse_smem_body<T, OWN>(a);
 }
 
 // One problem per block; a problem that has stopped is left alone.  (`go` was
@@ -468,7 +522,7 @@ __global__ void __launch_bounds__(kNT, 1) k_coarse_smem_batch(const SmArgs<float
   const int* src = reinterpret_cast<const int*>(args + blockIdx.x);
   for (int e = threadIdx.x; e < int(sizeof(a) / sizeof(int)); e += kNT) reinterpret_cast<int*>(&a)[e] = src[e];
   __syncthreads();
-  coarse_smem_body<float>(a);
+  coarse_smem_body<float, false>(a);
 }
 
 // The image: blockIdx.x walks the constant planes of the levels (NK9 + NPW
@@ -549,7 +603,8 @@ size_t layout(const Hierarchy* h, int thr, SmArgs<T>& a) {
 
 template <typename T>
 void prepare() {
-  static const bool done = use_shared(k_coarse_smem<T>, kCoarseImageMax);
+  static const bool done =
+      use_shared(k_coarse_smem<T, true>, kCoarseImageMax) && use_shared(k_coarse_smem<T, false>, kCoarseImageMax);
   (void)done;
 }
 
@@ -597,7 +652,13 @@ void launch_coarse_smem(Hierarchy* h, const LevelV<T>& top, int thr, bool top_ze
   a.x = top.x;
   a.b = top.b;
   a.pitch = top.pitch;
-  launch_pdl(k_coarse_smem<T>, dim3(1), dim3(kNT), bytes, s, a);
+  // threads of its own for every level, where the block has as many
+  int threads = 0;
+  for (int l = 1; l < thr; ++l) threads += (((a.nx[l] + 1) / 2) * ((a.ny[l] + 1) / 2) + 31) / 32 * 32;
+  if (threads <= kNT)
+    launch_pdl(k_coarse_smem<T, true>, dim3(1), dim3(kNT), bytes, s, a);
+  else
+    launch_pdl(k_coarse_smem<T, false>, dim3(1), dim3(kNT), bytes, s, a);
 }
 
 size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned char>& out) {
