@@ -5,7 +5,9 @@
 // redistribution of Section 2.2 / Algorithm 2), residual norms with the
 // device-side stop test, and the FP64 kernels of iterative refinement.
 #include "bmg_coarse.cuh"
+#include "bmg_krylov.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 
@@ -287,68 +289,89 @@ __global__ void __launch_bounds__(kNormThreads) k_norm_final(const double* parti
 }
 
 // FP32_REFINE: r = b - A x in FP64 on the finest level (partials of ||r||^2)
-// and the FP32 right-hand side r / ||r_prev|| of the next FP32 V-cycle; the
-// FP32 fine iterate is reset to zero.  The scaling to the FP32 right-hand
-// side is done in FP32 (float(r) * float(1/||r_prev||), one more FP32
-// rounding than an FP64 product, and one FP64 instruction less per point)
-// while 1/||r_prev|| lies in (1e-28, 1e28), where every entry that matters
-// for the FP32 correction is a normal FP32 number; outside, in FP64.  The
-// choice is uniform over the launch, so each loop is branch-free.
-template <bool NINE, bool SCALE32>
-__device__ __forceinline__ double refine_rows(const LevelV<double>& L, const LevelV<float>& F,
-                                              double inv) {
+// and the FP32 right-hand side r / ||r_prev|| of the next FP32 V-cycle
+// (zero_x: and a zero FP32 fine iterate, for cycles that read it).  The
+// scaling to the FP32 right-hand side is done in FP32 (float(r) *
+// float(1/||r_prev||), one more FP32 rounding than an FP64 product, and one
+// FP64 instruction less per point) while 1/||r_prev|| lies in (1e-28, 1e28),
+// where every entry that matters for the FP32 correction is a normal FP32
+// number; outside, in FP64.  Bound by the FP64 pipe: six operations a point,
+// the conversion in integer arithmetic (with it on the pipe too, and rows
+// dealt whole, 830 us at 8191^2; now 682, the pipe's floor is 677).
+template <bool SCALE32>
+__device__ __forceinline__ double refine_pairs(const LevelV<double>& L, const LevelV<float>& F,
+                                               double inv, bool zero_x) {
   const float inv32 = float(inv);
-  const double* __restrict__ x = L.x;
-  const double* __restrict__ b = L.b;
-  float* __restrict__ fb = F.b;
-  float* __restrict__ fx = F.x;
+  const int pitch = L.pitch, fpitch = F.pitch;
+  const double* const x = L.x;
+  const double* const b = L.b;
+  float *const fb = F.b, *const fx = F.x;
+  struct V {
+    ResidPair r;
+    double2 b;
+  };
   double acc = 0.0;
-  for (int j = blockIdx.x + 1; j <= L.ny; j += gridDim.x) {
-    for (int i = threadIdx.x + 1; i <= L.nx; i += blockDim.x) {
-      const int o = j * L.pitch + i;
-      const double r = resid_value<double, NINE>(L, x, b[o], o);
-      acc = fma(r, r, acc);
-      const int of = j * F.pitch + i;
-      fb[of] = SCALE32 ? float(r) * inv32 : float(r * inv);
-      fx[of] = 0.0f;
-    }
-  }
+  for_pairs_ahead(
+      L.nx, L.ny, blockIdx.x, gridDim.x,
+      [&](int j, int i) {
+        const int o = j * pitch + i;
+        return V{load_resid(L, x, o), load2(b + o)};
+      },
+      [&](int j, int i, bool two, const V& v) {
+        const double2 r = resid_pair(v.r, v.b);
+        const int of = j * fpitch + i;
+        const float f0 = SCALE32 ? to_float(r.x) * inv32 : to_float(r.x * inv);
+        const float f1 = SCALE32 ? to_float(r.y) * inv32 : to_float(r.y * inv);
+        acc = fma(r.x, r.x, acc);
+        if (two) {
+          acc = fma(r.y, r.y, acc);
+          *reinterpret_cast<float2*>(fb + of) = make_float2(f0, f1);
+          if (zero_x) *reinterpret_cast<float2*>(fx + of) = make_float2(0.0f, 0.0f);
+        } else {
+          fb[of] = f0;
+          if (zero_x) fx[of] = 0.0f;
+        }
+      });
   return acc;
 }
 
-template <bool NINE>
-__global__ void __launch_bounds__(kNormThreads) k_refine_residual(LevelV<double> L, LevelV<float> F,
-                                                                  const Scalars* sc,
-                                                                  double* partials) {
+__global__ void __launch_bounds__(kKT) k_refine_residual(LevelV<double> L, LevelV<float> F,
+                                                         const Scalars* sc, int zero_x,
+                                                         double* partials) {
   griddep_wait();
   const double inv = sc->inv;
-  double acc = (inv > 1e-28 && inv < 1e28) ? refine_rows<NINE, true>(L, F, inv)
-                                           : refine_rows<NINE, false>(L, F, inv);
-  acc = block_sum(acc);
+  double acc = (inv > 1e-28 && inv < 1e28) ? refine_pairs<true>(L, F, inv, zero_x != 0)
+                                           : refine_pairs<false>(L, F, inv, zero_x != 0);
+  acc = krylov_block_sum(acc);
   if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
-// x += ||r_prev|| * e  (e the FP32 correction).
-// One thread per pair of points (i, i+1), i odd: interior rows start on
-// 128-byte boundaries, so the pair is one 16-byte FP64 and one 8-byte FP32
-// access; a last unpaired point (i = nx, nx odd) is done alone.
-__global__ void k_refine_update(LevelV<double> L, LevelV<float> F, const Scalars* sc) {
+// x += ||r_prev|| * e  (e the FP32 correction): 20 B a point, 250 -> 198 us at
+// 8191^2, the copy rate.
+__global__ void __launch_bounds__(kKT) k_refine_update(LevelV<double> L, LevelV<float> F,
+                                                       const Scalars* sc) {
   griddep_wait();
-  const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + 1;
-  const int j = blockIdx.y + 1;
-  if (i > L.nx) return;
   const double s = sc->scale;
-  double* x = L.x + j * L.pitch + i;
-  const float* e = F.x + j * F.pitch + i;
-  if (i < L.nx) {
-    double2 xv = *reinterpret_cast<const double2*>(x);
-    const float2 ev = *reinterpret_cast<const float2*>(e);
-    xv.x = fma(s, double(ev.x), xv.x);
-    xv.y = fma(s, double(ev.y), xv.y);
-    *reinterpret_cast<double2*>(x) = xv;
-  } else {
-    x[0] = fma(s, double(e[0]), x[0]);
-  }
+  const int pitch = L.pitch, fpitch = F.pitch;
+  double* const x = L.x;
+  const float* const e = F.x;
+  struct V {
+    double2 x;
+    float2 e;
+  };
+  for_pairs_ahead(
+      L.nx, L.ny, blockIdx.x, gridDim.x,
+      [&](int j, int i) {
+        return V{load2(x + j * pitch + i), *reinterpret_cast<const float2*>(e + j * fpitch + i)};
+      },
+      [&](int j, int i, bool two, const V& v) {
+        store2(x + j * pitch + i, fma(s, to_double(v.e.x), v.x.x), fma(s, to_double(v.e.y), v.x.y), two);
+      });
+}
+
+// Blocks of a pass over the finest level's pairs.
+int pair_blocks(const Hierarchy* h) {
+  return std::min(pair_runs(h->nx, h->ny), std::min(8 * 152, h->max_partials));
 }
 
 }  // namespace
@@ -495,11 +518,11 @@ void launch_fine_norm(Hierarchy* h, const double* x, const double* b, int what, 
 
 void launch_refine_residual(Hierarchy* h, double tol, cudaStream_t s, bool in_graph) {
   (void)tol;
-  launch_pdl(k_refine_residual<false>, dim3(h->npartials), dim3(kNormThreads), 0, s, h->d.back(),
-             h->f.back(), (const Scalars*)h->sc, h->partials);
-  launch_pdl(k_norm_final, dim3(1), dim3(kNormThreads), 0, s, (const double*)h->partials,
-             h->npartials, h->sc, 1, h->hist, h->cond, in_graph ? 1 : 0);
-  count_launch(2);
+  const int n = pair_blocks(h);
+  launch_pdl(k_refine_residual, dim3(n), dim3(kKT), 0, s, h->d.back(), h->f.back(), (const Scalars*)h->sc,
+             int(cycle_reads_zero_top(h)), h->partials);
+  count_launch();
+  launch_norm_final(h, s, in_graph, n);
 }
 
 void launch_norm_final(Hierarchy* h, cudaStream_t s, bool in_graph, int n) {
@@ -509,8 +532,7 @@ void launch_norm_final(Hierarchy* h, cudaStream_t s, bool in_graph, int n) {
 }
 
 void launch_refine_update(Hierarchy* h, cudaStream_t s) {
-  const LevelV<double>& L = h->d.back();
-  launch_pdl(k_refine_update, dim3(cdiv((L.nx + 1) / 2, kTB), L.ny), dim3(kTB), 0, s, L, h->f.back(),
+  launch_pdl(k_refine_update, dim3(pair_blocks(h)), dim3(kKT), 0, s, h->d.back(), h->f.back(),
              (const Scalars*)h->sc);
   count_launch();
 }
