@@ -503,11 +503,12 @@ void enqueue_vcycle(Hierarchy* h, std::vector<LevelV<T>>& lv, const LevelV<T>* d
       continue;
     }
     if (nine) prof_begin(BMG_PROF_LEVELS, s);
+    const bool red_only = !nine && !rc && nu2 > 0 && h->opt.smoother == BMG_SMOOTH_POINT;
     if (interp_oop) {
-      launch_interp<T>(lv[l], lv[l - 1].x, rc, s, lv[l].x2);
+      launch_interp<T>(lv[l], lv[l - 1].x, rc, s, lv[l].x2, red_only);
       std::swap(lv[l].x, lv[l].x2);
     } else {
-      launch_interp<T>(lv[l], lv[l - 1].x, rc, s);
+      launch_interp<T>(lv[l], lv[l - 1].x, rc, s, nullptr, red_only);
     }
     for (int k = 0; k < nu2; ++k) sweep(l, true, false);
     if (nine) prof_end(BMG_PROF_LEVELS, s);

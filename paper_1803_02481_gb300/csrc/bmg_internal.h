@@ -507,9 +507,11 @@ void launch_resid_restrict(const LevelV<T>& fine, bool nine, LevelV<T> coarse, c
 bool rr_fused(bool nine, bool fp64);
 // Threads of the one-block persistent coarse kernel.
 int coarse_block_threads();
+// red_only: a point sweep in reverse order follows on a 5-point level (its
+// first phase replaces the black points without reading them).
 template <typename T>
 void launch_interp(const LevelV<T>& fine, const T* xc, bool add_r_over_c, cudaStream_t s,
-                   T* out = nullptr);
+                   T* out = nullptr, bool red_only = false);
 void prepare_sweep_kernels();
 
 // The legs of a V-cycle level as one kernel each (bmg_legs.cuh).  leg_shape:
