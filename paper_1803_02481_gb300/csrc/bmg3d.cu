@@ -23,12 +23,16 @@
 #include <new>
 #include <vector>
 
+#include "bmg_divide.cuh"
 #include "bmg_internal.h"
 #include "boxmg3d.h"
 
 namespace bmg3 {
 
 using bmg::count_launch;
+using bmg::denominator;
+using bmg::Denominator;
+using bmg::divide;
 using bmg::griddep_wait;
 using bmg::set_last_error;
 
@@ -162,28 +166,6 @@ __global__ void __launch_bounds__(kA3X * kA3Y) k3_assemble(const double* __restr
 // couplings only, which are not negative (the other terms are exact zeros),
 // and the divisions by one denominator share its reciprocal: 7.7 -> 2.3 ms at
 // 255^3.
-
-// w / den for several w: q = w r with r = 1 / den rounded, corrected by the
-// exact remainder, which gives the rounded quotient (Markstein, "Computation
-// of elementary functions on the IBM RISC System/6000 processor", 1990),
-// inside the range where no product over- or underflows (judged by the high
-// words, in integers).
-static __device__ __noinline__ double rare_divide(double a, double b) { return a / b; }
-struct Denominator {
-  double den, r;
-  int hd;        // high word of den (its sign and exponent)
-  bool plain;
-};
-__device__ __forceinline__ Denominator denominator(double d) {
-  const int hd = __double2hiint(d);
-  return Denominator{d, __drcp_rn(d), hd, hd < (200 << 20) || hd > (1800 << 20)};
-}
-__device__ __forceinline__ double divide(double w, const Denominator& d) {
-  const int hw = __double2hiint(w) & 0x7FFFFFFF;
-  if (d.plain || (hw != 0 && (hw < d.hd - (100 << 20) || hw > d.hd + (100 << 20)))) return rare_divide(w, d.den);
-  const double q = w * d.r;
-  return fma(fma(-q, d.den, w), d.r, q);
-}
 
 // The weights of fine point (i, j, k) that lies between coarse points in the
 // directions with FX, FY, FZ = 1 (at least one).

@@ -3,6 +3,7 @@
 //   interpolation weights, the Galerkin product P^T A P, the Cholesky factor
 //   of the coarsest operator, dense <-> plane copies, and the backward of the
 //   assembly (adjoint gradient).
+#include "bmg_divide.cuh"
 #include "bmg_internal.h"
 
 #include <cmath>
@@ -26,7 +27,8 @@ __device__ __forceinline__ double cell_k(const double* __restrict__ k, size_t q,
   return log_k ? exp(k[q]) : k[q];
 }
 
-// Assembly tile: kAX x kAY cells per block, one thread per cell.
+// Tile of the assembly (cells) and of the weights (coarse indices): one thread
+// each.
 constexpr int kAX = 32, kAY = 8;
 
 // Face and cell factors of the assembly: D = diag(k / r, k r) on cells of
@@ -48,54 +50,89 @@ __device__ __forceinline__ double boundary_face(double d, double kn, double beta
 }
 
 // Writes C, 1/C, W, S of the finest level and a dense copy of k; flags k that
-// is not finite and positive.  Each thread forms the west and south faces of
-// its cell (each interior face once); the east and north faces come from the
-// neighbours through shared memory, the tile's last column and row forming
-// the faces beyond it.  The east face of cell q is the same call as the west
-// face of cell q+1, so C is what forming all four faces per cell would give.
-template <typename T>
+// is not finite and positive.  The tile's coefficients and a halo of one cell
+// are read (and their exponential taken) once, into shared memory; each thread
+// forms the west and south faces of its cell (each interior face once); the
+// east and north faces come from the neighbours through shared memory.  The
+// east face of cell q is the same call as the west face of cell q+1, so C is
+// what forming all four faces per cell would give.
+//
+// What bounds it: FP64 instructions, which a warp issues at the same cost
+// whatever its active lanes.  The faces beyond the tile and the halo's
+// exponentials are therefore dealt to whole warps instead of to every warp's
+// last lane, the range check is done on the bits, and with UNIT (r = aspect =
+// 1) the multiplications by an exact 1 are left out: 57 -> 38 operations a
+// cell (6.5 -> 4.0 ms at 8191^2).
+template <typename T, bool UNIT>
 __global__ void __launch_bounds__(kAX * kAY) k_assemble(const double* __restrict__ k, int nx,
                                                         int ny, LevelV<T> L,
                                                         double* __restrict__ kcopy, int* derr,
                                                         bool log_k, AssemblyScale f) {
-  __shared__ double fw[kAY][kAX + 1];   // west faces, column kAX = east of the tile
-  __shared__ double fs[kAY + 1][kAX];   // south faces, row kAY = north of the tile
+  __shared__ double kt[kAY + 2][kAX + 2];   // k with a halo of one cell
+  __shared__ double fw[kAY][kAX + 1];       // west faces, column kAX = east of the tile
+  __shared__ double fs[kAY + 1][kAX];       // south faces, row kAY = north of the tile
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int i0 = blockIdx.x * kAX + tx;
-  const int j0 = blockIdx.y * kAY + ty;
+  const int ib = blockIdx.x * kAX, jb = blockIdx.y * kAY;
+  const int i0 = ib + tx, j0 = jb + ty;
   const bool in = i0 < nx && j0 < ny;
   const size_t q = size_t(j0) * nx + i0;
-  double kc = 1.0;
-  auto kx = [&](size_t c) { return cell_k(k, c, log_k) * f.inv_r; };
-  auto ky = [&](size_t c) { return cell_k(k, c, log_k) * f.r; };
-  if (in) {
-    kc = cell_k(k, q, log_k);
-    if (!(kc > 0.0) || !(kc < INFINITY)) atomicOr(derr, DEV_BADK);
-    kcopy[q] = kc;
-    const double kxc = kc * f.inv_r, kyc = kc * f.r;
-    fw[ty][tx] = i0 > 0 ? harmonic(kx(q - 1), kxc) * f.aspect : 0.0;
-    fs[ty][tx] = j0 > 0 ? harmonic(ky(q - nx), kyc) * f.inv_aspect : 0.0;
-    if (tx == kAX - 1)
-      fw[ty][kAX] = i0 < nx - 1 ? harmonic(kxc, kx(q + 1)) * f.aspect : 0.0;
-    if (ty == kAY - 1)
-      fs[kAY][tx] = j0 < ny - 1 ? harmonic(kyc, ky(q + nx)) * f.inv_aspect : 0.0;
-  }
+  // cell (i, j) of the grid into the tile; warps 0 and 1 add the rows below
+  // and above it, warp 2 the columns beside it
+  auto cell = [&](int i, int j) {
+    if (i >= 0 && i < nx && j >= 0 && j < ny)
+      kt[j - jb + 1][i - ib + 1] = cell_k(k, size_t(j) * nx + i, log_k);
+  };
+  cell(i0, j0);
+  if (ty == 0) cell(i0, jb - 1);
+  if (ty == 1) cell(i0, jb + kAY);
+  if (ty == 2 && tx < 2 * kAY) cell(tx < kAY ? ib - 1 : ib + kAX, jb + tx % kAY);
+  __syncthreads();
+  auto kx = [&](int x, int y) { return UNIT ? kt[y + 1][x + 1] : kt[y + 1][x + 1] * f.inv_r; };
+  auto ky = [&](int x, int y) { return UNIT ? kt[y + 1][x + 1] : kt[y + 1][x + 1] * f.r; };
+  // west face of tile cell (x, y), south face likewise; 0 on the boundary and
+  // beyond the grid
+  auto west = [&](int x, int y) {
+    double v = 0.0;
+    if (ib + x > 0 && ib + x < nx && jb + y < ny) {
+      v = harmonic(kx(x - 1, y), kx(x, y));
+      if (!UNIT) v = v * f.aspect;
+    }
+    fw[y][x] = v;
+  };
+  auto south = [&](int x, int y) {
+    double v = 0.0;
+    if (ib + x < nx && jb + y > 0 && jb + y < ny) {
+      v = harmonic(ky(x, y - 1), ky(x, y));
+      if (!UNIT) v = v * f.inv_aspect;
+    }
+    fs[y][x] = v;
+  };
+  west(tx, ty);
+  south(tx, ty);
+  if (ty == 0 && tx < kAY) west(kAX, tx);
+  if (ty == 1) south(tx, kAY);
   __syncthreads();
   if (!in) return;
-  const double kxc = kc * f.inv_r, kyc = kc * f.r;
+  const double kc = kt[ty + 1][tx + 1];
+  const long long bits = __double_as_longlong(kc);
+  if (!(bits > 0 && bits < 0x7FF0000000000000LL)) atomicOr(derr, DEV_BADK);
+  kcopy[q] = kc;
   const double aw = fw[ty][tx], as = fs[ty][tx];
-  const double ae = i0 < nx - 1 ? fw[ty][tx + 1] : 0.0;
-  const double an = j0 < ny - 1 ? fs[ty + 1][tx] : 0.0;
+  const double ae = fw[ty][tx + 1];
+  const double an = fs[ty + 1][tx];
   // boundary faces, in the order west, east, south, north
   double bw = 0.0;
-  if (i0 == 0) bw = bw + boundary_face(2.0 * kxc * f.aspect, kxc, f.beta[0]);
-  if (i0 == nx - 1) bw = bw + boundary_face(2.0 * kxc * f.aspect, kxc, f.beta[1]);
-  if (j0 == 0) bw = bw + boundary_face(2.0 * kyc * f.inv_aspect, kyc, f.beta[2]);
-  if (j0 == ny - 1) bw = bw + boundary_face(2.0 * kyc * f.inv_aspect, kyc, f.beta[3]);
+  if (i0 == 0 || i0 == nx - 1 || j0 == 0 || j0 == ny - 1) {
+    const double kxc = kx(tx, ty), kyc = ky(tx, ty);
+    if (i0 == 0) bw = bw + boundary_face(2.0 * kxc * f.aspect, kxc, f.beta[0]);
+    if (i0 == nx - 1) bw = bw + boundary_face(2.0 * kxc * f.aspect, kxc, f.beta[1]);
+    if (j0 == 0) bw = bw + boundary_face(2.0 * kyc * f.inv_aspect, kyc, f.beta[2]);
+    if (j0 == ny - 1) bw = bw + boundary_face(2.0 * kyc * f.inv_aspect, kyc, f.beta[3]);
+  }
   const double c = (((aw + ae) + as) + an) + bw;
   const int o = (j0 + 1) * L.pitch + (i0 + 1);
   L.C[o] = T(c);
-  L.iC[o] = T(1.0 / c);
+  L.iC[o] = T(__drcp_rn(c));
   L.W[o] = T(aw);
   L.S[o] = T(as);
 }
@@ -106,6 +143,8 @@ __global__ void __launch_bounds__(kAX * kAY) k_assemble(const double* __restrict
 //   a_X+ = max(a_X, 0),  C_eff = C - sum_X min(a_X, 0) - min(sigma, 0).
 // On M-matrix rows with sigma >= 0 (the whole assembled level) this is the
 // plain row.  Sums run in the order W, E, S, N, SW, SE, NW, NE.
+// Entries below zero are rare (the sign bits tell, in integers), a row sum
+// rounded below zero is not.
 template <typename T, bool NINE>
 struct St {
   T c, w, e, s, n, sw, se, nw, ne;
@@ -124,12 +163,23 @@ struct St {
     } else {
       sw = se = nw = ne = T(0);
     }
-    const T total = ((((((((T(0) + w) + e) + s) + n) + sw) + se) + nw) + ne);
+    T total = ((w + e) + s) + n;
+    if (NINE) total = (((total + sw) + se) + nw) + ne;
     const T sigma = c - total;
+    bool lump = sign_bit(w) || sign_bit(e) || sign_bit(s) || sign_bit(n);
+    if (NINE) lump = lump || sign_bit(sw) || sign_bit(se) || sign_bit(nw) || sign_bit(ne);
+    if (lump) {
+      St t = *this;
+      t.drop_negative();
+      *this = t;
+    }
+    c = c - (below_zero(sigma) ? sigma : T(0));
+  }
+  __device__ __noinline__ void drop_negative() {
     const T z = T(0);
     const T neg = ((((((((z + fmin(w, z)) + fmin(e, z)) + fmin(s, z)) + fmin(n, z)) + fmin(sw, z)) +
                      fmin(se, z)) + fmin(nw, z)) + fmin(ne, z));
-    c = (c - neg) - fmin(sigma, z);
+    c = c - neg;
     w = fmax(w, z);
     e = fmax(e, z);
     s = fmax(s, z);
@@ -148,8 +198,9 @@ __device__ __forceinline__ void xedge(const LevelV<T>& L, int o, T& ww, T& we, i
   St<T, NINE> a(L, o);
   const T den = (a.c - a.s) - a.n;
   if (!(den > T(0))) atomicOr(derr, DEV_BADDEN | lbit);
-  ww = ((a.w + a.sw) + a.nw) / den;
-  we = ((a.e + a.se) + a.ne) / den;
+  const auto d = denominator(den);
+  ww = divide(NINE ? (a.w + a.sw) + a.nw : a.w, d);
+  we = divide(NINE ? (a.e + a.se) + a.ne : a.e, d);
 }
 
 // y-edge point: collapse the fine row in x.
@@ -159,8 +210,9 @@ __device__ __forceinline__ void yedge(const LevelV<T>& L, int o, T& ws, T& wn, i
   St<T, NINE> a(L, o);
   const T den = (a.c - a.w) - a.e;
   if (!(den > T(0))) atomicOr(derr, DEV_BADDEN | lbit);
-  ws = ((a.s + a.sw) + a.se) / den;
-  wn = ((a.n + a.nw) + a.ne) / den;
+  const auto d = denominator(den);
+  ws = divide(NINE ? (a.s + a.sw) + a.se : a.s, d);
+  wn = divide(NINE ? (a.n + a.nw) + a.ne : a.n, d);
 }
 
 // One thread per coarse-grid index (I, J), 0 <= I <= ncx, 0 <= J <= ncy
@@ -168,44 +220,66 @@ __device__ __forceinline__ void yedge(const LevelV<T>& L, int o, T& ws, T& wn, i
 // (2I+1, 2J), the y-edge point (2I, 2J+1) and the centre point (2I+1, 2J+1)
 // where those fine points exist: on an even side the last fine point is a
 // coarse point, so column 2I+1 (or row 2J+1) may lie beyond the grid; its
-// weights stay zero and nothing is read there.  The centre point's four edge
-// neighbours are recomputed here with the same code, so the stored edge
-// weights and the ones used for the centre agree bit for bit.
+// weights stay zero and nothing is read there.  The centre point's other two
+// edge neighbours, (2I+1, 2J+2) and (2I+2, 2J+1), come from the neighbouring
+// threads through shared memory; a whole warp each computes those beyond the
+// tile.
+//
+// What bounds it: FP64 instructions (small levels: the chain of divisions).
+// Each edge once instead of twice, one reciprocal per denominator instead of a
+// division per weight, comparisons in integers: 210 -> 75 operations per
+// coarse point of a 5-point level, 350 -> 100 of a 9-point one
+// (9088 x 568: 548 -> 172 us and, for all coarser levels, 355 -> 127 us).
 template <typename T, bool NINE>
-__global__ void k_interp_weights(LevelV<T> F, int ncx, int ncy, int* derr, int level) {
+__global__ void __launch_bounds__(kAX * kAY) k_interp_weights(LevelV<T> F, int ncx, int ncy,
+                                                              int* derr, int level) {
+  __shared__ T xw[kAY + 1][kAX], xe[kAY + 1][kAX];   // x-edges (2I+1, 2J)
+  __shared__ T ys[kAY][kAX + 1], yn[kAY][kAX + 1];   // y-edges (2I, 2J+1)
   const int lbit = 1 << (8 + level);
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  const int J = blockIdx.y;
-  if (I > ncx || J > ncy) return;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int Ib = blockIdx.x * kAX, Jb = blockIdx.y * kAY;
+  const int I = Ib + tx, J = Jb + ty;
   const int p = F.pitch, cp = F.cpitch;
+  auto x_at = [&](int x, int y) {
+    const int i = 2 * (Ib + x) + 1, j = 2 * (Jb + y);
+    T w = T(0), e = T(0);
+    if (i <= F.nx && j >= 2 && j <= 2 * ncy) xedge<T, NINE>(F, j * p + i, w, e, derr, lbit);
+    xw[y][x] = w;
+    xe[y][x] = e;
+  };
+  auto y_at = [&](int x, int y) {
+    const int i = 2 * (Ib + x), j = 2 * (Jb + y) + 1;
+    T s = T(0), n = T(0);
+    if (j <= F.ny && i >= 2 && i <= 2 * ncx) yedge<T, NINE>(F, j * p + i, s, n, derr, lbit);
+    ys[y][x] = s;
+    yn[y][x] = n;
+  };
+  x_at(tx, ty);
+  y_at(tx, ty);
+  if (ty == 0) x_at(tx, kAY);
+  if (ty == 1 && tx < kAY) y_at(kAX, tx);
+  __syncthreads();
+  if (I > ncx || J > ncy) return;
   const int c = J * cp + I;
   const bool col_odd = 2 * I + 1 <= F.nx;   // fine column 2I+1 exists
   const bool row_odd = 2 * J + 1 <= F.ny;   // fine row 2J+1 exists
-  T xw0 = 0, xe0 = 0, xw1 = 0, xe1 = 0, ys0 = 0, yn0 = 0, ys1 = 0, yn1 = 0;
-  // x-edge (2I+1, 2J) and (2I+1, 2J+2)
-  if (col_odd && J >= 1) xedge<T, NINE>(F, (2 * J) * p + 2 * I + 1, xw0, xe0, derr, lbit);
-  if (col_odd && J + 1 <= ncy)
-    xedge<T, NINE>(F, (2 * J + 2) * p + 2 * I + 1, xw1, xe1, derr, lbit);
-  // y-edge (2I, 2J+1) and (2I+2, 2J+1)
-  if (row_odd && I >= 1) yedge<T, NINE>(F, (2 * J + 1) * p + 2 * I, ys0, yn0, derr, lbit);
-  if (row_odd && I + 1 <= ncx)
-    yedge<T, NINE>(F, (2 * J + 1) * p + 2 * I + 2, ys1, yn1, derr, lbit);
   if (col_odd && J >= 1) {
-    F.P[XW][c] = xw0;
-    F.P[XE][c] = xe0;
+    F.P[XW][c] = xw[ty][tx];
+    F.P[XE][c] = xe[ty][tx];
   }
   if (row_odd && I >= 1) {
-    F.P[YS][c] = ys0;
-    F.P[YN][c] = yn0;
+    F.P[YS][c] = ys[ty][tx];
+    F.P[YN][c] = yn[ty][tx];
   }
   if (!(col_odd && row_odd)) return;
   // centre (2I+1, 2J+1): the fine equation with the edge neighbours replaced
   // by their interpolants.
   St<T, NINE> a(F, (2 * J + 1) * p + 2 * I + 1);
-  F.P[CSW][c] = ((a.sw + a.w * ys0) + a.s * xw0) / a.c;
-  F.P[CSE][c] = ((a.se + a.e * ys1) + a.s * xe0) / a.c;
-  F.P[CNW][c] = ((a.nw + a.w * yn0) + a.n * xw1) / a.c;
-  F.P[CNE][c] = ((a.ne + a.e * yn1) + a.n * xe1) / a.c;
+  const auto d = denominator(a.c);
+  F.P[CSW][c] = divide((a.sw + a.w * ys[ty][tx]) + a.s * xw[ty][tx], d);
+  F.P[CSE][c] = divide((a.se + a.e * ys[ty][tx + 1]) + a.s * xe[ty][tx], d);
+  F.P[CNW][c] = divide((a.nw + a.w * yn[ty][tx]) + a.n * xw[ty + 1][tx], d);
+  F.P[CNE][c] = divide((a.ne + a.e * yn[ty][tx + 1]) + a.n * xe[ty + 1][tx], d);
 }
 
 // Matrix entry A[p, p + (dx, dy)] of the fine operator at plane offset o.
@@ -419,8 +493,11 @@ int launch_assemble(const double* k, int nx, int ny, LevelV<T> L, double* kcopy,
                     bool log_k, double r, double aspect, const double* bc_beta, cudaStream_t s) {
   const AssemblyScale f{1.0 / r, r, aspect, 1.0 / aspect,
                         {bc_beta[0], bc_beta[1], bc_beta[2], bc_beta[3]}};
-  k_assemble<T><<<dim3(cdiv(nx, kAX), cdiv(ny, kAY)), dim3(kAX, kAY), 0, s>>>(k, nx, ny, L, kcopy,
-                                                                            derr, log_k, f);
+  const dim3 grid(cdiv(nx, kAX), cdiv(ny, kAY)), block(kAX, kAY);
+  if (r == 1.0 && aspect == 1.0)
+    k_assemble<T, true><<<grid, block, 0, s>>>(k, nx, ny, L, kcopy, derr, log_k, f);
+  else
+    k_assemble<T, false><<<grid, block, 0, s>>>(k, nx, ny, L, kcopy, derr, log_k, f);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? 0 : BMG_ECUDA;
 }
@@ -428,11 +505,11 @@ int launch_assemble(const double* k, int nx, int ny, LevelV<T> L, double* kcopy,
 template <typename T>
 int launch_interp_weights(const LevelV<T>& fine, bool nine, int* derr, int level, cudaStream_t s) {
   const int ncx = fine.nx / 2, ncy = fine.ny / 2;
-  dim3 grid(cdiv(ncx + 1, 128), ncy + 1);
+  const dim3 grid(cdiv(ncx + 1, kAX), cdiv(ncy + 1, kAY)), block(kAX, kAY);
   if (nine)
-    k_interp_weights<T, true><<<grid, 128, 0, s>>>(fine, ncx, ncy, derr, level);
+    k_interp_weights<T, true><<<grid, block, 0, s>>>(fine, ncx, ncy, derr, level);
   else
-    k_interp_weights<T, false><<<grid, 128, 0, s>>>(fine, ncx, ncy, derr, level);
+    k_interp_weights<T, false><<<grid, block, 0, s>>>(fine, ncx, ncy, derr, level);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? 0 : BMG_ECUDA;
 }
