@@ -346,20 +346,38 @@ __global__ void k_rap(LevelV<T> F, LevelV<T> Cc) {
 }
 
 // Dense A_0 (FP64) from the coarsest planes, then an in-place right-looking
-// Cholesky factorisation in one thread block; stores 1/L[i][i] too.
-template <typename T>
-__global__ void k_coarse_factor(LevelV<T> L0, double* __restrict__ a, double* __restrict__ idiag,
-                                int* derr) {
+// Cholesky factorisation in one thread block; stores 1/L[i][i] too.  The
+// matrix is worked on in shared memory where it fits (SMEM, up to 160
+// unknowns: rows of n | 1, free of bank conflicts), else in `a`.
+//
+// What bounds it: the chain of n square roots and reciprocals and one SM's
+// FP64 rate in the updates.  Threads are 16 x 32 over the trailing matrix, no
+// index divisions: 70 unknowns 121 -> 90 us.
+constexpr size_t kDenseSmem = 160 * 161 * sizeof(double);
+
+inline size_t dense_smem(int n) {
+  const size_t bytes = size_t(n) * (n | 1) * sizeof(double);
+  return bytes <= kDenseSmem ? bytes : 0;
+}
+
+template <typename T, bool SMEM>
+__global__ void __launch_bounds__(512) k_coarse_factor(LevelV<T> L0, double* __restrict__ a,
+                                                       double* __restrict__ idiag, int* derr) {
+  extern __shared__ double dense[];
   const int nx = L0.nx, ny = L0.ny, n = nx * ny, p = L0.pitch;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) a[e] = 0.0;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, rows = blockDim.x >> 5;
+  double* const m = SMEM ? dense : a;
+  const int mp = SMEM ? n | 1 : n;
+  for (int i = ty; i < n; i += rows)
+    for (int j = tx; j < n; j += 32) m[size_t(i) * mp + j] = 0.0;
   __syncthreads();
   for (int r = threadIdx.x; r < n; r += blockDim.x) {
     const int i = r % nx + 1, j = r / nx + 1, o = j * p + i;
-    a[size_t(r) * n + r] = double(L0.C[o]);
+    m[size_t(r) * mp + r] = double(L0.C[o]);
     auto put = [&](int di, int dj, double v) {
       const int ii = i + di, jj = j + dj;
       if (ii < 1 || ii > nx || jj < 1 || jj > ny) return;
-      a[size_t(r) * n + (jj - 1) * nx + (ii - 1)] = -v;
+      m[size_t(r) * mp + (jj - 1) * nx + (ii - 1)] = -v;
     };
     put(-1, 0, double(L0.W[o]));
     put(1, 0, double(L0.W[o + 1]));
@@ -378,29 +396,27 @@ __global__ void k_coarse_factor(LevelV<T> L0, double* __restrict__ a, double* __
   __syncthreads();
   for (int k = 0; k < n; ++k) {
     if (threadIdx.x == 0) {
-      const double d = a[size_t(k) * n + k];
+      const double d = m[size_t(k) * mp + k];
       if (!(d > 0.0)) {
         bad = 1;
         atomicOr(derr, DEV_NOTSPD);
       }
       const double s = sqrt(d > 0.0 ? d : 1.0);
-      a[size_t(k) * n + k] = s;
+      m[size_t(k) * mp + k] = s;
       idiag[k] = 1.0 / s;
     }
     __syncthreads();
     if (bad) return;
     const double inv = idiag[k];
-    for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) a[size_t(i) * n + k] *= inv;
+    for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) m[size_t(i) * mp + k] *= inv;
     __syncthreads();
-    const int m = n - k - 1;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-      const int i = k + 1 + e / m, j = k + 1 + e % m;
-      if (j <= i) a[size_t(i) * n + j] -= a[size_t(i) * n + k] * a[size_t(j) * n + k];
-    }
+    for (int i = k + 1 + ty; i < n; i += rows)
+      for (int j = k + 1 + tx; j <= i; j += 32)
+        m[size_t(i) * mp + j] -= m[size_t(i) * mp + k] * m[size_t(j) * mp + k];
     __syncthreads();
   }
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x)
-    if (e % n > e / n) a[e] = 0.0;
+  for (int i = ty; i < n; i += rows)
+    for (int j = tx; j < n; j += 32) a[size_t(i) * n + j] = j > i ? 0.0 : m[size_t(i) * mp + j];
 }
 
 // The inverse of the coarsest operator from its factor, one column per
@@ -408,29 +424,58 @@ __global__ void k_coarse_factor(LevelV<T> L0, double* __restrict__ a, double* __
 // column of the factor.  A product with it takes the place of a substitution
 // in every V-cycle: the substitution's 2 n dependent steps of two FP64
 // operations each (9 unknowns: 3.5 us of a 25 us sub-cycle; 70 unknowns: 20
-// us) become one short chain per unknown.
+// us) become one short chain per unknown.  The factor is read into shared
+// memory where it fits: a step's column then costs no trip to L2 (70
+// unknowns: 43 -> 31 us).
+template <bool SMEM>
 __global__ void __launch_bounds__(128) k_coarse_inverse(const double* __restrict__ lo,
                                                         const double* __restrict__ idiag, int n,
                                                         double* __restrict__ inv) {
-  __shared__ double v[BMG_MAX_COARSEST], y[BMG_MAX_COARSEST];
+  extern __shared__ double dense[];
   const int c = blockIdx.x;
+  const int mp = SMEM ? n | 1 : n;
+  double* const v = dense + (SMEM ? n * mp : 0);
+  double* const y = v + n;
+  double* const id = y + n;
+  if (SMEM)
+    for (int i = threadIdx.x >> 5; i < n; i += 4)
+      for (int j = threadIdx.x & 31; j <= i; j += 32) dense[i * mp + j] = lo[size_t(i) * n + j];
+  const double* const m = SMEM ? dense : lo;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     v[i] = i == c ? 1.0 : 0.0;
     y[i] = 0.0;
+    id[i] = idiag[i];
   }
   for (int j = c; j < n; ++j) {
     __syncthreads();
-    const double yj = v[j] * idiag[j];
+    const double yj = v[j] * id[j];
     if (threadIdx.x == 0) y[j] = yj;
     for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x)
-      v[i] = fma(-lo[size_t(i) * n + j], yj, v[i]);
+      v[i] = fma(-m[size_t(i) * mp + j], yj, v[i]);
   }
   for (int j = n - 1; j >= 0; --j) {
     __syncthreads();
-    const double xj = y[j] * idiag[j];
+    const double xj = y[j] * id[j];
     if (threadIdx.x == 0) inv[size_t(c) * n + j] = xj;
-    for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-lo[size_t(j) * n + i], xj, y[i]);
+    for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-m[size_t(j) * mp + i], xj, y[i]);
   }
+}
+
+template <typename T>
+int coarse_factor(Hierarchy* h, const LevelV<T>& l0, cudaStream_t s) {
+  int* derr = &h->sc->err;
+  const size_t smem = dense_smem(h->n0), vectors = 3 * h->n0 * sizeof(double);
+  if (smem) {
+    if (!use_shared(k_coarse_factor<T, true>, smem) || !use_shared(k_coarse_inverse<true>, smem + vectors))
+      return BMG_ECUDA;
+    k_coarse_factor<T, true><<<1, 512, smem, s>>>(l0, h->chol, h->chol_idiag, derr);
+    k_coarse_inverse<true><<<h->n0, 128, smem + vectors, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv);
+  } else {
+    k_coarse_factor<T, false><<<1, 512, 0, s>>>(l0, h->chol, h->chol_idiag, derr);
+    k_coarse_inverse<false><<<h->n0, 128, vectors, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv);
+  }
+  count_launch(2);
+  return cudaGetLastError() == cudaSuccess ? 0 : BMG_ECUDA;
 }
 
 __global__ void k_downcast(LevelV<double> D, LevelV<float> F) {
@@ -527,14 +572,7 @@ int launch_rap(const LevelV<T>& fine, bool nine, LevelV<T> coarse, cudaStream_t 
 
 int launch_coarse_factor(Hierarchy* h, const LevelV<double>* l0d, const LevelV<float>* l0f,
                          cudaStream_t s) {
-  int* derr = &h->sc->err;
-  if (l0d)
-    k_coarse_factor<double><<<1, 512, 0, s>>>(*l0d, h->chol, h->chol_idiag, derr);
-  else
-    k_coarse_factor<float><<<1, 512, 0, s>>>(*l0f, h->chol, h->chol_idiag, derr);
-  k_coarse_inverse<<<h->n0, 128, 0, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv);
-  count_launch(2);
-  return cudaGetLastError() == cudaSuccess ? 0 : BMG_ECUDA;
+  return l0d ? coarse_factor(h, *l0d, s) : coarse_factor(h, *l0f, s);
 }
 
 int launch_downcast_fine(const LevelV<double>& d, LevelV<float> f, cudaStream_t s) {
