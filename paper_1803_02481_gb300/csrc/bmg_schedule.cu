@@ -105,8 +105,8 @@ double predict_vcycle_us(const Hierarchy* h, int thr, int ctas) {
 
 // Points of the largest level the shared-memory sub-cycle takes by default.
 // Measured us per V-cycle with the largest level at 7^2, 15^2 and 31^2: FP64
-// 255^2 71.2, 67.1, 71.6; FP64 511^2 105, 103, 108; FP32 255^2 47.8, 46.6,
-// 46.8; FP32 511^2 62.2, 60.8, 61.7 (a 31^2 level keeps one SM's FP64 pipes
+// 255^2 65.2, 63.2, 71.8; FP64 511^2 91.9, 90.5, 100.3; FP32 255^2 41.7, 40.3,
+// 45.6; FP32 511^2 57.6, 55.6, 59.4 (a 31^2 level keeps one SM's FP64 pipes
 // busy for longer than two launches over many SMs take).
 constexpr double kSmemPoints = 300.0;
 // The same for line smoothing, whose sub-cycle works from L2.  Measured us
