@@ -312,7 +312,8 @@ typedef struct bmg_batch bmg_batch; /* opaque, library-owned */
  * or, with opt->solver BMG_SOLVER_PCG (nu1 == nu2, no r/C term), with FP64
  * conjugate gradients preconditioned by one symmetric FP32 V(nu, nu) cycle
  * (r / ||r|| cast down, ||r|| e cast back), all problems' iterations
- * advanced together; levels of side <= 31 run in the persistent coarse
+ * advanced together; opt->interp_residual_term is ignored by the V-cycles (no
+ * r/C term on any level); levels of side <= 31 run in the persistent coarse
  * kernel, one thread block per problem.  Setup also picks the tile shape of the batched sweeps for
  * every level side by timing the candidates on this batch (cached per
  * process, and in the file named by the environment variable BMG_TUNE_CACHE

@@ -667,6 +667,7 @@ size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned
   const size_t bytes = layout<float>(h, h->threshold, a);
   const LevelV<float>& top = h->f[h->threshold - 1];
   a.top_zero = 1;
+  a.add_rc = 0;   // (the batch leaves the r/C term out on every level)
   a.err = err;
   a.x = top.x;
   a.b = top.b;
