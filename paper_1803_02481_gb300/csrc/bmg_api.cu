@@ -405,7 +405,7 @@ static bool zero_start_on() {
 template <typename T>
 static int level_leg(const Hierarchy* h, const LevelV<T>& V, int l, int ns) {
   if (h->opt.smoother != BMG_SMOOTH_POINT || h->opt.interp_residual_term || h->opt.nu2 != 1 || ns < 1 ||
-      ns > 2 || prof_active() || V.PR[PR_B])
+      ns > 2 || h->by_operation || V.PR[PR_B])
     return 0;
   return leg_shape(V.nx, V.ny, l != h->L - 1, sizeof(T) == 8);
 }
@@ -698,6 +698,7 @@ static int solve_impl(Hierarchy* h, const double* b, double* x, double tol, bmg_
   if (!h || !b || !x || !(tol > 0.0)) return BMG_EINVAL;
   const double t0 = now_ms();
   const int L = h->L;
+  h->by_operation = prof_active();
   LevelV<double>& F = h->d.back();
   const bool pcg = h->opt.solver == BMG_SOLVER_PCG;
   // the iterate and right-hand side: the fine level's x and b planes, or the
@@ -720,7 +721,7 @@ static int solve_impl(Hierarchy* h, const double* b, double* x, double tol, bmg_
   int rc = BMG_OK;
   // Graph path: the whole loop in one launch (not while kernel classes are
   // being timed with events, which need the stream path).
-  if (!prof_active() && !graphs_disabled()) {
+  if (!h->by_operation && !graphs_disabled()) {
     if (h->graph_state == 0) h->graph_state = build_solve_graph(h) == BMG_OK ? 1 : -1;
     if (h->graph_state == 1) {
       BMG_CUDA(cudaGraphLaunch(h->gexec, s));
@@ -1126,6 +1127,7 @@ int bmg_op_vcycle_from(bmg_hierarchy* hp, int level, const double* b, double* x,
     return BMG_EINVAL;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  h->by_operation = bmg::prof_active();
   auto& L = h->d[level];
   bmg::launch_pack<double>(b, L.b, L.nx, L.ny, L.pitch, s);
   if (L.PR[bmg::PR_B]) bmg::launch_prescale_b<double>(L, s);

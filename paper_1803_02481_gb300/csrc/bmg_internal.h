@@ -429,6 +429,10 @@ struct Hierarchy {
   cudaGraphExec_t gexec = nullptr;
   cudaGraphConditionalHandle cond = 0;
   int graph_state = 0;               // 0 not built, 1 ready, -1 unavailable
+  bool by_operation = false;         // the running call launches every operation
+                                     // by itself (kernel classes were being timed
+                                     // when it began: prof_active() is a switch of
+                                     // the process and may change at any time)
   bool fused_norm_allowed = true;    // stop test inside the next fine sweep
                                      // where it applies (BMG_FUSED_NORM at setup)
   void* arena = nullptr;

@@ -25,7 +25,7 @@ struct ClassRec {
 
 struct Prof {
   std::mutex mu;
-  unsigned mask = 0;             // bit c: class c is recorded
+  std::atomic<unsigned> mask{0};   // bit c: class c is recorded
   ClassRec cls[kClasses];
 };
 
