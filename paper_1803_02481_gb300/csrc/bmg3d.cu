@@ -930,6 +930,7 @@ __global__ void k3_coarse_factor(Lev3 L0, double* __restrict__ lo, double* __res
     const int i = r % nx + 1, j = (r / nx) % ny + 1, k = r / (nx * ny) + 1;
     const int o = idx3(L0, i, j, k);
     lo[size_t(r) * n + r] = L0.C[o];
+    idiag[n + r] = L0.C[o];
     for (int dk = -1; dk <= 1; ++dk)
       for (int dj = -1; dj <= 1; ++dj)
         for (int di = -1; di <= 1; ++di) {
@@ -982,27 +983,37 @@ __global__ void __launch_bounds__(128) k3_coarse_inverse(const double* __restric
   for (int j = n - 1; j >= 0; --j) {
     __syncthreads();
     const double xj = y[j] * idiag[j];
-    if (threadIdx.x == 0) inv[size_t(c) * n + j] = xj;
+    if (threadIdx.x == 0) {
+      inv[size_t(c) * n + j] = xj;
+      if (j == c) bmg::raise(inv + size_t(n) * n, xj * idiag[n + c]);
+    }
     for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-lo[size_t(j) * n + i], xj, y[i]);
   }
 }
 
 // x_0 = A_0^{-1} b_0 with the stored inverse: four lanes per unknown, one of
-// four interleaved partial sums each.  Substitution with the factor took 2 n
-// dependent steps with two barriers each (27 unknowns 20.6 us, 60 37 us).
+// four interleaved partial sums each.  Substitution with the factor takes 2 n
+// dependent steps with two barriers each (27 unknowns 20.6 us, 60 37 us) and
+// serves the operators that the inverse would lose accuracy on.
 constexpr int kSolveT = 256;
 template <typename T>
-__global__ void __launch_bounds__(kSolveT) k3_coarse_solve(Lev3T<T> L0, const double* __restrict__ inv) {
-  griddep_wait();
+__global__ void __launch_bounds__(kSolveT) k3_coarse_solve(Lev3T<T> L0, bmg::CoarseSolve s) {
   __shared__ double v[BMG_MAX_COARSEST];
+  const bool product = bmg::use_inverse(s);   // (constant since the setup)
+  griddep_wait();
   const int nx = L0.nx, ny = L0.ny, n = nx * ny * L0.nz;
   auto at = [&](int r) { return idx3(L0, r % nx + 1, (r / nx) % ny + 1, r / (nx * ny) + 1); };
   for (int r = threadIdx.x; r < n; r += kSolveT) v[r] = double(L0.b[at(r)]);
   __syncthreads();
+  if (!product) {
+    bmg::substitute(s, v);
+    for (int r = threadIdx.x; r < n; r += kSolveT) L0.x[at(r)] = T(v[r]);
+    return;
+  }
   for (int e = threadIdx.x; e < (4 * n + 31) / 32 * 32; e += kSolveT) {   // (whole warps)
     const int r = e >> 2, q = r < n ? r : 0;
     double x = bmg::inverse_part(
-        n, e & 3, 4, [&](int c) { return inv[size_t(c) * n + q]; }, [&](int c) { return v[c]; });
+        n, e & 3, 4, [&](int c) { return s.inv[size_t(c) * n + q]; }, [&](int c) { return v[c]; });
     x += __shfl_xor_sync(0xffffffffu, x, 1);
     x += __shfl_xor_sync(0xffffffffu, x, 2);
     if ((e & 3) == 0 && r < n) L0.x[at(r)] = T(x);
@@ -1159,7 +1170,8 @@ void enqueue_vcycle3(bmg3_hierarchy* h, std::vector<Lev3T<T>>& lv, cudaStream_t 
       bmg::launch_pdl(k3_restrict<T, false>, dim3(grid_pts(lv[l - 1])), dim3(kT), 0, s, V, lv[l - 1]);
     count_launch(2);
   }
-  bmg::launch_pdl(k3_coarse_solve<T>, dim3(1), dim3(kSolveT), 0, s, lv[0], (const double*)h->cinv);
+  bmg::launch_pdl(k3_coarse_solve<T>, dim3(1), dim3(kSolveT), 0, s, lv[0],
+                  bmg::CoarseSolve{h->cinv, h->chol, h->chol_idiag, h->n0, L == 1 ? 0.0 : bmg::kInverseLimit});
   count_launch();
   for (int l = 1; l < L; ++l) {
     bmg::NvtxRange r("interp_leg", l);
@@ -1452,8 +1464,8 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     o_x2 = reserve(size_t(Ff.nz + 2) * Ff.py * Ff.px * sizeof(double));
   }
   const size_t o_chol = reserve(sizeof(double) * size_t(h->n0) * h->n0);
-  const size_t o_idiag = reserve(sizeof(double) * h->n0);
-  const size_t o_cinv = reserve(sizeof(double) * size_t(h->n0) * h->n0);
+  const size_t o_idiag = reserve(2 * sizeof(double) * h->n0);
+  const size_t o_cinv = reserve(sizeof(double) * (size_t(h->n0) * h->n0 + 1));
   const size_t o_part = reserve(sizeof(double) * kNormBlocks);
   const size_t o_sc = reserve(sizeof(Scal3));
   h->arena = bmg::pool_alloc(total);

@@ -283,8 +283,8 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
     if (fp32) carve_levels<float>(cv, h->geo32, 0, h->f, L - 1, opt.smoother);
     h->kcopy = cv.raw<double>(size_t(nx) * ny);
     h->chol = cv.raw<double>(size_t(h->n0) * h->n0);
-    h->chol_idiag = cv.raw<double>(h->n0);
-    h->cinv = cv.raw<double>(size_t(h->n0) * h->n0);
+    h->chol_idiag = cv.raw<double>(2 * size_t(h->n0));
+    h->cinv = cv.raw<double>(size_t(h->n0) * h->n0 + 1);
     h->partials = cv.raw<double>(h->max_partials);
     h->hist = cv.raw<double>(BMG_MAX_HISTORY);
     h->sc = cv.raw<Scalars>(1);

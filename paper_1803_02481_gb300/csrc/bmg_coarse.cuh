@@ -62,8 +62,7 @@ struct CoarseArgs {
   int nu1, nu2, add_rc;
   int smoother;              // BMG_SMOOTH_*
   int top_nine;              // is level thr-1 9-point (else red-black)
-  const double* cinv;        // inverse of the coarsest operator
-  int n0;
+  CoarseSolve solve;         // the coarsest operator
 };
 
 template <typename T, bool NINE, class Team = BlockTeam>
@@ -140,19 +139,24 @@ __device__ void blk_interp(const LevelV<T>& F, const T* xc, int add_rc) {
   Team::sync();
 }
 
-// x_0 = A_0^{-1} b_0 with the stored inverse, one unknown per thread, in FP64.
+// x_0 = A_0^{-1} b_0 with the stored inverse, one unknown per thread, or by
+// substitution, in FP64.
 template <typename T>
-__device__ void blk_coarse_solve(const LevelV<T>& L0, const double* __restrict__ cinv, int n) {
+__device__ void blk_coarse_solve(const LevelV<T>& L0, const CoarseSolve& s) {
   __shared__ double v[BMG_MAX_COARSEST];
-  const int nx = L0.nx;
+  const int nx = L0.nx, n = s.n;
   for (int r = threadIdx.x; r < n; r += blockDim.x)
     v[r] = double(L0.b[(r / nx + 1) * L0.pitch + r % nx + 1]);
   __syncthreads();
+  const bool product = use_inverse(s);
+  if (!product) substitute(s, v);
   for (int r = threadIdx.x; r < n; r += blockDim.x) {
-    auto inv = [&](int c) { return cinv[size_t(c) * n + r]; };
+    auto inv = [&](int c) { return s.inv[size_t(c) * n + r]; };
     auto b = [&](int c) { return v[c]; };
     double x;
-    if (n <= kInverseSerial) {
+    if (!product) {
+      x = v[r];
+    } else if (n <= kInverseSerial) {
       x = inverse_part(n, 0, 1, inv, b);
     } else {
       const double s0 = inverse_part(n, 0, 4, inv, b), s1 = inverse_part(n, 1, 4, inv, b);
@@ -180,7 +184,7 @@ __device__ void coarse_cycle_body(const CoarseArgs<T>& a) {
   }
   // the coarsest solve is one block's work (block rank 0 of a cluster; its
   // own barriers are block barriers), then the whole team resumes
-  if (Team::rank() == 0) blk_coarse_solve<T>(a.lev[0], a.cinv, a.n0);
+  if (Team::rank() == 0) blk_coarse_solve<T>(a.lev[0], a.solve);
   if constexpr (Team::kCluster) Team::sync();
   for (int l = 1; l < a.thr; ++l) {
     const LevelV<T> L = a.lev[l];

@@ -54,9 +54,8 @@ struct SmArgs {
   int top_zero;            // its iterate is zero on entry
   T *x, *b;                // its planes in global memory
   int pitch;
-  const double* inv;       // inverse of the coarsest operator
-  int n0;
-  int inv_smem;            // it is in the image
+  CoarseSolve solve;       // the coarsest operator
+  int inv_smem;            // its inverse is in the image
   int nx[kMaxLevels], ny[kMaxLevels];
   int koff[kMaxLevels];    // element offset of a level's constant planes
   int voff[kMaxLevels];    // element offset of its x, b (and r) planes
@@ -392,10 +391,16 @@ __device__ __forceinline__ void up(const Lv& L, const Lv& C, Cell<T>& held, bool
 
 // x_0 = A_0^{-1} b_0 with the stored inverse (the sums of blk_coarse_solve):
 // one unknown per thread, or above kInverseSerial unknowns four lanes for
-// each, one partial sum a lane.
+// each, one partial sum a lane; or (not `product`) by substitution.
 template <typename T>
-__device__ __forceinline__ void solve0(const SmArgs<T>& a, const Lv& L) {
-  const int n = a.n0, nx = L.nx;
+__device__ __forceinline__ void solve0(const SmArgs<T>& a, const Lv& L, bool product) {
+  const int n = a.solve.n, nx = L.nx;
+  if (!product) {
+    substitute(a.solve, &sh<double>(a.soff));
+    for (int r = threadIdx.x; r < n; r += kNT)
+      sh<T>(L.x + (r / nx + 1) * L.sp + r % nx + 1) = T(sh<double>(a.soff + r));
+    return;
+  }
   const bool quad = n > kInverseSerial;
   const int per = quad ? 4 : 1, k = quad ? int(threadIdx.x) & 3 : 0;
   for (int r0 = 0; r0 < n; r0 += kNT / per) {
@@ -403,7 +408,7 @@ __device__ __forceinline__ void solve0(const SmArgs<T>& a, const Lv& L) {
     if (r0 + (int(threadIdx.x) & ~31) / per >= n) break;   // (warp-uniform)
     const int q = r < n ? r : 0;
     auto inv = [&](int c) {
-      return a.inv_smem ? sh<double>(a.foff + c * n + q) : a.inv[size_t(c) * n + q];
+      return a.inv_smem ? sh<double>(a.foff + c * n + q) : a.solve.inv[size_t(c) * n + q];
     };
     auto b = [&](int c) { return sh<double>(a.soff + c); };
     double x = inverse_part(n, k, per, inv, b);
@@ -433,6 +438,7 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   // zero iterates (with their ghosts) and the residuals' ghosts, which the
   // restriction of an even side reads
   for (int e = a.voff[0] + threadIdx.x; e < a.end; e += kNT) sh<T>(e) = T(0);
+  const bool product = use_inverse(a.solve);   // (constant since the setup, like the image)
   __syncthreads();
   Cell<T> held{};
   int mine = 0;                          // OWN: this thread's level
@@ -484,10 +490,10 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   }
   {
     const Lv L(a, 0);
-    for (int r = threadIdx.x; r < a.n0; r += kNT)
+    for (int r = threadIdx.x; r < a.solve.n; r += kNT)
       sh<double>(a.soff + r) = double(sh<T>(L.b + (r / L.nx + 1) * L.sp + r % L.nx + 1));
     __syncthreads();
-    solve0<T>(a, L);
+    solve0<T>(a, L, product);
   }
   __syncthreads();
   for (int l = 1; l <= top; ++l) {
@@ -533,7 +539,7 @@ __global__ void k_coarse_image(const __grid_constant__ SmArgs<T> a, const LevelV
   if (blockIdx.x == gridDim.x - 1) {
     double* d = reinterpret_cast<double*>(image) + a.foff;
     if (a.inv_smem)
-      for (int e = threadIdx.x; e < a.n0 * a.n0; e += blockDim.x) d[e] = a.inv[e];
+      for (int e = threadIdx.x; e < a.solve.n * a.solve.n; e += blockDim.x) d[e] = a.solve.inv[e];
     return;
   }
   const int l = 1 + blockIdx.x / (NK9 + NPW), p = blockIdx.x % (NK9 + NPW);
@@ -572,7 +578,6 @@ size_t layout(const Hierarchy* h, int thr, SmArgs<T>& a) {
     if (off * sizeof(T) > kCoarseImageMax) return 0;
   }
   const size_t n0 = size_t(h->n0);
-  a.n0 = int(n0);
   a.inv_smem = n0 <= kInvSmem;
   a.foff = int((off * sizeof(T) + 7) / 8);
   size_t bytes = 8 * (size_t(a.foff) + (a.inv_smem ? n0 * n0 : 0));
@@ -595,7 +600,7 @@ size_t layout(const Hierarchy* h, int thr, SmArgs<T>& a) {
   a.nu1 = h->opt.nu1;
   a.nu2 = h->opt.nu2;
   a.add_rc = h->opt.interp_residual_term;
-  a.inv = h->cinv;
+  a.solve = coarse_solve(h);
   a.image = h->coarse_image;
   a.err = &h->sc->err;
   return bytes <= kCoarseImageMax ? bytes : 0;

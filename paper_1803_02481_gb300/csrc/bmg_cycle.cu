@@ -519,8 +519,7 @@ void launch_coarse_cycle(Hierarchy* h, const std::vector<LevelV<T>>& lv, const L
   a.add_rc = h->opt.interp_residual_term;
   a.smoother = h->opt.smoother;
   a.top_nine = (thr < h->L) ? 1 : 0;
-  a.cinv = h->cinv;
-  a.n0 = h->n0;
+  a.solve = coarse_solve(h);
   prof_begin(BMG_PROF_COARSE, s);
   if (a.smoother != BMG_SMOOTH_POINT)
     launch_pdl(k_coarse_cycle_line<T>, dim3(1), dim3(512), 0, s, a);

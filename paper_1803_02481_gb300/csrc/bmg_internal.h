@@ -339,8 +339,56 @@ __device__ __forceinline__ T interp_value(T* const* P, int cp, const T* __restri
   return v;
 }
 
-// Unknown r of x = A_0^{-1} b: row r of the stored inverse (entry (r, c) at
-// c * n + r) times b, read through `inv(c)` and `b(c)`.  More than 16
+// The coarsest operator A_0 of n unknowns as its solve takes it.  A V-cycle
+// multiplies by the stored inverse (2 n dependent steps of a substitution
+// become one short chain per unknown), but the residual of that product grows
+// with the condition number, which a substitution's does not: on 3 x 40 points
+// with three no-flux walls and beta = 1e-4 on the fourth a zero-mean right-hand
+// side was left at 3e-11 of its norm instead of 3e-15.  So the inverse is for
+// operators whose measure max_i A_ii (A^-1)_ii is below kInverseLimit: it is 1
+// for a diagonal matrix, the diagonally scaled operator's condition to within
+// a factor n^2, and at most 2.2 on the timed workloads (up to 12 on others of
+// their kinds); at the limit the product's excess is about 1e3 n u.  A hierarchy of one level
+// substitutes always: its cycle is this solve alone, and no later one corrects
+// it.
+struct CoarseSolve {
+  const double* inv;     // entry (r, c) at c * n + r; then the measure
+  const double* lo;      // Cholesky factor, row-major
+  const double* idiag;   // 1 / its diagonal
+  int n;
+  double limit;
+};
+constexpr double kInverseLimit = 1e3;
+
+__device__ __forceinline__ bool use_inverse(const CoarseSolve& s) { return s.inv[size_t(s.n) * s.n] < s.limit; }
+
+// Raises *most to v (> 0; anything else counts as infinite).
+__device__ __forceinline__ void raise(double* most, double v) {
+  atomicMax(reinterpret_cast<unsigned long long*>(most),
+            static_cast<unsigned long long>(__double_as_longlong(v > 0.0 ? v : INFINITY)));
+}
+
+// Forward and backward substitution on v (shared memory, b in, x out) by the
+// whole block; the caller's barriers stand before and after it.
+__device__ __forceinline__ void substitute(const CoarseSolve& s, double* v) {
+  const int n = s.n;
+  for (int j = 0; j < n; ++j) {
+    const double y = v[j] * s.idiag[j];
+    __syncthreads();
+    if (threadIdx.x == 0) v[j] = y;
+    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) v[i] = fma(-s.lo[size_t(i) * n + j], y, v[i]);
+    __syncthreads();
+  }
+  for (int j = n - 1; j >= 0; --j) {
+    const double x = v[j] * s.idiag[j];
+    __syncthreads();
+    if (threadIdx.x == 0) v[j] = x;
+    for (int i = threadIdx.x; i < j; i += blockDim.x) v[i] = fma(-s.lo[size_t(j) * n + i], x, v[i]);
+    __syncthreads();
+  }
+}
+
+// Unknown r of x = A_0^{-1} b: row r of the stored inverse times b, read through `inv(c)` and `b(c)`.  More than 16
 // unknowns: four interleaved partial sums, part `k` of them here, added as
 // (s0 + s1) + (s2 + s3).
 constexpr int kInverseSerial = 16;
@@ -411,8 +459,8 @@ struct Hierarchy {
   std::vector<Geom> geo64, geo32;
   double* kcopy = nullptr;           // dense (ny, nx) copy of k
   double* chol = nullptr;            // N0 x N0 lower factor (row-major)
-  double* chol_idiag = nullptr;      // 1 / L[i][i]
-  double* cinv = nullptr;            // inverse of the coarsest operator, column by column
+  double* chol_idiag = nullptr;      // 1 / L[i][i], then A_0's diagonal
+  double* cinv = nullptr;            // inverse of the coarsest operator and its measure (CoarseSolve)
   int n0 = 0;
   double* partials = nullptr;        // reduction scratch
   double* hist = nullptr;            // relative residual per cycle (BMG_MAX_HISTORY)
@@ -479,6 +527,10 @@ void pinned_slot_free(void* p);
 int setup_impl(const double* k, int nx, int ny, const bmg_options* opt, cudaStream_t s,
                Hierarchy** out);
 void free_hierarchy(Hierarchy* h);
+
+inline CoarseSolve coarse_solve(const Hierarchy* h) {
+  return CoarseSolve{h->cinv, h->chol, h->chol_idiag, h->n0, h->L == 1 ? 0.0 : kInverseLimit};
+}
 
 // Kernel launch wrappers (defined in the .cu files).
 template <typename T>

@@ -346,7 +346,8 @@ __global__ void k_rap(LevelV<T> F, LevelV<T> Cc) {
 }
 
 // Dense A_0 (FP64) from the coarsest planes, then an in-place right-looking
-// Cholesky factorisation in one thread block; stores 1/L[i][i] too.  The
+// Cholesky factorisation in one thread block; stores 1/L[i][i] and the
+// diagonal of A_0 too.  The
 // matrix is worked on in shared memory where it fits (SMEM, up to 160
 // unknowns: rows of n | 1, free of bank conflicts), else in `a`.
 //
@@ -374,6 +375,7 @@ __global__ void __launch_bounds__(512) k_coarse_factor(LevelV<T> L0, double* __r
   for (int r = threadIdx.x; r < n; r += blockDim.x) {
     const int i = r % nx + 1, j = r / nx + 1, o = j * p + i;
     m[size_t(r) * mp + r] = double(L0.C[o]);
+    idiag[n + r] = double(L0.C[o]);
     auto put = [&](int di, int dj, double v) {
       const int ii = i + di, jj = j + dj;
       if (ii < 1 || ii > nx || jj < 1 || jj > ny) return;
@@ -419,7 +421,8 @@ __global__ void __launch_bounds__(512) k_coarse_factor(LevelV<T> L0, double* __r
     for (int j = tx; j < n; j += 32) a[size_t(i) * n + j] = j > i ? 0.0 : m[size_t(i) * mp + j];
 }
 
-// The inverse of the coarsest operator from its factor, one column per
+// The inverse of the coarsest operator from its factor, and its measure (see
+// CoarseSolve; zeroed by the caller), one column per
 // block: forward and backward substitution of a unit vector, one barrier per
 // column of the factor.  A product with it takes the place of a substitution
 // in every V-cycle: the substitution's 2 n dependent steps of two FP64
@@ -456,7 +459,10 @@ __global__ void __launch_bounds__(128) k_coarse_inverse(const double* __restrict
   for (int j = n - 1; j >= 0; --j) {
     __syncthreads();
     const double xj = y[j] * id[j];
-    if (threadIdx.x == 0) inv[size_t(c) * n + j] = xj;
+    if (threadIdx.x == 0) {
+      inv[size_t(c) * n + j] = xj;
+      if (j == c) raise(inv + size_t(n) * n, xj * idiag[n + c]);
+    }
     for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-m[size_t(j) * mp + i], xj, y[i]);
   }
 }
