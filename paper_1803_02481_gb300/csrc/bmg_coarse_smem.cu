@@ -425,7 +425,10 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   using namespace tma_detail;
   __shared__ __align__(8) uint64_t bar;
   const int top = a.thr - 1;
-  if (threadIdx.x == 0) {
+  // no level above the coarsest here and an inverse too large to stage: the
+  // image is empty, and a bulk copy of no bytes is not defined
+  const bool staged = a.image_bytes > 0;
+  if (staged && threadIdx.x == 0) {
     mbar_init(&bar, 1);
     fence_mbar_init();
     mbar_expect_tx(&bar, unsigned(a.image_bytes));
@@ -445,7 +448,7 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   bool ok = true;
   if (OWN) {
     // levels top .. 1 take warps in turn
-    ok = mbar_wait_bounded(&bar, 0);
+    if (staged) ok = mbar_wait_bounded(&bar, 0);
     int first = 0;
     for (int l = top; ok && l >= 1; --l) {
       const Lv L(a, l);
@@ -471,7 +474,7 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
       if (!a.top_zero) sh<T>(L.x + j * L.sp + i) = a.x[j * a.pitch + i];
     }
   }
-  if (!OWN) ok = mbar_wait_bounded(&bar, 0);
+  if (!OWN && staged) ok = mbar_wait_bounded(&bar, 0);
   if (!__syncthreads_and(ok)) {
     if (threadIdx.x == 0) {
       atomicOr(a.err, DEV_TIMEOUT);

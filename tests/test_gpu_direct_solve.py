@@ -76,3 +76,21 @@ def test_one_level_solve_3d(nx, ny, nz, prec, tol):
     h.destroy()
     want = np.linalg.solve(O3.assemble_fv7(k).toarray(), b.ravel())
     assert np.abs(x.cpu().numpy().ravel() - want).max() <= tol * np.abs(want).max()
+
+
+@pytest.mark.parametrize("kw", [{}, {"precision": bm.BMG_FP32_REFINE}, {"solver": bm.BMG_SOLVER_PCG, "nu1": 1},
+                                {"solver": bm.BMG_SOLVER_PCG, "nu1": 1, "precision": bm.BMG_FP32_REFINE}])
+@pytest.mark.parametrize("nx,ny", [(500, 31), (31, 500), (3, 33), (3, 32)])
+def test_sub_cycle_with_nothing_to_stage(nx, ny, kw):
+    """A coarsest level of more than 96 unknowns (186, 99) with no other level
+    in the sub-cycle, and one of exactly 96: the stop test is met.  Bound as
+    above."""
+    rng = np.random.default_rng(nx + ny)
+    k = 10.0 ** rng.uniform(-0.5, 0.5, (ny, nx))
+    b = rng.uniform(-1, 1, (ny, nx))
+    h = bm.setup(torch.from_numpy(k).cuda(), bm.default_options(**kw))
+    x, info = h.solve(torch.from_numpy(b).cuda(), tol=1e-10)
+    h.destroy()
+    assert info.threshold == 1
+    r = O.residual(O.assemble_fv5(k), x.cpu().numpy(), b)
+    assert np.linalg.norm(r) <= 1.05e-10 * np.linalg.norm(b)
