@@ -1051,6 +1051,7 @@ struct bmg3_hierarchy {
   cudaGraph_t pcg_graph[2] = {nullptr, nullptr};          // first iteration, later ones
   cudaGraphExec_t pcg_exec[2] = {nullptr, nullptr};
   void* arena = nullptr;
+  bool failed = false;              // a call failed: its work may be under way
   double *chol = nullptr, *chol_idiag = nullptr, *cinv = nullptr, *partials = nullptr;
   Scal3* sc = nullptr;
   Scal3* sc_host = nullptr;
@@ -1089,7 +1090,7 @@ void free3(bmg3_hierarchy* h) {
     if (h->pcg_exec[g]) cudaGraphExecDestroy(h->pcg_exec[g]);
     if (h->pcg_graph[g]) cudaGraphDestroy(h->pcg_graph[g]);
   }
-  bmg::pool_free(h->arena);   // (waits for the device)
+  bmg::pool_free(h->arena, !h->failed);
   bmg::pinned_slot_free(h->sc_host);
   delete h;
 }
@@ -1527,6 +1528,7 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
   h->sc = reinterpret_cast<Scal3*>(base + o_sc);
   h->err = &h->sc->err;
   if (cudaMemsetAsync(h->arena, 0, total, s) != cudaSuccess) {
+    h->failed = true;
     free3(h);
     return BMG_ECUDA;
   }
@@ -1553,11 +1555,13 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     count_launch();
   }
   if (cudaGetLastError() != cudaSuccess) {
+    h->failed = true;
     free3(h);
     return BMG_ECUDA;
   }
   int rc = check_err(h, s);
   if (rc) {
+    h->failed = rc == BMG_ECUDA;   // (any other code: the stream was waited for)
     free3(h);
     return rc;
   }
@@ -1566,9 +1570,8 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
   return BMG_OK;
 }
 
-int bmg3_solve(bmg3_hierarchy* h, const double* b, double* x, double tol, bmg_info* info,
-               bmg_stream_t stream) {
-  if (!h || !b || !x || !(tol >= 0.0)) return BMG_EINVAL;
+static int solve3(bmg3_hierarchy* h, const double* b, double* x, double tol, bmg_info* info,
+                  bmg_stream_t stream) {
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const double t0 = now_ms();
   if (h->pcg) {
@@ -1680,6 +1683,14 @@ int bmg3_solve(bmg3_hierarchy* h, const double* b, double* x, double tol, bmg_in
     info->solve_ms = now_ms() - t0;
     info->coarse_ctas = 1;
   }
+  return rc;
+}
+
+int bmg3_solve(bmg3_hierarchy* h, const double* b, double* x, double tol, bmg_info* info,
+               bmg_stream_t stream) {
+  if (!h || !b || !x || !(tol >= 0.0)) return BMG_EINVAL;
+  const int rc = solve3(h, b, x, tol, info, stream);
+  if (rc == BMG_ECUDA) h->failed = true;
   return rc;
 }
 

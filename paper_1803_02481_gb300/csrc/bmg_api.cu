@@ -177,7 +177,7 @@ void free_hierarchy(Hierarchy* h) {
   if (!h) return;
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
   if (h->graph) cudaGraphDestroy(h->graph);
-  pool_free(h->arena);   // (waits for the device)
+  pool_free(h->arena, h->pending.wait());
   pinned_slot_free(h->sc_host);
   for (auto* m : h->maps64) delete m;
   for (auto* m : h->maps32) delete m;
@@ -315,6 +315,7 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
   }
   int rc = BMG_OK;
   auto fail = [&](int code) {
+    if (code == BMG_ECUDA) h->pending.lost();   // (any other code: the stream was waited for)
     free_hierarchy(h);
     return code;
   };
@@ -876,7 +877,9 @@ int bmg_setup(const double* k_dev, int nx, int ny, const bmg_options* opt, bmg_s
 
 int bmg_solve(bmg_hierarchy* h, const double* b_dev, double* x_dev, double tol, bmg_info* info,
               bmg_stream_t stream) {
-  return bmg::solve_impl(H(h), b_dev, x_dev, tol, info, reinterpret_cast<cudaStream_t>(stream));
+  const int rc = bmg::solve_impl(H(h), b_dev, x_dev, tol, info, reinterpret_cast<cudaStream_t>(stream));
+  if (rc == BMG_ECUDA) H(h)->pending.lost();
+  return rc;
 }
 
 void bmg_destroy(bmg_hierarchy* h) { bmg::free_hierarchy(H(h)); }
@@ -909,8 +912,10 @@ int bmg_solve_host(const double* k_host, const double* b_host, double* x_host, i
     }
   }
   if (info) info->setup_ms = setup_ms;
+  // (an argument that setup refuses leaves the copies under way)
+  const bool idle = cudaStreamSynchronize(s) == cudaSuccess;
   bmg_destroy(h);
-  bmg::pool_free(buf);
+  bmg::pool_free(buf, idle);
   return rc;
 }
 
@@ -1038,6 +1043,12 @@ int bmg_coarse_factor(const bmg_hierarchy* hp, double* host_out, int n0_capacity
   return BMG_OK;
 }
 
+// The end of a call whose work on `s` is not waited for.
+static int op_end(bmg_hierarchy* hp, cudaStream_t s) {
+  H(hp)->pending.left(s);
+  return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
+}
+
 static int op_check(bmg_hierarchy* hp, int level, int lo) {
   Hierarchy* h = H(hp);
   if (!h || level < lo || level >= h->L) return BMG_EINVAL;
@@ -1068,7 +1079,7 @@ int bmg_op_relax(bmg_hierarchy* hp, int level, double* x, const double* b, int n
   bmg::launch_unpack<double>(L.x, x, L.nx, L.ny, L.pitch, s);
   // keep the level's buffer roles as the recorded solve graph expects them
   if (nu & 1) std::swap(L.x, L.x2);
-  return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
+  return op_end(hp, s);
 }
 
 int bmg_op_residual(bmg_hierarchy* hp, int level, const double* x, const double* b, double* r,
@@ -1083,7 +1094,7 @@ int bmg_op_residual(bmg_hierarchy* hp, int level, const double* x, const double*
   bmg::launch_pack<double>(b, L.b, L.nx, L.ny, L.pitch, s);
   bmg::launch_residual<double>(L, level != h->L - 1, L.x, L.b, L.r, s);
   bmg::launch_unpack<double>(L.r, r, L.nx, L.ny, L.pitch, s);
-  return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
+  return op_end(hp, s);
 }
 
 int bmg_op_restrict(bmg_hierarchy* hp, int level, const double* r, double* bc,
@@ -1098,7 +1109,7 @@ int bmg_op_restrict(bmg_hierarchy* hp, int level, const double* r, double* bc,
   bmg::launch_pack<double>(r, L.r, L.nx, L.ny, L.pitch, s);
   bmg::launch_restrict<double>(L, L.r, Lc, false, s);
   bmg::launch_unpack<double>(Lc.b, bc, Lc.nx, Lc.ny, Lc.pitch, s);
-  return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
+  return op_end(hp, s);
 }
 
 int bmg_op_interp(bmg_hierarchy* hp, int level, const double* xc, double* x,
@@ -1114,7 +1125,7 @@ int bmg_op_interp(bmg_hierarchy* hp, int level, const double* xc, double* x,
   bmg::launch_pack<double>(x, L.x, L.nx, L.ny, L.pitch, s);
   bmg::launch_interp<double>(L, Lc.x, false, s);
   bmg::launch_unpack<double>(L.x, x, L.nx, L.ny, L.pitch, s);
-  return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
+  return op_end(hp, s);
 }
 
 int bmg_op_vcycle_from(bmg_hierarchy* hp, int level, const double* b, double* x, bmg_stream_t stream) {
@@ -1132,11 +1143,13 @@ int bmg_op_vcycle_from(bmg_hierarchy* hp, int level, const double* b, double* x,
   bmg::launch_pack<double>(b, L.b, L.nx, L.ny, L.pitch, s);
   if (L.PR[bmg::PR_B]) bmg::launch_prescale_b<double>(L, s);
   if (cudaMemsetAsync(L.x - bmg::base_shift<double>(), 0, h->geo64[level].elems * sizeof(double), s) !=
-      cudaSuccess)
+      cudaSuccess) {
+    h->pending.lost();
     return BMG_ECUDA;
+  }
   bmg::enqueue_vcycle<double>(h, h->d, h->dlev64, h->threshold, s, level);
   bmg::launch_unpack<double>(L.x, x, L.nx, L.ny, L.pitch, s);
-  return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
+  return op_end(hp, s);
 }
 
 int bmg_assemble_backward(bmg_hierarchy* hp, const double* u, const double* lam, double* dtheta,
@@ -1146,9 +1159,9 @@ int bmg_assemble_backward(bmg_hierarchy* hp, const double* u, const double* lam,
   if (h->opt.aniso_r != 1.0 || h->opt.cell_aspect != 1.0) return BMG_EINVAL;
   for (double b : h->opt.bc_beta)
     if (b >= 0.0) return BMG_EINVAL;
-  bmg::launch_assemble_backward(h->kcopy, u, lam, dtheta, h->nx, h->ny,
-                                reinterpret_cast<cudaStream_t>(stream));
-  return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  bmg::launch_assemble_backward(h->kcopy, u, lam, dtheta, h->nx, h->ny, s);
+  return op_end(hp, s);
 }
 
 }  // extern "C"

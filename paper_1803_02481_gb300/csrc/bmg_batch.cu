@@ -498,8 +498,11 @@ T* carve(char*& p, size_t n) {
   return r;
 }
 
-void destroy_batch(Batch* b) {
+// failed: work of a call that failed may be under way on the hierarchies.
+void destroy_batch(Batch* b, bool failed = false) {
   if (!b) return;
+  if (failed)
+    for (Hierarchy* h : b->hs) h->pending.lost();
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   for (Hierarchy* h : b->hs) free_hierarchy(h);
@@ -790,7 +793,7 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
   b->nprob = nprob;
   b->opt = opt;
   auto fail = [&](int code) {
-    destroy_batch(b);
+    destroy_batch(b, code == BMG_ECUDA);
     return code;
   };
   // individual hierarchies (threshold: levels of side <= 31 in the coarse kernel)
@@ -920,11 +923,9 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
   return BMG_OK;
 }
 
-extern "C" int bmg_batch_solve(bmg_batch* bp, const double* const* b_dev, double* const* x_dev,
-                               double tol, bmg_info* per_prob, bmg_stream_t stream) {
+static int batch_solve(bmg::Batch* b, const double* const* b_dev, double* const* x_dev, double tol,
+                       bmg_info* per_prob, bmg_stream_t stream) {
   using namespace bmg;
-  Batch* b = reinterpret_cast<Batch*>(bp);
-  if (!b || !b_dev || !x_dev || !(tol > 0.0)) return BMG_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const double t0 = now_ms();
   const bool pcg = b->opt.solver == BMG_SOLVER_PCG;
@@ -964,6 +965,16 @@ extern "C" int bmg_batch_solve(bmg_batch* bp, const double* const* b_dev, double
     else if ((r.err & DEV_TIMEOUT) && (rc == BMG_OK || rc == BMG_ENOCONV)) rc = BMG_ETIMEOUT;
     else if (!(r.rel <= tol) && r.bnorm2 > 0.0 && rc == BMG_OK) rc = BMG_ENOCONV;
   }
+  return rc;
+}
+
+extern "C" int bmg_batch_solve(bmg_batch* bp, const double* const* b_dev, double* const* x_dev,
+                               double tol, bmg_info* per_prob, bmg_stream_t stream) {
+  Batch* b = reinterpret_cast<Batch*>(bp);
+  if (!b || !b_dev || !x_dev || !(tol > 0.0)) return BMG_EINVAL;
+  const int rc = batch_solve(b, b_dev, x_dev, tol, per_prob, stream);
+  if (rc == BMG_ECUDA)
+    for (bmg::Hierarchy* h : b->hs) h->pending.lost();
   return rc;
 }
 

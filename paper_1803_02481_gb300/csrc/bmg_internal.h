@@ -446,6 +446,27 @@ struct SweepMaps {
 
 struct Timing;
 
+// Work on an object's memory that its calls returned from without waiting
+// (the single operations; solves and setups end with a synchronised stream).
+// The memory is handed on only once all of it is done, and that is found out
+// by these events: a wait for the whole device would spoil any recording
+// (stream capture) that another thread has under way.
+class Pending {
+ public:
+  ~Pending();
+  void left(cudaStream_t s);   // a call ends here, its work on s under way
+  void lost() { unknown_ = true; }   // work that no event marks (a call failed)
+  bool wait();                 // waits for the work left; false: not all of it is known
+
+ private:
+  struct Entry {
+    cudaStream_t stream;
+    cudaEvent_t done;
+  };
+  std::vector<Entry> entries_;
+  bool unknown_ = false;
+};
+
 struct Hierarchy {
   int nx = 0, ny = 0, L = 0;
   bmg_options opt{};
@@ -485,6 +506,7 @@ struct Hierarchy {
                                      // where it applies (BMG_FUSED_NORM at setup)
   void* arena = nullptr;
   size_t arena_bytes = 0;
+  Pending pending;                   // work on the arena
   double setup_ms = 0.0;
   // TMA descriptors per level of d / f (null where a level is swept by the
   // tiled kernel)
@@ -517,9 +539,10 @@ void prof_end(int which, cudaStream_t s);
 
 // Device memory kept between hierarchies, and pinned slots of up to 256 bytes
 // (bmg_pool.cu); null when there is none to be had.  pool_free and
-// pinned_slot_free take what these returned, or null.
+// pinned_slot_free take what these returned, or null; idle: no work on the
+// block is under way (else it goes back to the driver, which waits).
 void* pool_alloc(size_t bytes);
-void pool_free(void* p);
+void pool_free(void* p, bool idle);
 void* pinned_slot(size_t bytes);
 void pinned_slot_free(void* p);
 

@@ -10,9 +10,10 @@
 //  * Bounded: at most 1/32 of the device's memory is kept per device; the
 //    oldest blocks go back to the driver first, and all of them when an
 //    allocation fails (and the allocation is tried again).
-//  * A block is handed on only after the device has finished all work
-//    submitted before it was given back (what cudaFree waits for as well), so
-//    it does not matter which streams used it or will use it.
+//  * A block is kept only if the work on it is done when it is given back (its
+//    owner waits for what it left under way, see Pending), so it does not
+//    matter which streams used it or will use it; any other goes to cudaFree,
+//    which waits for it.
 //  * Thread-safe; blocks stay on their device.
 #include "bmg_internal.h"
 
@@ -114,7 +115,42 @@ void* pool_alloc(size_t bytes) {
   return p;
 }
 
-void pool_free(void* p) {
+Pending::~Pending() {
+  for (Entry& e : entries_) cudaEventDestroy(e.done);
+}
+
+void Pending::left(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    unknown_ = true;   // runs whenever the caller's graph does
+    return;
+  }
+  for (Entry& e : entries_)
+    if (e.stream == s) {
+      // (the wait holds nothing up on the stream that recorded the event, and
+      // orders a new stream of the same handle behind the old one)
+      if (cudaStreamWaitEvent(s, e.done, 0) != cudaSuccess || cudaEventRecord(e.done, s) != cudaSuccess)
+        unknown_ = true;
+      return;
+    }
+  Entry e{s, nullptr};
+  if (cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming) != cudaSuccess) {
+    unknown_ = true;
+    return;
+  }
+  entries_.push_back(e);
+  if (cudaEventRecord(e.done, s) != cudaSuccess) unknown_ = true;
+}
+
+bool Pending::wait() {
+  for (Entry& e : entries_)
+    if (cudaEventSynchronize(e.done) != cudaSuccess) unknown_ = true;
+  if (unknown_) cudaGetLastError();
+  return !unknown_;
+}
+
+void pool_free(void* p, bool idle) {
   if (!p) return;
   Pool& P = pool();
   Block b{};
@@ -128,12 +164,8 @@ void pool_free(void* p) {
   int cur = b.dev;
   cudaGetDevice(&cur);
   if (cur != b.dev) cudaSetDevice(b.dev);
-  // every stream's work on the block, before anyone else gets it; a device
-  // that cannot be waited for (an error, a capture in progress) keeps nothing
   const size_t limit = keep_limit(b.dev);
-  const bool idle = b.bytes <= limit && cudaDeviceSynchronize() == cudaSuccess;
-  if (!idle) {
-    cudaGetLastError();
+  if (!idle || b.bytes > limit) {
     cudaFree(p);
   } else {
     std::lock_guard<std::mutex> g(P.mu);

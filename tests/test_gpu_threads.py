@@ -1,0 +1,108 @@
+"""Hierarchies made, solved and destroyed by several threads at once."""
+import threading
+
+import pytest
+
+torch = pytest.importorskip("torch")
+import paper_1803_02481_gb300 as bm  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def run_threads(works):
+    errors = []
+
+    def guard(work):
+        try:
+            work()
+        except Exception as e:   # a thread's exception must fail the test
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=guard, args=(w,)) for w in works]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[:3]
+
+
+def test_destroying_leaves_other_threads_recordings_alone_3d():
+    """A first solve records its cycle; hierarchies destroyed by other threads
+    meanwhile must not spoil the recording."""
+    k = torch.ones((9, 10, 11), device="cuda", dtype=torch.float64)
+    b = torch.ones_like(k)
+    torch.cuda.synchronize()
+
+    def work():
+        s = torch.cuda.Stream()
+        x = torch.zeros_like(b)
+        s.synchronize()
+        for _ in range(60):
+            h = bm.setup3(k, stream=s)
+            h.solve(b, x=x, tol=1e-6, stream=s)
+            h.destroy()
+
+    run_threads([work] * 4)
+
+
+def test_destroying_leaves_other_threads_recordings_alone_2d():
+    """A hierarchy whose recording failed would launch its cycles one by one:
+    many kernel launches in every later solve, where the recorded loop has a
+    few."""
+    k = torch.ones((100, 90), device="cuda", dtype=torch.float64)
+    b = torch.ones_like(k)
+    torch.cuda.synchronize()
+    kept, done = [], threading.Event()
+
+    def make():
+        s = torch.cuda.Stream()
+        x = torch.zeros_like(b)
+        s.synchronize()
+        try:
+            for _ in range(60):
+                h = bm.setup(k, stream=s)
+                h.solve(b, x=x, tol=1e-10, stream=s)
+                kept.append(h)
+        finally:
+            done.set()
+
+    def churn():
+        s = torch.cuda.Stream()
+        while not done.is_set():
+            bm.setup(k, stream=s).destroy()
+
+    run_threads([make, churn, churn])
+    counts = set()
+    for h in kept:
+        before = bm.kernel_launches()
+        h.solve(b, tol=1e-10)
+        counts.add(bm.kernel_launches() - before)
+        h.destroy()
+    assert len(counts) == 1 and max(counts) < 12, counts
+
+
+def test_destroy_waits_for_the_work_a_call_left():
+    """The single operations return with their work under way; a hierarchy
+    destroyed then keeps its memory until they are done, on either of two
+    streams, whoever asks for memory next."""
+    n = 2000
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    k = 10.0 ** torch.rand((n, n), generator=g, device="cuda", dtype=torch.float64)
+    b = torch.rand((n, n), generator=g, device="cuda", dtype=torch.float64)
+    h = bm.setup(k)
+    want = h.op_relax(h.nlevels - 1, torch.zeros_like(b), b, 60)
+    torch.cuda.synchronize()
+    h.destroy()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for s in streams * 2:
+        h = bm.setup(k)
+        x = torch.zeros_like(b)
+        torch.cuda.synchronize()
+        r = torch.empty((n // 2, n // 2), device="cuda", dtype=torch.float64)
+        h.op_restrict(h.nlevels - 1, b, r, stream=streams[0])
+        h.op_relax(h.nlevels - 1, x, b, 60, stream=s)
+        h.destroy()
+        bm.setup(k * 2.0, stream=streams[1 if s is streams[0] else 0]).destroy()
+        torch.cuda.synchronize()
+        assert torch.equal(x, want)
