@@ -519,8 +519,7 @@ template <int NS, int TX, int TY, int NT>
 void launch_bdown(const BClass& c, const Scalars* sc, cudaStream_t s) {
   constexpr size_t s9 = DownLeg<float, true, NS, TX, TY>::SMEM, s5 = DownLeg<float, false, NS, TX, TY>::SMEM;
   constexpr size_t smem = s9 > s5 ? s9 : s5;
-  static const bool ready = use_shared(k_bdown<NS, TX, TY, NT>, smem);
-  (void)ready;
+  use_shared(k_bdown<NS, TX, TY, NT>, smem);
   launch_pdl(k_bdown<NS, TX, TY, NT>, dim3(cdiv(c.n, TX), cdiv(c.n, TY), c.count), dim3(NT), smem, s,
              (const LevelV<float>*)c.view[0], (const LevelV<float>*)c.coarse, (const int*)c.pids, sc);
   count_launch();
@@ -529,8 +528,7 @@ template <int TX, int TY, int NT>
 void launch_bup(const BClass& c, const Scalars* sc, cudaStream_t s) {
   constexpr size_t s9 = UpLeg<float, true, TX, TY, false>::SMEM, s5 = UpLeg<float, false, TX, TY, false>::SMEM;
   constexpr size_t smem = s9 > s5 ? s9 : s5;
-  static const bool ready = use_shared(k_bup<TX, TY, NT>, smem);
-  (void)ready;
+  use_shared(k_bup<TX, TY, NT>, smem);
   launch_pdl(k_bup<TX, TY, NT>, dim3(cdiv(c.n, TX), cdiv(c.n, TY), c.count), dim3(NT), smem, s,
              (const LevelV<float>*)c.view[0], (const LevelV<float>*)c.coarse, (const int*)c.pids, sc);
   count_launch();

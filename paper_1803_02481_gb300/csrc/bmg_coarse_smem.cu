@@ -610,10 +610,8 @@ size_t layout(const Hierarchy* h, int thr, SmArgs<T>& a) {
 }
 
 template <typename T>
-void prepare() {
-  static const bool done =
-      use_shared(k_coarse_smem<T, true>, kCoarseImageMax) && use_shared(k_coarse_smem<T, false>, kCoarseImageMax);
-  (void)done;
+bool prepare() {
+  return use_shared(k_coarse_smem<T, true>, kCoarseImageMax) && use_shared(k_coarse_smem<T, false>, kCoarseImageMax);
 }
 
 template <typename T>
@@ -633,12 +631,10 @@ bool coarse_smem_fits(const Hierarchy* h, int thr) {
   if (thr == h->L && h->opt.precision != BMG_FP32_REFINE && h->d.back().PR[PR_B]) return false;
   if (h->opt.precision == BMG_FP32_REFINE) {
     SmArgs<float> a{};
-    prepare<float>();
-    return layout<float>(h, thr, a) > 0;
+    return layout<float>(h, thr, a) > 0 && prepare<float>();
   }
   SmArgs<double> a{};
-  prepare<double>();
-  return layout<double>(h, thr, a) > 0;
+  return layout<double>(h, thr, a) > 0 && prepare<double>();
 }
 
 int launch_coarse_image(Hierarchy* h, cudaStream_t s) {
@@ -686,8 +682,7 @@ size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned
 }
 
 void launch_coarse_smem_batch(const void* args, int count, size_t bytes, const Scalars* sc, cudaStream_t s) {
-  static const bool ready = use_shared(k_coarse_smem_batch, kCoarseImageMax);
-  (void)ready;
+  use_shared(k_coarse_smem_batch, kCoarseImageMax);
   launch_pdl(k_coarse_smem_batch, dim3(unsigned(count)), dim3(kNT), bytes, s,
              static_cast<const SmArgs<float>*>(args), sc);
   count_launch();

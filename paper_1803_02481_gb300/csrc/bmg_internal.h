@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "../../include/boxmg.h"
+#include "bmg_optin.h"
 
 namespace bmg {
 
@@ -135,18 +136,29 @@ __device__ __forceinline__ void griddep_launch() {
 }
 bool pdl_enabled();
 
-// Opts a kernel into `bytes` of dynamic shared memory and asks for the whole
+// Opts a kernel into `bytes` of dynamic shared memory on the current device
+// (see SharedOptIn); whether it has them.  use_shared also asks for the whole
 // of the unified L1 as shared memory: with the default carve-out the driver
 // made room for one block of the kernels here, and they ran at one block per
 // SM (measured).
+inline SharedOptIn& shared_opt_in() {
+  static SharedOptIn* s = new SharedOptIn;   // (outlives every static object)
+  return *s;
+}
+template <typename... KArgs>
+inline bool allow_shared(void (*kern)(KArgs...), size_t bytes, bool carveout = false) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  return shared_opt_in().ensure(reinterpret_cast<const void*>(kern), dev, bytes, [&](size_t n) {
+    return (n <= 48 * 1024 ||
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(n)) == cudaSuccess) &&
+           (!carveout || cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                              int(cudaSharedmemCarveoutMaxShared)) == cudaSuccess);
+  });
+}
 template <typename... KArgs>
 inline bool use_shared(void (*kern)(KArgs...), size_t bytes) {
-  const bool a = bytes <= 48 * 1024 ||
-                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)) ==
-                     cudaSuccess;
-  const bool b = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      int(cudaSharedmemCarveoutMaxShared)) == cudaSuccess;
-  return a && b;
+  return allow_shared(kern, bytes, true);
 }
 
 template <typename... KArgs, typename... Args>

@@ -42,8 +42,7 @@ __global__ void __launch_bounds__(NT) k_up(LevelV<T> F, const T* __restrict__ xi
 template <typename T, bool NINE, int NS, bool ZERO, int TX, int TY, int NT>
 void down_shape(const LevelV<T>& F, const T* xin, T* xout, const LevelV<T>& Cc, cudaStream_t s) {
   constexpr size_t smem = DownLeg<T, NINE, NS, TX, TY>::SMEM;
-  static const bool ready = use_shared(k_down<T, NINE, NS, ZERO, TX, TY, NT>, smem);
-  (void)ready;
+  use_shared(k_down<T, NINE, NS, ZERO, TX, TY, NT>, smem);
   launch_pdl(k_down<T, NINE, NS, ZERO, TX, TY, NT>, dim3(cdiv(F.nx, TX), cdiv(F.ny, TY)), dim3(NT), smem,
              s, F, xin, xout, Cc);
 }
@@ -52,8 +51,7 @@ template <typename T, bool NINE, int TX, int TY, int NT, bool NRM>
 void up_shape(const LevelV<T>& F, const T* xin, const T* xc, T* xout, T* xnext, double* partials,
               cudaStream_t s) {
   constexpr size_t smem = UpLeg<T, NINE, TX, TY, NRM>::SMEM;
-  static const bool ready = use_shared(k_up<T, NINE, TX, TY, NT, NRM>, smem);
-  (void)ready;
+  use_shared(k_up<T, NINE, TX, TY, NT, NRM>, smem);
   launch_pdl(k_up<T, NINE, TX, TY, NT, NRM>, dim3(cdiv(F.nx, TX), cdiv(F.ny, TY)), dim3(NT), smem, s, F,
              xin, xc, xout, xnext, partials);
 }

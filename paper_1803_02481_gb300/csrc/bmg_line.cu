@@ -522,8 +522,7 @@ bool launch_line_step_c(const LevelV<T>& L, int colour, const T* xs, T* xo, cuda
   const LineGeo g = line_geo<DIR>(L);
   const size_t smem = StepSmem<T, DIR, C>(g.n, L.sgl[DIR]).bytes();
   if (smem > kStepSmem) return false;
-  static const bool ready = use_shared(k_line_step<T, DIR, NINE, C, NT, MINB>, kStepSmem);
-  if (!ready) return false;
+  if (!use_shared(k_line_step<T, DIR, NINE, C, NT, MINB>, kStepSmem)) return false;
   launch_pdl(k_line_step<T, DIR, NINE, C, NT, MINB>, dim3(cdiv(line_count(g.nl, colour), C)), dim3(NT), smem, s, L,
              colour, xs, xo);
   count_launch();
@@ -712,13 +711,7 @@ void line_step(const LevelV<T>& L, int colour, const T* xs, T* xo, cudaStream_t 
 
 template <typename T>
 int launch_line_factor(const LevelV<T>& L, int smoother, int* derr, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_line_blocks_x<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(xblocks_smem<T>())) != cudaSuccess)
-      return BMG_ECUDA;
-    attr = true;
-  }
+  if (!allow_shared(k_line_blocks_x<T>, xblocks_smem<T>())) return BMG_ECUDA;
   auto one = [&](auto dir_tag) {
     constexpr int DIR = decltype(dir_tag)::value;
     const LineGeo g = line_geo<DIR>(L);

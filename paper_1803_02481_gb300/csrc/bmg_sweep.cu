@@ -290,9 +290,8 @@ static void launch_tma_shape(const LevelV<T>& L, const SweepMaps<T>& m, const CU
 template <typename T, bool NINE, int TX, int TY, int NT, int MINB, int NSTAGE, bool PRE = false,
           bool NRM = false, bool ZERO = false>
 static void allow_tma_smem() {
-  cudaFuncSetAttribute(k_sweep_tma<T, NINE, TX, TY, NT, MINB, NSTAGE, PRE, NRM, ZERO>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       int(TmaTile<T, NINE, TX, TY, NSTAGE, PRE>::SMEM));
+  allow_shared(k_sweep_tma<T, NINE, TX, TY, NT, MINB, NSTAGE, PRE, NRM, ZERO>,
+               TmaTile<T, NINE, TX, TY, NSTAGE, PRE>::SMEM);
   tma_resident<T, NINE, TX, TY, NT, MINB, NSTAGE, PRE, NRM, ZERO>();
 }
 
@@ -495,46 +494,38 @@ void launch_sweep(const LevelV<T>& L, bool nine, bool reverse, const T* xin, T* 
 }
 
 // Opt the streaming kernels into more than 48 KB of dynamic shared memory
-// (once per process, before any launch or graph capture).
+// on the current device (every setup, before any launch or graph capture).
 void prepare_sweep_kernels() {
-  static const bool done = [] {
-    using S64 = StreamRB<double, kStreamNT, kStreamR>;
-    using S32 = StreamRB<float, kStreamNT, kStreamR>;
-    cudaFuncSetAttribute(k_sweep_rb_stream<double, kStreamNT, kStreamR>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         int(sizeof(S64::Row) * S64::NSLOT));
-    cudaFuncSetAttribute(k_sweep_rb_stream<float, kStreamNT, kStreamR>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         int(sizeof(S32::Row) * S32::NSLOT));
+  using S64 = StreamRB<double, kStreamNT, kStreamR>;
+  using S32 = StreamRB<float, kStreamNT, kStreamR>;
+  allow_shared(k_sweep_rb_stream<double, kStreamNT, kStreamR>, sizeof(S64::Row) * S64::NSLOT);
+  allow_shared(k_sweep_rb_stream<float, kStreamNT, kStreamR>, sizeof(S32::Row) * S32::NSLOT);
 #define BMG_TMA_ALLOW(TT, NN, TX, TY, NT, MB, NS) allow_tma_smem<TT, NN, TX, TY, NT, MB, NS>()
 #define BMG_TMA_ALLOW_Z(TT, NN, TX, TY, NT, MB, NS) \
   allow_tma_smem<TT, NN, TX, TY, NT, MB, NS, false, false, true>()
-    BMG_TMA_DISPATCH(double, false, rb_cfg_index(), BMG_TMA_ALLOW);
-    BMG_TMA_DISPATCH(float, false, rb_cfg_index(), BMG_TMA_ALLOW);
-    BMG_TMA_DISPATCH(double, true, nine_cfg_index(), BMG_TMA_ALLOW);
-    BMG_TMA_DISPATCH(float, true, nine_cfg_index(), BMG_TMA_ALLOW);
-    BMG_TMA_DISPATCH(double, false, rb_cfg_index(), BMG_TMA_ALLOW_Z);
-    BMG_TMA_DISPATCH(float, false, rb_cfg_index(), BMG_TMA_ALLOW_Z);
-    BMG_TMA_DISPATCH(double, true, nine_cfg_index(), BMG_TMA_ALLOW_Z);
-    BMG_TMA_DISPATCH(float, true, nine_cfg_index(), BMG_TMA_ALLOW_Z);
+  BMG_TMA_DISPATCH(double, false, rb_cfg_index(), BMG_TMA_ALLOW);
+  BMG_TMA_DISPATCH(float, false, rb_cfg_index(), BMG_TMA_ALLOW);
+  BMG_TMA_DISPATCH(double, true, nine_cfg_index(), BMG_TMA_ALLOW);
+  BMG_TMA_DISPATCH(float, true, nine_cfg_index(), BMG_TMA_ALLOW);
+  BMG_TMA_DISPATCH(double, false, rb_cfg_index(), BMG_TMA_ALLOW_Z);
+  BMG_TMA_DISPATCH(float, false, rb_cfg_index(), BMG_TMA_ALLOW_Z);
+  BMG_TMA_DISPATCH(double, true, nine_cfg_index(), BMG_TMA_ALLOW_Z);
+  BMG_TMA_DISPATCH(float, true, nine_cfg_index(), BMG_TMA_ALLOW_Z);
 #undef BMG_TMA_ALLOW_Z
 #undef BMG_TMA_ALLOW
 #define BMG_TMA_PRE_ALLOW(TX, TY, NT, MB, NS) allow_tma_smem<double, false, TX, TY, NT, MB, NS, true>()
-    BMG_TMA_PRE_DISPATCH(pre_cfg_index(), BMG_TMA_PRE_ALLOW);
+  BMG_TMA_PRE_DISPATCH(pre_cfg_index(), BMG_TMA_PRE_ALLOW);
 #undef BMG_TMA_PRE_ALLOW
 #define BMG_TMA_PRE_NORM_ALLOW(TX, TY, NT, MB, NS) \
   allow_tma_smem<double, false, TX, TY, NT, MB, NS, true, true>()
-    BMG_TMA_PRE_DISPATCH(pre_cfg_index(), BMG_TMA_PRE_NORM_ALLOW);
+  BMG_TMA_PRE_DISPATCH(pre_cfg_index(), BMG_TMA_PRE_NORM_ALLOW);
 #undef BMG_TMA_PRE_NORM_ALLOW
 #define BMG_TMA_PRE_ZERO_ALLOW(TX, TY, NT, MB, NS) \
   allow_tma_smem<double, false, TX, TY, NT, MB, NS, true, false, true>()
-    BMG_TMA_PRE_DISPATCH(pre_cfg_index(), BMG_TMA_PRE_ZERO_ALLOW);
+  BMG_TMA_PRE_DISPATCH(pre_cfg_index(), BMG_TMA_PRE_ZERO_ALLOW);
 #undef BMG_TMA_PRE_ZERO_ALLOW
-    sm_count();
-    encode_tiled();
-    return true;
-  }();
-  (void)done;
+  sm_count();
+  encode_tiled();
 }
 
 // Failure-detection self-test: one thread waits, with the bounded wait of

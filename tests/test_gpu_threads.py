@@ -106,3 +106,19 @@ def test_destroy_waits_for_the_work_a_call_left():
         bm.setup(k * 2.0, stream=streams[1 if s is streams[0] else 0]).destroy()
         torch.cuda.synchronize()
         assert torch.equal(x, want)
+def test_setups_of_different_coarsest_sizes_at_once():
+    """The coarsest factorisation takes shared memory by its size: 81 to 159
+    unknowns, all above the 48 KB a kernel has without asking."""
+    ks = [torch.ones((3, n), device="cuda", dtype=torch.float64) for n in (27, 35, 45, 53)]
+    torch.cuda.synchronize()
+
+    def work(turn):
+        def run():
+            s = torch.cuda.Stream()
+            for r in range(250):
+                bm.setup(ks[(r + turn) % len(ks)], stream=s).destroy()
+        return run
+
+    run_threads([work(t) for t in range(4)])
+
+
