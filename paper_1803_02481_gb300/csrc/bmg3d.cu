@@ -1185,6 +1185,14 @@ void enqueue_vcycle3(bmg3_hierarchy* h, std::vector<Lev3T<T>>& lv, cudaStream_t 
 
 // FP32 refinement: the residual of the current x as the next FP32
 // right-hand side, and its norm (the stop test).
+// The solve's scalars into their pinned mirror.
+void scalars_to_host(bmg3_hierarchy* h, cudaStream_t s) {
+  if (bmg::GraphRecorder* r = bmg::recorder())
+    r->copy_to_host(h->sc_host, h->sc, sizeof(Scal3));
+  else
+    cudaMemcpyAsync(h->sc_host, h->sc, sizeof(Scal3), cudaMemcpyDeviceToHost, s);
+}
+
 void enqueue_refine_residual(bmg3_hierarchy* h, cudaStream_t s) {
   bmg::launch_pdl(k3_refine_residual, dim3(kNormBlocks), dim3(kNormThreads), 0, s, h->lv[h->L - 1], h->lv32[h->L - 1], h->sc, h->partials);
   bmg::launch_pdl(k3_refine_norm_final, dim3(1), dim3(kNormThreads), 0, s, h->partials, kNormBlocks, h->sc);
@@ -1210,7 +1218,7 @@ void enqueue_step(bmg3_hierarchy* h, cudaStream_t s) {
     bmg::launch_pdl(k3_norm_final, dim3(1), dim3(kNormThreads), 0, s, h->partials, kNormBlocks, h->sc, 1);
     count_launch(2);
   }
-  cudaMemcpyAsync(h->sc_host, h->sc, sizeof(Scal3), cudaMemcpyDeviceToHost, s);
+  scalars_to_host(h, s);
 }
 
 // The finest level's first pre-smoothing sweep (two colour launches, in
@@ -1237,7 +1245,7 @@ void enqueue_fused_step(bmg3_hierarchy* h, double* in, double* out, cudaStream_t
   bmg::launch_pdl(k3_norm_final, dim3(1), dim3(kNormThreads), 0, s, h->partials, kNormBlocks, h->sc, 1);
   bmg::prof_end(BMG_PROF_NORM, s);
   count_launch(2);
-  cudaMemcpyAsync(h->sc_host, h->sc, sizeof(Scal3), cudaMemcpyDeviceToHost, s);
+  scalars_to_host(h, s);
 }
 
 // z = M^{-1} r: one V-cycle on the residual held in the finest level's b
@@ -1270,19 +1278,19 @@ void enqueue_pcg_iter(bmg3_hierarchy* h, bool first, cudaStream_t s) {
   bmg::launch_pdl(k3_pcg_xr, dim3(kNormBlocks), dim3(kNormThreads), 0, s, F, h->pX, h->pP, h->pQ, h->sc, h->partials);
   bmg::launch_pdl(k3_norm_final, dim3(1), dim3(kNormThreads), 0, s, h->partials, kNormBlocks, h->sc, 1);
   count_launch(7);
-  cudaMemcpyAsync(h->sc_host, h->sc, sizeof(Scal3), cudaMemcpyDeviceToHost, s);
+  scalars_to_host(h, s);
 }
 
-// Records fn(stream) as a graph (on a private stream) and instantiates it.
+// Records fn(stream) as a graph and instantiates it.
 template <class Fn>
 bool record_graph(cudaGraph_t* g, cudaGraphExec_t* e, Fn fn) {
-  cudaStream_t cs;
-  if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return false;
-  bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-  if (ok) fn(cs);
-  ok = cudaStreamEndCapture(cs, g) == cudaSuccess && ok;
+  bool ok = cudaGraphCreate(g, 0) == cudaSuccess;
+  if (ok) {
+    bmg::GraphRecorder rec(*g);
+    fn(cudaStream_t(nullptr));
+    ok = rec.ok();
+  }
   ok = ok && cudaGraphInstantiate(e, *g, 0) == cudaSuccess;
-  cudaStreamDestroy(cs);
   if (!ok) cudaGetLastError();
   return ok;
 }
@@ -1638,21 +1646,11 @@ static int solve3(bmg3_hierarchy* h, const double* b, double* x, double tol, bmg
     k3_unpack<<<g, kT, 0, s>>>(cycles == 0 ? F.x : buf[(cycles - 1) & 1], x, F);
     count_launch();
   } else {
-    // one cycle as a graph, recorded on a private stream (stream launches
-    // while kernel classes are being timed)
+    // one cycle as a graph (stream launches while kernel classes are being
+    // timed)
     const bool use_graph = !bmg::prof_active();
     if (use_graph && !h->gexec) {
-      cudaStream_t cs;
-      if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return BMG_ECUDA;
-      bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-      if (ok) enqueue_step(h, cs);
-      ok = cudaStreamEndCapture(cs, &h->graph) == cudaSuccess && ok;
-      ok = ok && cudaGraphInstantiate(&h->gexec, h->graph, 0) == cudaSuccess;
-      cudaStreamDestroy(cs);
-      if (!ok) {
-        cudaGetLastError();
-        return BMG_ECUDA;
-      }
+      if (!record_graph(&h->graph, &h->gexec, [&](cudaStream_t cs) { enqueue_step(h, cs); })) return BMG_ECUDA;
     }
     // FP32 refinement: the first right-hand side is the initial residual
     if (h->refine && rel > tol && h->opt.max_cycles > 0) enqueue_refine_residual(h, s);

@@ -585,12 +585,10 @@ static int read_scalars(Hierarchy* h, cudaStream_t s) {
   return BMG_OK;
 }
 
-// Record the solve loop of h as one graph (see Hierarchy::graph).  Recording
-// runs on a private stream (the caller's may be the legacy default stream,
-// which cannot capture) and executes nothing.
+// Record the solve loop of h as one graph (see Hierarchy::graph); nothing is
+// executed.
 static int build_solve_graph(Hierarchy* h) {
-  cudaStream_t s = nullptr;
-  if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return BMG_ECUDA;
+  const cudaStream_t s = nullptr;   // (not used while recording)
   const bool fp32 = h->opt.precision == BMG_FP32_REFINE;
   const bool pcg = h->opt.solver == BMG_SOLVER_PCG;
   const bool fused = !pcg && !fp32 && fused_norm_on(h);
@@ -643,41 +641,23 @@ static int build_solve_graph(Hierarchy* h) {
     if (cudaGraphConditionalHandleCreate(&h->cond, h->graph, 0, cudaGraphCondAssignDefault) !=
         cudaSuccess)
       break;
-    if (cudaStreamBeginCaptureToGraph(s, h->graph, nullptr, nullptr, 0,
-                                      cudaStreamCaptureModeRelaxed) != cudaSuccess)
-      break;
-    prologue();
-    cudaStreamCaptureStatus st;
-    const cudaGraphNode_t* deps = nullptr;
-    size_t ndeps = 0;
-    if (cudaStreamGetCaptureInfo(s, &st, nullptr, nullptr, &deps, nullptr, &ndeps) != cudaSuccess)
-      break;
-    alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)];
-    std::memset(raw, 0, sizeof(raw));
-    cudaGraphNodeParams& cp = *reinterpret_cast<cudaGraphNodeParams*>(raw);
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h->cond;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t node;
-    if (cudaGraphAddNode(&node, h->graph, deps, nullptr, ndeps, &cp) != cudaSuccess) break;
-    if (cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1,
-                                            cudaStreamSetCaptureDependencies) != cudaSuccess)
-      break;
-    cudaGraph_t g = nullptr;
-    if (cudaStreamEndCapture(s, &g) != cudaSuccess) break;
-    cudaGraph_t gbody = cp.conditional.phGraph_out[0];
-    if (cudaStreamBeginCaptureToGraph(s, gbody, nullptr, nullptr, 0,
-                                      cudaStreamCaptureModeRelaxed) != cudaSuccess)
-      break;
-    body();
-    if (cudaStreamEndCapture(s, &g) != cudaSuccess) break;
+    cudaGraph_t loop = nullptr;
+    {
+      GraphRecorder rec(h->graph);
+      prologue();
+      loop = rec.loop(h->cond);
+      if (!rec.ok()) break;
+    }
+    {
+      GraphRecorder rec(loop);
+      body();
+      if (!rec.ok()) break;
+    }
     if (cudaGraphInstantiate(&h->gexec, h->graph, 0) != cudaSuccess) break;
     rc = BMG_OK;
   } while (0);
   for (size_t l = 0; l < h->d.size(); ++l) std::tie(h->d[l].x, h->d[l].x2) = roles64[l];
   for (size_t l = 0; l < h->f.size(); ++l) std::tie(h->f[l].x, h->f[l].x2) = roles32[l];
-  cudaStreamDestroy(s);
   if (rc != BMG_OK) {
     cudaGetLastError();
     if (h->graph) cudaGraphDestroy(h->graph);

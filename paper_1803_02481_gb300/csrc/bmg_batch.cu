@@ -393,9 +393,9 @@ void launch_bsweep(int variant, bool nine, int n, int count, const LevelV<float>
   do {                                                                                  \
     const dim3 grid(cdiv(n, TX), cdiv(n, TY), count);                                   \
     if (nine)                                                                           \
-      k_bsweep<true, TX, TY, NT><<<grid, NT, 0, s>>>(views, pids, sc, order);           \
+      launch_plain(k_bsweep<true, TX, TY, NT>, grid, dim3(NT), 0, s, views, pids, sc, order);  \
     else                                                                                \
-      k_bsweep<false, TX, TY, NT><<<grid, NT, 0, s>>>(views, pids, sc, order);          \
+      launch_plain(k_bsweep<false, TX, TY, NT>, grid, dim3(NT), 0, s, views, pids, sc, order); \
   } while (0)
   switch (variant) {
     case 0: BMG_BSWEEP(32, 16, 128); break;
@@ -575,12 +575,12 @@ void enqueue_bvcycle(Batch* b, cudaStream_t s) {
     }
     const dim3 g(cdiv(c.n, 128), c.n, c.count);
     if (c.nine)
-      k_bresid<true><<<g, 128, 0, s>>>(c.view[par], c.pids, b->sc);
+      launch_plain(k_bresid<true>, g, dim3(128), 0, s, c.view[par], c.pids, b->sc);
     else
-      k_bresid<false><<<g, 128, 0, s>>>(c.view[par], c.pids, b->sc);
+      launch_plain(k_bresid<false>, g, dim3(128), 0, s, c.view[par], c.pids, b->sc);
     const int nc = (c.n - 1) / 2;
-    k_brestrict<<<dim3(cdiv(nc, 128), nc, c.count), 128, 0, s>>>(c.view[par], c.coarse, c.pids,
-                                                                  b->sc);
+    launch_plain(k_brestrict, dim3(cdiv(nc, 128), nc, c.count), dim3(128), 0, s, c.view[par], c.coarse, c.pids,
+                 b->sc);
     count_launch(2);
     c.parity_after_pre = par;
   }
@@ -588,8 +588,8 @@ void enqueue_bvcycle(Batch* b, cudaStream_t s) {
   for (auto it = b->cls.rbegin(); it != b->cls.rend(); ++it) {
     BClass& c = *it;
     int par = c.parity_after_pre;
-    k_binterp<<<dim3(cdiv(c.n, 128), c.n, c.count), 128, 0, s>>>(c.view[par], c.coarse, c.pids,
-                                                                  b->sc, oop ? 1 : 0);
+    launch_plain(k_binterp, dim3(cdiv(c.n, 128), c.n, c.count), dim3(128), 0, s, c.view[par], c.coarse, c.pids,
+                 b->sc, oop ? 1 : 0);
     count_launch();
     if (oop) par ^= 1;
     for (int k = 0; k < nu2; ++k) {
@@ -703,51 +703,32 @@ int autotune(Batch* b, cudaStream_t s) {
   return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ECUDA;
 }
 
-int build_graph_on(Batch* b, cudaStream_t s);
-
 // The refinement loop as one graph: WHILE(any active) { V-cycle; update;
 // residuals + stop tests + any }, or (BMG_SOLVER_PCG) WHILE(any active) {
-// one PCG iteration }.  Recorded on a private stream (the
-// caller's stream may be the legacy default stream, which cannot capture);
-// recording executes nothing.
+// one PCG iteration }.  Recording executes nothing.
 int build_graph(Batch* b) {
-  cudaStream_t s = nullptr;
-  if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return BMG_ECUDA;
-  const int rc = build_graph_on(b, s);
-  cudaStreamDestroy(s);
-  return rc;
-}
-
-int build_graph_on(Batch* b, cudaStream_t s) {
   if (cudaGraphCreate(&b->graph, 0) != cudaSuccess) return BMG_ECUDA;
   if (cudaGraphConditionalHandleCreate(&b->handle, b->graph, 1, cudaGraphCondAssignDefault) !=
       cudaSuccess)
     return BMG_ECUDA;
-  // zeroed storage: the struct's unions have no default constructor
-  alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)];
-  std::memset(raw, 0, sizeof(raw));
-  cudaGraphNodeParams& cp = *reinterpret_cast<cudaGraphNodeParams*>(raw);
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = b->handle;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t node;
-  if (cudaGraphAddNode(&node, b->graph, nullptr, nullptr, 0, &cp) != cudaSuccess) return BMG_ECUDA;
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  if (cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) !=
-      cudaSuccess)
-    return BMG_ECUDA;
-  if (b->opt.solver == BMG_SOLVER_PCG) {
-    enqueue_pcg_iter(b, true, s);
-  } else {
-    enqueue_bvcycle(b, s);
-    enqueue_update(b, s);
-    enqueue_residuals(b, 1, true, s);
+  cudaGraph_t body = nullptr;
+  {
+    GraphRecorder rec(b->graph);
+    body = rec.loop(b->handle);
   }
-  cudaGraph_t out = nullptr;
-  if (cudaStreamEndCapture(s, &out) != cudaSuccess) return BMG_ECUDA;
-  if (cudaGraphInstantiate(&b->exec, b->graph, 0) != cudaSuccess) return BMG_ECUDA;
-  return BMG_OK;
+  if (!body) return BMG_ECUDA;
+  {
+    GraphRecorder rec(body);
+    if (b->opt.solver == BMG_SOLVER_PCG) {
+      enqueue_pcg_iter(b, true, nullptr);
+    } else {
+      enqueue_bvcycle(b, nullptr);
+      enqueue_update(b, nullptr);
+      enqueue_residuals(b, 1, true, nullptr);
+    }
+    if (!rec.ok()) return BMG_ECUDA;
+  }
+  return cudaGraphInstantiate(&b->exec, b->graph, 0) == cudaSuccess ? BMG_OK : BMG_ECUDA;
 }
 
 double now_ms() {

@@ -190,6 +190,9 @@ __global__ void __launch_bounds__(kCoarseClusterThreads, 1) k_coarse_cycle_clust
 
 template <typename T>
 static cudaError_t launch_cluster_kernel(int ctas, cudaStream_t s, const CoarseArgs<T>& a) {
+  if (GraphRecorder* r = recorder())
+    return record_kernel(r, pdl_enabled(), unsigned(ctas), k_coarse_cycle_cluster<T>, dim3(unsigned(ctas)),
+                         dim3(kCoarseClusterThreads), 0, a);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(ctas));
   cfg.blockDim = dim3(kCoarseClusterThreads);

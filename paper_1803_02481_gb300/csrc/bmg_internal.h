@@ -34,6 +34,7 @@
 #include <cuda_runtime.h>
 #include <cstddef>
 #include <cstdint>
+#include <tuple>
 #include <vector>
 
 #include "../../include/boxmg.h"
@@ -161,9 +162,62 @@ inline bool use_shared(void (*kern)(KArgs...), size_t bytes) {
   return allow_shared(kern, bytes, true);
 }
 
+// While one is alive on a thread, that thread's launches become the nodes of
+// `graph`, each after the one before it, instead of running.  The solve graphs
+// are made this way and not by stream capture, which other threads can spoil:
+// while any stream captures, a wait for the whole device (a call any part of
+// the program may make) is an error, breaks the capture, and at times brought
+// the process down in the driver.
+class GraphRecorder {
+ public:
+  explicit GraphRecorder(cudaGraph_t graph);
+  ~GraphRecorder();
+  GraphRecorder(const GraphRecorder&) = delete;
+  GraphRecorder& operator=(const GraphRecorder&) = delete;
+  // programmatic: the edge from a kernel before it lets this one start early
+  // (launch_pdl); cluster: blocks per cluster.
+  cudaError_t kernel(const void* func, dim3 grid, dim3 block, size_t smem, void** params, bool programmatic,
+                     unsigned cluster = 1);
+  cudaError_t copy_to_host(void* dst, const void* src, size_t bytes);
+  // A WHILE node; the graph of its body (null: it could not be added).
+  cudaGraph_t loop(cudaGraphConditionalHandle handle);
+  bool ok() const { return status_ == cudaSuccess; }
+
+ private:
+  cudaError_t added(cudaGraphNode_t node, cudaError_t e, bool kernel);
+  cudaGraph_t graph_;
+  GraphRecorder* outer_;
+  cudaGraphNode_t last_ = nullptr;
+  bool last_kernel_ = false;
+  cudaError_t status_ = cudaSuccess;
+};
+GraphRecorder* recorder();   // this thread's, or null
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t record_kernel(GraphRecorder* r, bool programmatic, unsigned cluster, void (*kern)(KArgs...),
+                                 dim3 grid, dim3 block, size_t smem, Args... args) {
+  std::tuple<KArgs...> params(args...);
+  return std::apply(
+      [&](auto&... a) {
+        void* p[] = {static_cast<void*>(&a)...};
+        return r->kernel(reinterpret_cast<const void*>(kern), grid, block, smem, p, programmatic, cluster);
+      },
+      params);
+}
+
+// A launch behind everything before it on the stream.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_plain(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                Args... args) {
+  if (GraphRecorder* r = recorder()) return record_kernel(r, false, 1, kern, grid, block, smem, args...);
+  kern<<<grid, block, smem, s>>>(args...);
+  return cudaPeekAtLastError();
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t s, Args... args) {
+  if (GraphRecorder* r = recorder()) return record_kernel(r, pdl_enabled(), 1, kern, grid, block, smem, args...);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -461,8 +515,8 @@ struct Timing;
 // Work on an object's memory that its calls returned from without waiting
 // (the single operations; solves and setups end with a synchronised stream).
 // The memory is handed on only once all of it is done, and that is found out
-// by these events: a wait for the whole device would spoil any recording
-// (stream capture) that another thread has under way.
+// by these events: a wait for the whole device would spoil any stream capture
+// that another thread has under way.
 class Pending {
  public:
   ~Pending();

@@ -55,7 +55,7 @@ bool prof_active() { return prof().mask != 0; }
 
 void prof_begin(int which, cudaStream_t s) {
   Prof& p = prof();
-  if (!(p.mask & (1u << which))) return;
+  if (!(p.mask & (1u << which)) || recorder()) return;   // (nothing runs while a graph is recorded)
   std::lock_guard<std::mutex> g(p.mu);
   ClassRec& c = p.cls[which];
   if (c.open || c.used + 2 > 2 * kMaxPairs) return;
@@ -70,7 +70,7 @@ void prof_begin(int which, cudaStream_t s) {
 
 void prof_end(int which, cudaStream_t s) {
   Prof& p = prof();
-  if (!(p.mask & (1u << which))) return;
+  if (!(p.mask & (1u << which)) || recorder()) return;
   std::lock_guard<std::mutex> g(p.mu);
   ClassRec& c = p.cls[which];
   if (!c.open) return;

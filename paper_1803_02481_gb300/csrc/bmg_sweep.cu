@@ -478,8 +478,8 @@ void launch_sweep(const LevelV<T>& L, bool nine, bool reverse, const T* xin, T* 
       constexpr int NT = kStreamNT, R = kStreamR;
       using S = StreamRB<T, NT, R>;
       const size_t smem = sizeof(typename S::Row) * S::NSLOT;
-      k_sweep_rb_stream<T, NT, R><<<dim3(cdiv(L.nx, S::OWN), cdiv(L.ny, R)), NT, smem, s>>>(
-          L, xin, xout, reverse ? 1 : 0);
+      launch_plain(k_sweep_rb_stream<T, NT, R>, dim3(cdiv(L.nx, S::OWN), cdiv(L.ny, R)), dim3(NT), smem, s, L, xin,
+                   xout, reverse ? 1 : 0);
     } else if (rb_kernel_choice() == 2) {
       constexpr int TX = 128, TY = 32;
       launch_pdl(k_sweep<T, false, TX, TY, 256, 2>, dim3(cdiv(L.nx, TX), cdiv(L.ny, TY)), dim3(256), 0, s, L, xin, xout,

@@ -81,6 +81,51 @@ def test_destroying_leaves_other_threads_recordings_alone_2d():
     assert len(counts) == 1 and max(counts) < 12, counts
 
 
+@pytest.mark.parametrize("kind", ["2d", "refine", "pcg", "lines", "3d", "batch"])
+def test_device_wide_waits_beside_first_solves(kind):
+    """A wait for the whole device, which any part of a program may make at
+    any time, is no concern of a solve that is being recorded: every first
+    solve goes through and gives the same values."""
+    opts = {"2d": {}, "refine": {"precision": bm.BMG_FP32_REFINE}, "pcg": {"solver": bm.BMG_SOLVER_PCG, "nu1": 1},
+            "lines": {"smoother": bm.BMG_SMOOTH_ALTLINE}}.get(kind, {})
+    shape = (17, 18, 19) if kind == "3d" else (63, 63) if kind == "batch" else (70, 90)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(7)
+    k = 10.0 ** torch.rand(shape, generator=g, device="cuda", dtype=torch.float64)
+    b = torch.rand(shape, generator=g, device="cuda", dtype=torch.float64) - 0.5
+    torch.cuda.synchronize()
+
+    def solve(s=None):
+        x = torch.zeros_like(b)
+        torch.cuda.current_stream().synchronize()
+        if kind == "batch":
+            h = bm.Batch([k, k], bm.default_options(), stream=s)
+            y = torch.zeros_like(b)
+            torch.cuda.current_stream().synchronize()
+            h.solve([b, b], [x, y], tol=1e-9, stream=s)
+        else:
+            h = (bm.setup3 if kind == "3d" else bm.setup)(k, bm.default_options(**opts), stream=s)
+            h.solve(b, x=x, tol=1e-9, stream=s)
+        h.destroy()
+        return x
+
+    want, done = solve(), threading.Event()
+
+    def work():
+        s = torch.cuda.Stream()
+        try:
+            for _ in range(40):
+                assert torch.equal(solve(s), want)
+        finally:
+            done.set()
+
+    def wait():
+        while not done.is_set():
+            torch.cuda.synchronize()
+
+    run_threads([work, work, wait])
+
+
 def test_destroy_waits_for_the_work_a_call_left():
     """The single operations return with their work under way; a hierarchy
     destroyed then keeps its memory until they are done, on either of two
