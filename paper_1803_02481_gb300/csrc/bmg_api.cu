@@ -408,7 +408,9 @@ static int level_leg(const Hierarchy* h, const LevelV<T>& V, int l, int ns) {
   if (h->opt.smoother != BMG_SMOOTH_POINT || h->opt.interp_residual_term || h->opt.nu2 != 1 || ns < 1 ||
       ns > 2 || h->by_operation || V.PR[PR_B])
     return 0;
-  return leg_shape(V.nx, V.ny, l != h->L - 1, sizeof(T) == 8);
+  const bool nine = l != h->L - 1;
+  const int shape = leg_shape(V.nx, V.ny, nine, sizeof(T) == 8);
+  return shape && leg_ready<T>(shape, nine) ? shape : 0;
 }
 
 template <typename T>

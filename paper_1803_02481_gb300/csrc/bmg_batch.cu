@@ -515,20 +515,33 @@ void destroy_batch(Batch* b, bool failed = false) {
 template <int TX, int TY>
 int side_tiles(const BClass& c) { return cdiv(c.n, TX) * cdiv(c.n, TY) * c.count; }
 
+// A kernel serves finest and coarse levels; its shared memory is the larger.
+template <int NS, int TX, int TY>
+constexpr size_t bdown_smem() {
+  return std::max(DownLeg<float, true, NS, TX, TY>::SMEM, DownLeg<float, false, NS, TX, TY>::SMEM);
+}
+template <int TX, int TY>
+constexpr size_t bup_smem() {
+  return std::max(UpLeg<float, true, TX, TY, false>::SMEM, UpLeg<float, false, TX, TY, false>::SMEM);
+}
+template <int TX, int TY, int NT>
+bool bleg_ready() {
+  return use_shared(k_bdown<1, TX, TY, NT>, bdown_smem<1, TX, TY>()) &&
+         use_shared(k_bdown<2, TX, TY, NT>, bdown_smem<2, TX, TY>()) &&
+         use_shared(k_bup<TX, TY, NT>, bup_smem<TX, TY>());
+}
+bool blegs_ready() { return bleg_ready<32, 16, 256>() && bleg_ready<16, 8, 128>() && bleg_ready<8, 8, 128>(); }
+
 template <int NS, int TX, int TY, int NT>
 void launch_bdown(const BClass& c, const Scalars* sc, cudaStream_t s) {
-  constexpr size_t s9 = DownLeg<float, true, NS, TX, TY>::SMEM, s5 = DownLeg<float, false, NS, TX, TY>::SMEM;
-  constexpr size_t smem = s9 > s5 ? s9 : s5;
-  use_shared(k_bdown<NS, TX, TY, NT>, smem);
+  constexpr size_t smem = bdown_smem<NS, TX, TY>();
   launch_pdl(k_bdown<NS, TX, TY, NT>, dim3(cdiv(c.n, TX), cdiv(c.n, TY), c.count), dim3(NT), smem, s,
              (const LevelV<float>*)c.view[0], (const LevelV<float>*)c.coarse, (const int*)c.pids, sc);
   count_launch();
 }
 template <int TX, int TY, int NT>
 void launch_bup(const BClass& c, const Scalars* sc, cudaStream_t s) {
-  constexpr size_t s9 = UpLeg<float, true, TX, TY, false>::SMEM, s5 = UpLeg<float, false, TX, TY, false>::SMEM;
-  constexpr size_t smem = s9 > s5 ? s9 : s5;
-  use_shared(k_bup<TX, TY, NT>, smem);
+  constexpr size_t smem = bup_smem<TX, TY>();
   launch_pdl(k_bup<TX, TY, NT>, dim3(cdiv(c.n, TX), cdiv(c.n, TY), c.count), dim3(NT), smem, s,
              (const LevelV<float>*)c.view[0], (const LevelV<float>*)c.coarse, (const int*)c.pids, sc);
   count_launch();
@@ -806,7 +819,8 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
     std::vector<int> pids;
     std::vector<LevelV<float>> v0, v1, vc;
   };
-  b->legs = (opt.nu1 == 1 || opt.nu1 == 2) && opt.nu2 == 1;
+  if (!coarse_smem_batch_ready()) return fail(BMG_ECUDA);
+  b->legs = (opt.nu1 == 1 || opt.nu1 == 2) && opt.nu2 == 1 && blegs_ready();
   std::vector<HostClass> hc;
   for (int m : sides) {
     // legs: one class per side (kind 2); else one per side and kind

@@ -681,8 +681,9 @@ size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned
   return bytes;
 }
 
+bool coarse_smem_batch_ready() { return use_shared(k_coarse_smem_batch, kCoarseImageMax); }
+
 void launch_coarse_smem_batch(const void* args, int count, size_t bytes, const Scalars* sc, cudaStream_t s) {
-  use_shared(k_coarse_smem_batch, kCoarseImageMax);
   launch_pdl(k_coarse_smem_batch, dim3(unsigned(count)), dim3(kNT), bytes, s,
              static_cast<const SmArgs<float>*>(args), sc);
   count_launch();

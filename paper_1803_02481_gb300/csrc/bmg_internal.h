@@ -669,6 +669,8 @@ void prepare_sweep_kernels();
 int leg_shape(int nx, int ny, bool nine, bool fp64);
 int leg_tiles(int shape, int nx, int ny);
 template <typename T>
+bool leg_ready(int shape, bool nine);   // its kernels have their shared memory (asks for it)
+template <typename T>
 void launch_down_leg(const LevelV<T>& F, bool nine, int shape, int ns, bool zero, const T* xin, T* xout,
                      const LevelV<T>& Cc, cudaStream_t s);
 template <typename T>
@@ -730,6 +732,7 @@ void launch_coarse_smem(Hierarchy* h, const LevelV<T>& top, int threshold, bool 
 // `out` and returns the shared memory it needs; `args`: their copies on the device, `sc` the
 // problems' states (go).
 size_t coarse_smem_batch_args(const Hierarchy* h, int* err, std::vector<unsigned char>& out);
+bool coarse_smem_batch_ready();   // the kernel has its shared memory (asks for it)
 void launch_coarse_smem_batch(const void* args, int count, size_t bytes, const Scalars* sc, cudaStream_t s);
 
 // Prescaled finest level (bmg_sweep.cu): whether the finest FP64 level of a

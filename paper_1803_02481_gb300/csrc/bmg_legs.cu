@@ -42,7 +42,6 @@ __global__ void __launch_bounds__(NT) k_up(LevelV<T> F, const T* __restrict__ xi
 template <typename T, bool NINE, int NS, bool ZERO, int TX, int TY, int NT>
 void down_shape(const LevelV<T>& F, const T* xin, T* xout, const LevelV<T>& Cc, cudaStream_t s) {
   constexpr size_t smem = DownLeg<T, NINE, NS, TX, TY>::SMEM;
-  use_shared(k_down<T, NINE, NS, ZERO, TX, TY, NT>, smem);
   launch_pdl(k_down<T, NINE, NS, ZERO, TX, TY, NT>, dim3(cdiv(F.nx, TX), cdiv(F.ny, TY)), dim3(NT), smem,
              s, F, xin, xout, Cc);
 }
@@ -51,7 +50,6 @@ template <typename T, bool NINE, int TX, int TY, int NT, bool NRM>
 void up_shape(const LevelV<T>& F, const T* xin, const T* xc, T* xout, T* xnext, double* partials,
               cudaStream_t s) {
   constexpr size_t smem = UpLeg<T, NINE, TX, TY, NRM>::SMEM;
-  use_shared(k_up<T, NINE, TX, TY, NT, NRM>, smem);
   launch_pdl(k_up<T, NINE, TX, TY, NT, NRM>, dim3(cdiv(F.nx, TX), cdiv(F.ny, TY)), dim3(NT), smem, s, F,
              xin, xc, xout, xnext, partials);
 }
@@ -84,6 +82,20 @@ void up_kind(const LevelV<T>& F, bool nine, const T* xin, const T* xc, T* xout, 
     up_shape<T, false, TX, TY, NT, false>(F, xin, xc, xout, nullptr, nullptr, s);
 }
 
+// The shared memory of a shape's kernels, on the current device.
+template <typename T, bool NINE, int TX, int TY, int NT>
+bool shape_ready() {
+  using D1 = DownLeg<T, NINE, 1, TX, TY>;
+  using D2 = DownLeg<T, NINE, 2, TX, TY>;
+  bool ok = use_shared(k_down<T, NINE, 1, false, TX, TY, NT>, D1::SMEM) &&
+            use_shared(k_down<T, NINE, 1, true, TX, TY, NT>, D1::SMEM) &&
+            use_shared(k_down<T, NINE, 2, false, TX, TY, NT>, D2::SMEM) &&
+            use_shared(k_down<T, NINE, 2, true, TX, TY, NT>, D2::SMEM) &&
+            use_shared(k_up<T, NINE, TX, TY, NT, false>, UpLeg<T, NINE, TX, TY, false>::SMEM);
+  if constexpr (!NINE) ok = ok && use_shared(k_up<T, false, TX, TY, NT, true>, UpLeg<T, false, TX, TY, true>::SMEM);
+  return ok;
+}
+
 }  // namespace
 
 // Which levels take the fused legs, and with which tile.  Every leg is a
@@ -104,6 +116,18 @@ void up_kind(const LevelV<T>& F, bool nine, const T* xin, const T* xc, T* xout, 
 // Launched one operation at a time the same cycles take 106 (255^2), 131
 // (511^2), in FP32 82 and 100.
 enum { LEG_16x8 = 1, LEG_32x16, LEG_8x8 };
+
+template <typename T>
+bool leg_ready(int shape, bool nine) {
+  switch (shape) {
+    case LEG_8x8: return nine ? shape_ready<T, true, 8, 8, 128>() : shape_ready<T, false, 8, 8, 128>();
+    case LEG_16x8: return nine ? shape_ready<T, true, 16, 8, 128>() : shape_ready<T, false, 16, 8, 128>();
+    case LEG_32x16: return nine ? shape_ready<T, true, 32, 16, 256>() : shape_ready<T, false, 32, 16, 256>();
+    default: return false;
+  }
+}
+template bool leg_ready<double>(int, bool);
+template bool leg_ready<float>(int, bool);
 
 int leg_shape(int nx, int ny, bool nine, bool fp64) {
   if (cdiv(nx, 8) * cdiv(ny, 8) <= 304) return LEG_8x8;
