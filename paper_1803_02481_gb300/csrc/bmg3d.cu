@@ -718,6 +718,7 @@ struct Scal3 {
   double rz, alpha, beta;   // PCG scalars
   double rnorm, rinv;       // sqrt(rnorm2) and its inverse (0 for a zero residual)
   int err;                  // E3_* bits set by setup kernels
+  double measure;           // set by the setup (see bmg::CoarseSolve)
 };
 
 __global__ void k3_norm_final(const double* __restrict__ partials, int n, Scal3* sc, int what) {
@@ -967,7 +968,7 @@ __global__ void k3_coarse_factor(Lev3 L0, double* __restrict__ lo, double* __res
 // same kind of factor; entry (r, c) at c * n + r).
 __global__ void __launch_bounds__(128) k3_coarse_inverse(const double* __restrict__ lo,
                                                          const double* __restrict__ idiag, int n,
-                                                         double* __restrict__ inv) {
+                                                         double* __restrict__ inv, double* __restrict__ measure) {
   __shared__ double v[BMG_MAX_COARSEST], y[BMG_MAX_COARSEST];
   const int c = blockIdx.x;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -985,7 +986,7 @@ __global__ void __launch_bounds__(128) k3_coarse_inverse(const double* __restric
     const double xj = y[j] * idiag[j];
     if (threadIdx.x == 0) {
       inv[size_t(c) * n + j] = xj;
-      if (j == c) bmg::raise(inv + size_t(n) * n, xj * idiag[n + c]);
+      if (j == c) bmg::raise(measure, xj * idiag[n + c]);
     }
     for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-lo[size_t(j) * n + i], xj, y[i]);
   }
@@ -998,14 +999,13 @@ __global__ void __launch_bounds__(128) k3_coarse_inverse(const double* __restric
 constexpr int kSolveT = 256;
 template <typename T>
 __global__ void __launch_bounds__(kSolveT) k3_coarse_solve(Lev3T<T> L0, bmg::CoarseSolve s) {
-  __shared__ double v[BMG_MAX_COARSEST];
-  const bool product = bmg::use_inverse(s);   // (constant since the setup)
   griddep_wait();
+  __shared__ double v[BMG_MAX_COARSEST];
   const int nx = L0.nx, ny = L0.ny, n = nx * ny * L0.nz;
   auto at = [&](int r) { return idx3(L0, r % nx + 1, (r / nx) % ny + 1, r / (nx * ny) + 1); };
   for (int r = threadIdx.x; r < n; r += kSolveT) v[r] = double(L0.b[at(r)]);
   __syncthreads();
-  if (!product) {
+  if (!s.product) {
     bmg::substitute(s, v);
     for (int r = threadIdx.x; r < n; r += kSolveT) L0.x[at(r)] = T(v[r]);
     return;
@@ -1057,6 +1057,7 @@ struct bmg3_hierarchy {
   Scal3* sc_host = nullptr;
   int* err = nullptr;
   int n0 = 0;
+  double measure = 0.0;           // see bmg::CoarseSolve
   int gs27_pairs = 1;             // 27-point sweeps as four colour-pair launches (1) or
                                   // eight colour launches (0; environment BMG3_GS27_PAIRS)
   cudaGraph_t graph = nullptr;
@@ -1172,7 +1173,7 @@ void enqueue_vcycle3(bmg3_hierarchy* h, std::vector<Lev3T<T>>& lv, cudaStream_t 
     count_launch(2);
   }
   bmg::launch_pdl(k3_coarse_solve<T>, dim3(1), dim3(kSolveT), 0, s, lv[0],
-                  bmg::CoarseSolve{h->cinv, h->chol, h->chol_idiag, h->n0, L == 1 ? 0.0 : bmg::kInverseLimit});
+                  bmg::CoarseSolve{h->cinv, h->chol, h->chol_idiag, h->n0, bmg::multiplies(L, h->measure)});
   count_launch();
   for (int l = 1; l < L; ++l) {
     bmg::NvtxRange r("interp_leg", l);
@@ -1354,6 +1355,7 @@ int check_err(bmg3_hierarchy* h, cudaStream_t s) {
   if (cudaMemcpyAsync(h->sc_host, h->sc, sizeof(Scal3), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return BMG_ECUDA;
+  h->measure = h->sc_host->measure;
   const int e = h->sc_host->err;
   if (e & E3_BADK) {
     set_last_error("3D setup: a coefficient k is not finite and positive");
@@ -1474,7 +1476,7 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
   }
   const size_t o_chol = reserve(sizeof(double) * size_t(h->n0) * h->n0);
   const size_t o_idiag = reserve(2 * sizeof(double) * h->n0);
-  const size_t o_cinv = reserve(sizeof(double) * (size_t(h->n0) * h->n0 + 1));
+  const size_t o_cinv = reserve(sizeof(double) * size_t(h->n0) * h->n0);
   const size_t o_part = reserve(sizeof(double) * kNormBlocks);
   const size_t o_sc = reserve(sizeof(Scal3));
   h->arena = bmg::pool_alloc(total);
@@ -1555,7 +1557,7 @@ int bmg3_setup(const double* k, int nx, int ny, int nz, const bmg_options* opt_i
     }
   }
   k3_coarse_factor<<<1, 512, 0, s>>>(h->lv[0], h->chol, h->chol_idiag, h->err);
-  k3_coarse_inverse<<<h->n0, 128, 0, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv);
+  k3_coarse_inverse<<<h->n0, 128, 0, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv, &h->sc->measure);
   count_launch(2);
   for (int l = 0; l < int(h->lv32.size()); ++l) {
     const Lev3& V = h->lv[l];

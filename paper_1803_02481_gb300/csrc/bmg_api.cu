@@ -134,6 +134,7 @@ static int check_derr(Hierarchy* h, cudaStream_t s) {
     set_last_error("setup: %s", cudaGetErrorString(cudaGetLastError()));
     return BMG_ECUDA;
   }
+  h->measure = h->sc_host->measure;
   const int e = h->sc_host->err;
   if (e & DEV_BADK) {
     set_last_error("setup: a coefficient k is not finite and positive");
@@ -284,7 +285,7 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt_in, cudaS
     h->kcopy = cv.raw<double>(size_t(nx) * ny);
     h->chol = cv.raw<double>(size_t(h->n0) * h->n0);
     h->chol_idiag = cv.raw<double>(2 * size_t(h->n0));
-    h->cinv = cv.raw<double>(size_t(h->n0) * h->n0 + 1);
+    h->cinv = cv.raw<double>(size_t(h->n0) * h->n0);
     h->partials = cv.raw<double>(h->max_partials);
     h->hist = cv.raw<double>(BMG_MAX_HISTORY);
     h->sc = cv.raw<Scalars>(1);

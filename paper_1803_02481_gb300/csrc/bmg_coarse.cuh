@@ -148,7 +148,7 @@ __device__ void blk_coarse_solve(const LevelV<T>& L0, const CoarseSolve& s) {
   for (int r = threadIdx.x; r < n; r += blockDim.x)
     v[r] = double(L0.b[(r / nx + 1) * L0.pitch + r % nx + 1]);
   __syncthreads();
-  const bool product = use_inverse(s);
+  const bool product = s.product;
   if (!product) substitute(s, v);
   for (int r = threadIdx.x; r < n; r += blockDim.x) {
     auto inv = [&](int c) { return s.inv[size_t(c) * n + r]; };

@@ -391,11 +391,11 @@ __device__ __forceinline__ void up(const Lv& L, const Lv& C, Cell<T>& held, bool
 
 // x_0 = A_0^{-1} b_0 with the stored inverse (the sums of blk_coarse_solve):
 // one unknown per thread, or above kInverseSerial unknowns four lanes for
-// each, one partial sum a lane; or (not `product`) by substitution.
+// each, one partial sum a lane; or by substitution.
 template <typename T>
-__device__ __forceinline__ void solve0(const SmArgs<T>& a, const Lv& L, bool product) {
+__device__ __forceinline__ void solve0(const SmArgs<T>& a, const Lv& L) {
   const int n = a.solve.n, nx = L.nx;
-  if (!product) {
+  if (!a.solve.product) {
     substitute(a.solve, &sh<double>(a.soff));
     for (int r = threadIdx.x; r < n; r += kNT)
       sh<T>(L.x + (r / nx + 1) * L.sp + r % nx + 1) = T(sh<double>(a.soff + r));
@@ -441,7 +441,6 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
   // zero iterates (with their ghosts) and the residuals' ghosts, which the
   // restriction of an even side reads
   for (int e = a.voff[0] + threadIdx.x; e < a.end; e += kNT) sh<T>(e) = T(0);
-  const bool product = use_inverse(a.solve);   // (constant since the setup, like the image)
   __syncthreads();
   Cell<T> held{};
   int mine = 0;                          // OWN: this thread's level
@@ -496,7 +495,7 @@ __device__ __forceinline__ void coarse_smem_body(const SmArgs<T>& a) {
     for (int r = threadIdx.x; r < a.solve.n; r += kNT)
       sh<double>(a.soff + r) = double(sh<T>(L.b + (r / L.nx + 1) * L.sp + r % L.nx + 1));
     __syncthreads();
-    solve0<T>(a, L, product);
+    solve0<T>(a, L);
   }
   __syncthreads();
   for (int l = 1; l <= top; ++l) {

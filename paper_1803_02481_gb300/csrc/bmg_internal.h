@@ -418,15 +418,14 @@ __device__ __forceinline__ T interp_value(T* const* P, int cp, const T* __restri
 // substitutes always: its cycle is this solve alone, and no later one corrects
 // it.
 struct CoarseSolve {
-  const double* inv;     // entry (r, c) at c * n + r; then the measure
+  const double* inv;     // entry (r, c) at c * n + r
   const double* lo;      // Cholesky factor, row-major
   const double* idiag;   // 1 / its diagonal
   int n;
-  double limit;
+  int product;           // multiply by inv, else substitute
 };
 constexpr double kInverseLimit = 1e3;
-
-__device__ __forceinline__ bool use_inverse(const CoarseSolve& s) { return s.inv[size_t(s.n) * s.n] < s.limit; }
+inline int multiplies(int levels, double measure) { return levels > 1 && measure < kInverseLimit; }
 
 // Raises *most to v (> 0; anything else counts as infinite).
 __device__ __forceinline__ void raise(double* most, double v) {
@@ -495,6 +494,7 @@ struct Scalars {            // device-resident solve state
   int max_cycles;
   int go;                   // 1 while the loop should continue
   int err;                  // DevErr bits
+  double measure;           // set by the setup (see CoarseSolve)
 };
 
 // 2-D TMA descriptors of the planes the TMA-staged sweep reads, for one
@@ -547,7 +547,8 @@ struct Hierarchy {
   double* kcopy = nullptr;           // dense (ny, nx) copy of k
   double* chol = nullptr;            // N0 x N0 lower factor (row-major)
   double* chol_idiag = nullptr;      // 1 / L[i][i], then A_0's diagonal
-  double* cinv = nullptr;            // inverse of the coarsest operator and its measure (CoarseSolve)
+  double* cinv = nullptr;            // inverse of the coarsest operator, column by column
+  double measure = 0.0;              // see CoarseSolve
   int n0 = 0;
   double* partials = nullptr;        // reduction scratch
   double* hist = nullptr;            // relative residual per cycle (BMG_MAX_HISTORY)
@@ -618,7 +619,7 @@ int setup_impl(const double* k, int nx, int ny, const bmg_options* opt, cudaStre
 void free_hierarchy(Hierarchy* h);
 
 inline CoarseSolve coarse_solve(const Hierarchy* h) {
-  return CoarseSolve{h->cinv, h->chol, h->chol_idiag, h->n0, h->L == 1 ? 0.0 : kInverseLimit};
+  return CoarseSolve{h->cinv, h->chol, h->chol_idiag, h->n0, multiplies(h->L, h->measure)};
 }
 
 // Kernel launch wrappers (defined in the .cu files).

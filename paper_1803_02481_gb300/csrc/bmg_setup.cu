@@ -433,7 +433,8 @@ __global__ void __launch_bounds__(512) k_coarse_factor(LevelV<T> L0, double* __r
 template <bool SMEM>
 __global__ void __launch_bounds__(128) k_coarse_inverse(const double* __restrict__ lo,
                                                         const double* __restrict__ idiag, int n,
-                                                        double* __restrict__ inv) {
+                                                        double* __restrict__ inv,
+                                                        double* __restrict__ measure) {
   extern __shared__ double dense[];
   const int c = blockIdx.x;
   const int mp = SMEM ? n | 1 : n;
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(128) k_coarse_inverse(const double* __restrict
     const double xj = y[j] * id[j];
     if (threadIdx.x == 0) {
       inv[size_t(c) * n + j] = xj;
-      if (j == c) raise(inv + size_t(n) * n, xj * idiag[n + c]);
+      if (j == c) raise(measure, xj * idiag[n + c]);
     }
     for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-m[size_t(j) * mp + i], xj, y[i]);
   }
@@ -475,10 +476,10 @@ int coarse_factor(Hierarchy* h, const LevelV<T>& l0, cudaStream_t s) {
     if (!use_shared(k_coarse_factor<T, true>, smem) || !use_shared(k_coarse_inverse<true>, smem + vectors))
       return BMG_ECUDA;
     k_coarse_factor<T, true><<<1, 512, smem, s>>>(l0, h->chol, h->chol_idiag, derr);
-    k_coarse_inverse<true><<<h->n0, 128, smem + vectors, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv);
+    k_coarse_inverse<true><<<h->n0, 128, smem + vectors, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv, &h->sc->measure);
   } else {
     k_coarse_factor<T, false><<<1, 512, 0, s>>>(l0, h->chol, h->chol_idiag, derr);
-    k_coarse_inverse<false><<<h->n0, 128, vectors, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv);
+    k_coarse_inverse<false><<<h->n0, 128, vectors, s>>>(h->chol, h->chol_idiag, h->n0, h->cinv, &h->sc->measure);
   }
   count_launch(2);
   return cudaGetLastError() == cudaSuccess ? 0 : BMG_ECUDA;
