@@ -196,8 +196,17 @@ int bmg_solve_host(const double *k_host, const double *b_host, double *x_host,
                    int nx, int ny, const bmg_options *opt, double tol,
                    bmg_info *info, bmg_stream_t stream);
 
-/* Release every device resource of the hierarchy (NULL is allowed). */
+/* Release every device resource of the hierarchy (NULL is allowed).  Waits
+ * for the work that calls on it left under way.  Its device memory is kept
+ * for the next hierarchy (2D or 3D) on the same device, up to 1/32 of the
+ * device's memory in all; it goes back to the driver when that is exceeded,
+ * when an allocation of this library would fail otherwise, and on
+ * bmg_release_memory. */
 void bmg_destroy(bmg_hierarchy *h);
+
+/* Give the memory kept from destroyed hierarchies back to the driver, on every
+ * device, for other allocators of the process to take. */
+void bmg_release_memory(void);
 
 /* ---- Introspection (parity checks against the CPU oracle) ---------------- */
 

@@ -18,7 +18,7 @@ __all__ = [
     "BMG_OK", "BMG_EINVAL", "BMG_ENOMEM", "BMG_ECUDA", "BMG_ENOCONV", "BMG_ENAN", "BMG_ETIMEOUT",
     "BMG_FP64", "BMG_FP32_REFINE", "BoxMGError", "Options", "Info", "lib", "library_path",
     "default_options", "setup", "Hierarchy", "solve_host", "EXPORTED", "EXPORTED3", "setup3",
-    "Hierarchy3", "STENCIL3_OFFSETS",
+    "Hierarchy3", "STENCIL3_OFFSETS", "release_memory",
 ]
 
 BMG_OK, BMG_EINVAL, BMG_ENOMEM, BMG_ECUDA, BMG_ENOCONV, BMG_ENAN, BMG_ETIMEOUT = 0, -1, -2, -3, -4, -5, -6
@@ -70,6 +70,7 @@ EXPORTED = {
     "bmg_solve_host": (_i, [_vp, _vp, _vp, _i, _i, ctypes.POINTER(Options), _d,
                             ctypes.POINTER(Info), _vp]),
     "bmg_destroy": (None, [_vp]),
+    "bmg_release_memory": (None, []),
     "bmg_num_levels": (_i, [_vp, ctypes.POINTER(_i)]),
     "bmg_level_shape": (_i, [_vp, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
     "bmg_level_prescaled": (_i, [_vp, _i, ctypes.POINTER(_i)]),
@@ -137,6 +138,12 @@ def max_coarse_ctas(precision: int = BMG_FP64) -> int:
     out = ctypes.c_int()
     _check(lib().bmg_max_coarse_ctas(int(precision), ctypes.byref(out)), "bmg_max_coarse_ctas")
     return out.value
+
+
+def release_memory() -> None:
+    """Give the device memory kept from destroyed hierarchies (at most 1/32 of
+    the device's) back to the driver."""
+    lib().bmg_release_memory()
 
 
 def kernel_launches() -> int:

@@ -864,10 +864,7 @@ extern "C" int bmg_batch_setup(int nprob, const double* const* k_dev, const int*
   bytes += al(sizeof(Scalars) * nprob) + al(sizeof(double) * b->nunits) + al(sizeof(BProb) * nprob) +
            al(sizeof(BUnit) * b->nunits) + al(sizeof(BSpan) * nprob) + al(cargs_one * nprob) +
            al(2 * sizeof(int)) + al(2 * sizeof(double*) * nprob);
-  if (cudaMalloc(&b->arena, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(BMG_ENOMEM);
-  }
+  if (device_malloc(&b->arena, bytes) != cudaSuccess) return fail(BMG_ENOMEM);
   if (cudaMallocHost(&b->sc_host, sizeof(Scalars) * nprob) != cudaSuccess) return fail(BMG_ENOMEM);
   char* cur = static_cast<char*>(b->arena);
   for (auto& x : hc) {

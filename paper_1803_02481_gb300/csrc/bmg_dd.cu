@@ -202,8 +202,7 @@ int bmg_dd_part_create(int nlev, const int* nx, const int* ny, const int* nine,
   bmg::DDCarver cv;
   bmg::carve(d, cv, nx, ny);
   const size_t bytes = cv.off;
-  if (cudaMalloc(&d->arena, bytes) != cudaSuccess) {
-    cudaGetLastError();
+  if (bmg::device_malloc(reinterpret_cast<void**>(&d->arena), bytes) != cudaSuccess) {
     delete d;
     return BMG_ENOMEM;
   }

@@ -610,6 +610,8 @@ void prof_end(int which, cudaStream_t s);
 // block is under way (else it goes back to the driver, which waits).
 void* pool_alloc(size_t bytes);
 void pool_free(void* p, bool idle);
+// cudaMalloc, tried again without the kept memory where it fails.
+cudaError_t device_malloc(void** p, size_t bytes);
 void* pinned_slot(size_t bytes);
 void pinned_slot_free(void* p);
 

@@ -9,7 +9,8 @@
 //
 //  * Bounded: at most 1/32 of the device's memory is kept per device; the
 //    oldest blocks go back to the driver first, and all of them when an
-//    allocation fails (and the allocation is tried again).
+//    allocation fails (and the allocation is tried again) or the caller asks
+//    (bmg_release_memory).
 //  * A block is kept only if the work on it is done when it is given back (its
 //    owner waits for what it left under way, see Pending), so it does not
 //    matter which streams used it or will use it; any other goes to cudaFree,
@@ -79,6 +80,17 @@ void trim(Pool& P, int dev, size_t most) {
   }
 }
 
+cudaError_t malloc_or_trim(Pool& P, int dev, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    trim(P, dev, 0);
+    e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+  }
+  return e;
+}
+
 }  // namespace
 
 void* pool_alloc(size_t bytes) {
@@ -103,16 +115,18 @@ void* pool_alloc(size_t bytes) {
     return b.p;
   }
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    trim(P, dev, 0);
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-  }
+  if (malloc_or_trim(P, dev, &p, bytes) != cudaSuccess) return nullptr;
   P.live[p] = Block{p, bytes, dev};
   return p;
+}
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  Pool& P = pool();
+  std::lock_guard<std::mutex> g(P.mu);
+  return malloc_or_trim(P, dev, p, bytes);
 }
 
 Pending::~Pending() {
@@ -211,3 +225,14 @@ void pinned_slot_free(void* p) {
 }
 
 }  // namespace bmg
+
+extern "C" void bmg_release_memory(void) {
+  using namespace bmg;
+  Pool& P = pool();
+  std::lock_guard<std::mutex> g(P.mu);
+  int cur = 0;
+  const bool known = cudaGetDevice(&cur) == cudaSuccess;
+  for (auto& kept : P.kept_bytes)
+    if (kept.second > 0 && cudaSetDevice(kept.first) == cudaSuccess) trim(P, kept.first, 0);
+  if (known) cudaSetDevice(cur);
+}

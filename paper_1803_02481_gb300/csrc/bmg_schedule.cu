@@ -266,10 +266,8 @@ int calibrate(cudaStream_t s, double* out) {
   CostParams p = cost_params();
   double* buf = nullptr;
   const size_t stream_elems = size_t(1) << 26;      // 2 x 512 MiB in double
-  if (cudaMalloc(&buf, sizeof(double) * (2 * stream_elems + 1024)) != cudaSuccess) {
-    cudaGetLastError();
+  if (device_malloc(reinterpret_cast<void**>(&buf), sizeof(double) * (2 * stream_elems + 1024)) != cudaSuccess)
     return BMG_ENOMEM;
-  }
   cudaMemsetAsync(buf, 0, sizeof(double) * (2 * stream_elems + 1024), s);
   // launch latency: back-to-back empty launches on the stream
   for (int i = 0; i < 20; ++i) k_empty<<<1, 32, 0, s>>>();

@@ -543,7 +543,7 @@ __global__ void k_selftest_wait(int* __restrict__ err) {
 
 int selftest_bounded_wait(cudaStream_t s) {
   int* d = nullptr;
-  if (cudaMalloc(&d, sizeof(int)) != cudaSuccess) return BMG_ENOMEM;
+  if (device_malloc(reinterpret_cast<void**>(&d), sizeof(int)) != cudaSuccess) return BMG_ENOMEM;
   int h = 0, rc = BMG_ECUDA;
   if (cudaMemsetAsync(d, 0, sizeof(int), s) == cudaSuccess) {
     k_selftest_wait<<<1, 32, 0, s>>>(d);
