@@ -833,7 +833,7 @@ def threshold_sweep(bm, torch, k, b, stream, cycles=20):
     _, info = hc.solve(b, x, tol=1e-30, stream=stream, allow_noconv=True)
     hc.destroy()
     best = min(rows, key=lambda r: r["measured_us_per_cycle"])
-    return {"levels": nl, "model_choice": [info.threshold, info.coarse_ctas],
+    return {"levels": nl, "default_choice": [info.threshold, info.coarse_ctas],
             "measured_best": [best["threshold"], best["coarse_ctas"]], "rows": rows,
             "note": "[threshold, blocks of the coarse kernel]; per cycle including the convergence norm "
                     "and one host read of the stop flag"}

@@ -558,7 +558,6 @@ struct Hierarchy {
   Scalars* sc_host = nullptr;        // pinned mirror
   LevelV<double>* dlev64 = nullptr;  // device copies of the level views (for
   LevelV<float>* dlev32 = nullptr;   // the persistent coarse kernel)
-  double predicted_us[16] = {};      // cost model: V-cycle time per threshold
   // The solve loop as one CUDA graph: [first residual + stop test] then
   // WHILE(go) { V-cycle; (refinement update;) residual + stop test }.
   cudaGraph_t graph = nullptr;

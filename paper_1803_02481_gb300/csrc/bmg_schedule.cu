@@ -112,16 +112,18 @@ constexpr double kSmemPoints = 300.0;
 // The same for line smoothing, whose sub-cycle works from L2.  Measured us
 // per alternating V(2,1) cycle with the largest level at 7^2, 15^2 and 31^2:
 // 255^2 FP64 564, 557, 613, FP32 365, 369, 418; 2047^2 FP64 2273, 2280, 2355,
-// FP32 1402, 1414, 1480.
+// FP32 1402, 1414, 1480.  Between 7^2 and 15^2 the difference is within 1 %
+// either way (7^2 ahead in three of four); from 31^2 on it is not.
 constexpr double kLinePoints = 100.0;
 
-void choose_schedule(Hierarchy* h) {
-  const bool point = h->opt.smoother == BMG_SMOOTH_POINT;
+// The threshold (and, unless fixed, one block or the largest cluster) with the
+// least predicted time, for the coarse kernels that work from L2.
+static void search_schedule(Hierarchy* h) {
   int cands[2] = {1, 1};
   int nc = 1;
   if (h->opt.coarse_ctas > 0) {
     cands[0] = h->opt.coarse_ctas;
-  } else if (point) {
+  } else {
     const int cmax = max_cluster_ctas(h->opt.precision == BMG_FP32_REFINE);
     if (cmax > 1) cands[nc++] = cmax;
   }
@@ -138,31 +140,30 @@ void choose_schedule(Hierarchy* h) {
       }
     }
   }
-  // The one-block sub-cycle in shared memory runs whatever fits it: any
-  // explicit threshold, and by default every level of at most kSmemPoints
-  // points.
-  if (point && h->opt.coarse_ctas <= 1) {
-    int thr = h->opt.coarse_threshold;
-    if (thr < 1) {
-      thr = 1;
-      while (thr < h->L && double(h->geo64[thr].nx) * h->geo64[thr].ny <= kSmemPoints &&
-             coarse_smem_fits(h, thr + 1))
-        ++thr;
-    }
-    if (coarse_smem_fits(h, thr)) {
-      h->coarse_smem = true;
-      h->threshold = thr;
-      h->coarse_ctas = 1;
-    }
+}
+
+void choose_schedule(Hierarchy* h) {
+  const bool point = h->opt.smoother == BMG_SMOOTH_POINT;
+  // levels 0 .. thr-1 of at most `points` points each
+  const double points = point ? kSmemPoints : kLinePoints;
+  int thr = h->opt.coarse_threshold;
+  if (thr < 1) {
+    thr = 1;
+    while (thr < h->L && double(h->geo64[thr].nx) * h->geo64[thr].ny <= points &&
+           (!point || coarse_smem_fits(h, thr + 1)))
+      ++thr;
   }
-  if (!point && h->opt.coarse_threshold < 1) {
-    h->threshold = 1;
-    while (h->threshold < h->L &&
-           double(h->geo64[h->threshold].nx) * h->geo64[h->threshold].ny <= kLinePoints)
-      ++h->threshold;
+  if (!point) {
+    h->threshold = thr;
+    h->coarse_ctas = 1;
+  } else if (h->opt.coarse_ctas <= 1 && coarse_smem_fits(h, thr)) {
+    // The one-block sub-cycle in shared memory runs whatever fits it.
+    h->coarse_smem = true;
+    h->threshold = thr;
+    h->coarse_ctas = 1;
+  } else {
+    search_schedule(h);
   }
-  for (int thr = 1; thr <= h->L && thr <= 16; ++thr)
-    h->predicted_us[thr - 1] = predict_vcycle_us(h, thr, h->coarse_ctas);
 }
 
 }  // namespace bmg
