@@ -12,8 +12,10 @@
  *     restriction R = P^T and interpolate-and-correct;
  *   - the coarse-grid redistribution of Section 2.2 / Algorithm 2 re-read for
  *     one GPU: every level below a threshold runs inside one persistent
- *     thread block, or one thread-block cluster, instead of one kernel launch
- *     per operation; a cost model in the spirit of Section 3 (Eq. (Vmodel))
+ *     thread block, or one thread-block cluster, instead of kernel launches of
+ *     its own.  By default one block takes the levels of at most 300 points
+ *     (100 with line smoothing), a measured size; where an explicit option
+ *     rules that out, a cost model in the spirit of Section 3 (Eq. (Vmodel))
  *     with measured parameters picks the threshold and the number of blocks.
  *
  * Conventions (all entry points):
@@ -87,8 +89,10 @@ typedef struct {
                                interpolating (Section 3, interpolation
                                equations); 0: x += P x_c (Algorithm 1)       */
   int coarse_threshold;     /* levels l < threshold run inside the persistent
-                               coarse kernel (1 <= threshold <= L); -1: chosen
-                               by the cost model                              */
+                               coarse kernel (1 <= threshold <= L); -1: those
+                               of at most 300 points (100 with line
+                               smoothing); with coarse_ctas > 1 chosen by the
+                               cost model                                     */
   int max_cycles;           /* cap on V-cycles (or refinement steps), 200    */
   int log_coefficients;     /* 1: the coefficient array holds theta = log k and
                                the assembly uses k = exp(theta) (adjoint
@@ -113,8 +117,9 @@ typedef struct {
                                phases separated by the hardware cluster
                                barrier (point smoother only; sizes above 8
                                need the device's non-portable cluster
-                               support); -1 (default) = chosen by the cost
-                               model together with the threshold            */
+                               support); -1 (default) = one block, or, where
+                               an explicit threshold does not fit one block's
+                               shared memory, chosen by the cost model       */
 } bmg_options;
 
 typedef struct {
@@ -288,7 +293,8 @@ int bmg_assemble_backward(bmg_hierarchy *h, const double *u_dev,
 
 /* Measure the cost-model parameters on the current device (the analogue of
  * the Section 3 machine parameters alpha, beta, gamma) and use them for every
- * later threshold choice in this process.  params_out (may be NULL) receives
+ * later choice the model makes in this process (see bmg_options.coarse_threshold
+ * and coarse_ctas) and for bmg_predict_cycle_us.  params_out (may be NULL) receives
  * 10 doubles: launch latency [us], in-block barrier phase [us], streaming
  * bandwidth [GB/s], FP64 and FP32 FMA rates of the whole GPU [GFLOP/s],
  * one-block L2 bandwidth [GB/s], one-block FP64 and FP32 rates [GFLOP/s],
@@ -307,7 +313,10 @@ int bmg_max_coarse_ctas(int precision, int *out);
 
 /* Model-predicted time [us] of one V-cycle of h with the given threshold
  * (levels l < threshold inside the persistent kernel, run by as many blocks
- * as h uses, see bmg_info.coarse_ctas). */
+ * as h uses, see bmg_info.coarse_ctas).  The model is of a coarse kernel that
+ * works from L2 and of one launch per operation on the other levels; cycles
+ * with the shared-memory coarse kernel and fused legs are faster than it
+ * says. */
 int bmg_predict_cycle_us(const bmg_hierarchy *h, int threshold, double *us);
 
 /* ---- Batched solves (many independent problems) -------------------------- */
@@ -323,22 +332,24 @@ typedef struct bmg_batch bmg_batch; /* opaque, library-owned */
  * (r / ||r|| cast down, ||r|| e cast back), all problems' iterations
  * advanced together; opt->interp_residual_term is ignored by the V-cycles (no
  * r/C term on any level); levels of side <= 31 run in the persistent coarse
- * kernel, one thread block per problem.  Setup also picks the tile shape of the batched sweeps for
- * every level side by timing the candidates on this batch (cached per
- * process, and in the file named by the environment variable BMG_TUNE_CACHE
- * if set) and records the refinement loop as one CUDA graph.  Errors as
- * bmg_setup, naming the failing problem in bmg_last_error. */
+ * kernel, one thread block per problem.  With nu1 of 1 or 2 and nu2 of 1 each
+ * leg of the cycle is one launch per level side; otherwise one per operation,
+ * and setup picks the tile shape of the batched sweeps for every level side
+ * by timing the candidates on this batch (cached per process, and in the file
+ * named by the environment variable BMG_TUNE_CACHE if set).  Setup records
+ * the refinement loop as one CUDA graph.  Errors as bmg_setup, naming the
+ * failing problem in bmg_last_error. */
 int bmg_batch_setup(int nprob, const double *const *k_dev, const int *n,
                     const bmg_options *opt, bmg_stream_t stream, bmg_batch **out);
 
 /* Solve every problem to ||b - A x||_2 / ||b||_2 <= tol with ONE launch of
- * the refinement-loop graph: every V-cycle operation is one launch over all
- * problems that have a level of that side, problems that have converged
- * drop out, and the loop ends when none is left.  b_dev[p], x_dev[p]: host
+ * the refinement-loop graph: every leg (or operation) of the V-cycle is one
+ * launch over all problems that have a level of that side, problems that have
+ * converged drop out, and the loop ends when none is left.  b_dev[p], x_dev[p]: host
  * arrays of device pointers to dense n[p] x n[p] float64 arrays (x: initial
  * guess in, solution out).  per_prob (may be NULL) receives nprob bmg_info
  * (cycles = refinement steps of that problem).  Returns BMG_OK, or
- * BMG_ENOCONV / BMG_ENAN if any problem ended that way. */
+ * BMG_ENOCONV / BMG_ENAN / BMG_ETIMEOUT if any problem ended that way. */
 int bmg_batch_solve(bmg_batch *b, const double *const *b_dev, double *const *x_dev,
                     double tol, bmg_info *per_prob, bmg_stream_t stream);
 
@@ -493,7 +504,11 @@ enum { BMG_PROF_FINE_SMOOTH = 1, BMG_PROF_FINE_RESID = 2, BMG_PROF_FINE_INTERP =
  * fine-sweep class then leaves out), one whole V-cycle, and the
  * conjugate-gradient vector
  * kernels of BMG_SOLVER_PCG (A p with p.q, the x/r update with r.r, r.z with
- * the scalars, and p = z + beta p; one bracket per iteration). */
+ * the scalars, and p = z + beta p; one bracket per iteration).
+ * A solve or cycle that begins while a class is recorded launches every
+ * operation by itself, without the solve graph; otherwise levels of a few
+ * hundred tiles run each leg of the V-cycle as one kernel.  The values are the
+ * same; the brackets of such levels are not what an untimed solve spends. */
 int bmg_profile_set(int mask);
 
 /* Synchronise the recorded events of class `which` and return the number of

@@ -67,12 +67,17 @@ int bmg3_setup(const double *k_dev, int nx, int ny, int nz, const bmg_options *o
  * C (x_new - x_old) at the other colour is the residual), which writes out of
  * place, so the iterate returned is the one the residual belongs to: the same
  * bits as with a separate residual pass (one extra half sweep per solve).
+ * FP64 cycles with nu1 >= 1 restrict the finest residual from the points of
+ * the first colour alone: those of the other were updated last, and theirs is
+ * the rounding of that update.
  * info (may be NULL): cycles (refinement steps, or CG iterations) run, final
  * relative residual, solve wall time.  BMG_ENOCONV after max_cycles, BMG_ENAN if the residual is
  * not finite. */
 int bmg3_solve(bmg3_hierarchy *h, const double *b_dev, double *x_dev, double tol, bmg_info *info,
                bmg_stream_t stream);
 
+/* Release the hierarchy (NULL is allowed); its device memory is kept for the
+ * next one as bmg_destroy describes. */
 void bmg3_destroy(bmg3_hierarchy *h);
 
 /* Introspection for parity checks (synchronous, host output). */

@@ -100,9 +100,12 @@ bool shape_ready() {
 
 // Which levels take the fused legs, and with which tile.  Every leg is a
 // chain of phases whose length does not depend on the tile, so as long as
-// the tiles do not fill the GPU the smallest are the best (fewest warps per
-// FP64 phase); past that the halo's redundant work decides.  Measured (us
-// per V-cycle, FP64 unless said otherwise):
+// the tiles do not fill the GPU (304: two for each of its 152 SMs) the
+// smallest are the best (fewest warps per FP64 phase); past that the halo's
+// redundant work decides.  The limits count tiles, and were measured on
+// square grids of 2^m - 1 points a side only: each lies somewhere between
+// the tile counts of two such levels.  Measured (us per V-cycle, FP64 unless
+// said otherwise):
 //  * 8 x 8 up to 304 tiles (two per SM): 127^2 52.9 against 53.9 with 16 x 8,
 //    255^2 66.5 against 67.2; up to 1100 tiles 255^2 takes 68.0;
 //  * 16 x 8 up to 320 tiles: 511^2 99.0; up to 608, 102.8 (its 255^2 level
