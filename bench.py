@@ -10,6 +10,9 @@ coarse operators, coarsest Cholesky) and the solve from x = 0 to
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
+prints one line of JSON; the whole record, with every measurement leg, goes to
+the file named by --details or to standard error.
+
 With N > 1 (torchrun) every rank solves its own copy (independent problems,
 weak scaling, no collective on the data path).  ``--impl reference`` times
 the CPU oracle on a bounded window of the same workload.
@@ -525,7 +528,43 @@ def run_ours(args, rank, world, local_rank):
         line["cpu_baseline"] = cpu_baseline()
         same_windows_ratio(line)
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        write_record(line, args.details)
+
+
+# The printed line: the headline and what explains it.  The whole record, with
+# every measurement leg, is several times as long, and a reader that keeps only
+# the end of a program's output lost the headline in front of it.
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "cycles", "rel_resid", "rel_resid_separate_pass",
+             "rel_resid_extended_precision", "threshold", "coarse_ctas", "unknown_cycles_per_s", "setup_ms",
+             "gpu_launches", "roofline", "e2e", "clocks", "cpu_baseline")
+
+
+def headline(leg):
+    """The first throughput of a leg, or None."""
+    for v in [leg, *leg.values()]:
+        if isinstance(v, dict) and isinstance(v.get("value"), (int, float)):
+            return v["value"]
+    return None
+
+
+def contract_line(record):
+    """The printed part of the record; of the legs their first throughputs."""
+    line = {k: record[k] for k in LINE_KEYS if k in record}
+    legs = {k: headline(v) for k, v in record.items() if k not in LINE_KEYS and isinstance(v, dict)}
+    line["legs_unknowns_per_s"] = {k: v for k, v in legs.items() if v is not None}
+    return line
+
+
+def write_record(record, details):
+    """One line on standard output; the whole record to the file `details`, or
+    to standard error."""
+    if details:
+        with open(details, "w") as f:
+            json.dump(record, f)
+    else:
+        print(json.dumps(record), file=sys.stderr, flush=True)
+    print(json.dumps(contract_line(record)), flush=True)
 
 
 def lognormal_leg(bm, torch, dev, stream, args, n=8191):
@@ -1238,13 +1277,15 @@ def main():
                          "poisson: the 255^2 Poisson problem")
     ap.add_argument("--threshold", type=int, default=None)
     ap.add_argument("--coarse-ctas", type=int, default=None,
-                    help="blocks of the persistent coarse kernel (1, or a cluster size); default: the cost model")
+                    help="blocks of the persistent coarse kernel (1, or a cluster size); default: one block")
     ap.add_argument("--max-cycles", type=int, default=4000)
     ap.add_argument("--n", type=int, default=None,
                     help="grid side (default 4095 block field, 8191 log-normal field)")
     ap.add_argument("--profile", action="store_true",
                     help="profiling run: allow stopping at --max-cycles, skip the extra legs")
     ap.add_argument("--quick", action="store_true", help="skip the e2e, fp32 and CPU legs")
+    ap.add_argument("--details", default=None,
+                    help="file for the whole record with every leg (default: standard error)")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU baseline leg")
     ap.add_argument("--only", default=None,
                     choices=["line_smoother", "three_d", "paper_workload", "paper_workload_9088x568",
