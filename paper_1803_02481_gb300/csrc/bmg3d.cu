@@ -1062,7 +1062,6 @@ struct bmg3_hierarchy {
                                   // eight colour launches (0; environment BMG3_GS27_PAIRS)
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  cudaStream_t gstream = nullptr;   // stream the graph was built for
   // FP64 V-cycles with the stop test in the next cycle's first fine sweep
   // (k3_gs_norm; environment BMG3_FUSED_NORM=0 at setup turns it off): the
   // finest iterate alternates between lv[L-1].x and x2, one step graph per

@@ -10,6 +10,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <map>
+#include <mutex>
 
 namespace bmg {
 
@@ -413,8 +415,13 @@ bool pdl_enabled() {
 }
 
 int max_cluster_ctas(bool fp32) {
-  static int cached[2] = {0, 0};
-  int& c = cached[fp32 ? 1 : 0];
+  // (per device: the query also allows the kernel the larger sizes there)
+  static std::mutex mu;
+  static std::map<std::pair<int, bool>, int> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  std::lock_guard<std::mutex> g(mu);
+  int& c = known[{dev, fp32}];
   if (c == 0) c = fp32 ? max_cluster_ctas_t<float>() : max_cluster_ctas_t<double>();
   return c;
 }

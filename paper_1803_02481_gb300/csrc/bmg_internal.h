@@ -150,12 +150,14 @@ template <typename... KArgs>
 inline bool allow_shared(void (*kern)(KArgs...), size_t bytes, bool carveout = false) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  return shared_opt_in().ensure(reinterpret_cast<const void*>(kern), dev, bytes, [&](size_t n) {
+  const bool ok = shared_opt_in().ensure(reinterpret_cast<const void*>(kern), dev, bytes, [&](size_t n) {
     return (n <= 48 * 1024 ||
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(n)) == cudaSuccess) &&
            (!carveout || cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                               int(cudaSharedmemCarveoutMaxShared)) == cudaSuccess);
   });
+  if (!ok) cudaGetLastError();   // (the caller takes another kernel)
+  return ok;
 }
 template <typename... KArgs>
 inline bool use_shared(void (*kern)(KArgs...), size_t bytes) {
@@ -414,9 +416,9 @@ __device__ __forceinline__ T interp_value(T* const* P, int cp, const T* __restri
 // operators whose measure max_i A_ii (A^-1)_ii is below kInverseLimit: it is 1
 // for a diagonal matrix, the diagonally scaled operator's condition to within
 // a factor n^2, and at most 2.2 on the timed workloads (up to 12 on others of
-// their kinds); at the limit the product's excess is about 1e3 n u.  A hierarchy of one level
-// substitutes always: its cycle is this solve alone, and no later one corrects
-// it.
+// their kinds); at the limit the product's excess is about 1e3 n u.  A
+// hierarchy of one level substitutes always: its cycle is this solve alone,
+// and no later one corrects it.
 struct CoarseSolve {
   const double* inv;     // entry (r, c) at c * n + r
   const double* lo;      // Cholesky factor, row-major
@@ -453,7 +455,8 @@ __device__ __forceinline__ void substitute(const CoarseSolve& s, double* v) {
   }
 }
 
-// Unknown r of x = A_0^{-1} b: row r of the stored inverse times b, read through `inv(c)` and `b(c)`.  More than 16
+// Unknown r of x = A_0^{-1} b: row r of the stored inverse times b, read
+// through `inv(c)` and `b(c)`.  More than 16
 // unknowns: four interleaved partial sums, part `k` of them here, added as
 // (s0 + s1) + (s2 + s3).
 constexpr int kInverseSerial = 16;
